@@ -37,9 +37,10 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // Per-chunk workspace layout of a search over qc queries.
 struct Layout {
-  size_t logits, codes, nprobe, L, nL, seg, slen, slab, perm, enc, total;
+  size_t logits, codes, nprobe, L, nL, seg, slen, slab, enc, refine, total;
 };
-Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C) {
+// Without k there is no refinement (its scratch is bounded, whatever qc).
+Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C, int k = 0) {
   Layout l;
   size_t o = 0;
   const size_t Lmax = (size_t)P + (size_t)C;
@@ -51,8 +52,8 @@ Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C) {
   l.seg = o;    o = align256(o + (size_t)qc * Lmax * sizeof(nr_seg));
   l.slen = o;   o = align256(o + (size_t)qc * 4);
   l.slab = o;   o = align256(o + nr_select_slab_total(qc, P, ix->K_max));
-  l.perm = o;   o = align256(o + (size_t)qc * 4);
   l.enc = o;    o = align256(o + nr_encode_scratch_bytes(ix, qc));
+  l.refine = o; o = align256(o + (k > 0 ? nr_refine_scratch_bytes(qc, k, false) : 0));
   l.total = o;
   return l;
 }
@@ -818,12 +819,11 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
   if (qc < 1) qc = 1;
   if (pipe && qc > pc) qc = pc;
   if (qc > nq) qc = nq;
-  Layout l = chunk_layout(ix, qc, P, C);
+  Layout l = chunk_layout(ix, qc, P, C, k);
   const size_t slot_bytes = align256(l.total);
-  // workspace: [per-query stats][one query counter per buffer][chunk buffers]
+  // workspace: [per-query stats][chunk buffers]
   const size_t stats_off = 0;
-  const size_t cnt_off = align256(stats_off + (size_t)nq * NR_QSTATS * 8);
-  const size_t chunk_off = align256(cnt_off + 16 * (size_t)slots);
+  const size_t chunk_off = align256(stats_off + (size_t)nq * NR_QSTATS * 8);
   if ((st = ensure_ws(ix, chunk_off + slot_bytes * (size_t)slots)) != NR_OK) return st;
   if (pipe && (st = ensure_pipe(ix)) != NR_OK) return st;
   char *w = (char *)ix->ws;
@@ -863,7 +863,6 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     const int64_t n = (nq - q0) < qc ? (nq - q0) : qc;
     const int slot = (int)(i % slots);
     char *cw = w + chunk_off + slot_bytes * (size_t)slot;
-    unsigned int *counter = (unsigned int *)(w + cnt_off + 16 * (size_t)slot);
     // buffer `slot` is free again once the refinement that last read it ended
     if (pipe && i >= slots && (e = cudaStreamWaitEvent(sa, ps.ref[slot], 0)) != cudaSuccess) break;
     const void *qp = (const char *)d_q + q0 * RB;
@@ -894,7 +893,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     ev = tstart(3, sb);
     e = nr_launch_refine(ix, qp, n, k, P + C, (nr_seg *)(cw + l.seg), (int32_t *)(cw + l.nL),
                          (uint32_t *)(cw + l.slen), d_ids + q0 * k, d_d + q0 * k, stats + q0 * NR_QSTATS,
-                         counter, (int32_t *)(cw + l.perm), sb);
+                         cw + l.refine, l.total - l.refine, sb);
     tend(ev, sb);
     if (pipe && e == cudaSuccess) e = cudaEventRecord(ps.ref[slot], sb);
   }

@@ -159,7 +159,11 @@ cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
                              void *d_slab, cudaStream_t s);
+// scratch of a refine launch over nq queries: room to refine one query's
+// stream by several blocks at once, or (least) only whole streams a block
+size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least);
+// scratch: at least the least bytes; whole streams a block below the others
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
-                             int64_t *d_ids, float *d_dists, int64_t *d_stats,
-                             unsigned int *d_counter, int32_t *d_perm, cudaStream_t s);
+                             int64_t *d_ids, float *d_dists, int64_t *d_stats, void *d_scratch,
+                             size_t scratch_bytes, cudaStream_t s);

@@ -1,54 +1,134 @@
 // K4 refine (Sec. 3.4, Algorithm 2's T_low rule; uint8 distances kept as
-// integers, Sec. 4.1.1): persistent CTAs pull queries from an atomic counter
-// and run nrq::refine_block on the segments K3 wrote to global memory.
+// integers, Sec. 4.1.1): a plan kernel cuts the queries' candidate streams
+// into spans, and persistent CTAs pull spans from an atomic counter, run
+// nrq::refine_span on the segments K3 wrote to global memory and commit the
+// spans of a query in stream order.
+//
+// Bound by HBM at large batches (10,000 queries of the 3e7-row uint8 index:
+// 8.48 ms for 63.8 GB of candidate rows, DRAM at 7.31 TB/s), by latency at
+// small ones: one block a query left a single query to one SM (one uint8 query
+// of 31,000 candidates 523 us, four fp32 queries of 154 MB each 7.8 ms; cut
+// into spans 60 us and 0.12 ms).
 //
 // Launch shapes measured on GB300 (u8-10m / f32-10m operating points): the
-// scan is limited by how many queries stream concurrently per SM, so tiles are
-// small (128 uint8 rows, 32-64 fp32 rows), two stages deep, and registers are
-// capped for many CTAs per SM.
+// scan is limited by how many rows are in flight per SM, so tiles are small
+// (128 uint8 rows, 32-64 fp32 rows), two stages deep, and registers are capped
+// for many CTAs per SM. Tiles held in registers (eight lanes a 128-byte row,
+// no shared memory) had fewer bytes in flight: 14.8 ms against 9.1 for that
+// batch.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "nr_internal.cuh"
 #include "nrq_refine.cuh"
 
 namespace {
 
-// Longest streams first: one CTA buckets the queries by stream length
-// (1024 buckets scaled to the longest stream) and writes them in decreasing
-// bucket order, so the persistent refinement CTAs finish together instead of
-// waiting on a long query picked up last. Order inside a bucket is arbitrary;
-// it does not affect any result.
+constexpr int kPlanThreads = 1024;
 constexpr int kOrderBins = 1024;
 
-__global__ void __launch_bounds__(1024) order_kernel(const uint32_t *__restrict__ slen, int64_t nq,
-                                                     int32_t *__restrict__ perm) {
+struct PlanArgs {
+  const uint32_t *slen;
+  int64_t nq;
+  int R;
+  int align;            // rounds of a span: a multiple of this (whole tiles)
+  int rounds_most;      // its rounds when there are items enough
+  unsigned int items_want;  // items that keep every CTA busy
+  unsigned int items_cap;   // items there is room for (nq: whole streams only)
+  nrq::RefinePlan *plan;
+  uint32_t *pre;        // [nq + 1] first item of the i-th query (not of whole streams)
+  int32_t *perm;        // processing order of whole streams
+};
+
+// inclusive prefix of v over the block's threads; *all = the sum
+__device__ __forceinline__ uint64_t plan_scan(uint64_t v, uint64_t *wsum, uint64_t *all) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint64_t x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(nrq::kFull, x, o);
+    if (lane >= o) x += y;
+  }
+  __syncthreads();
+  if (lane == 31) wsum[w] = x;
+  __syncthreads();
+  uint64_t t = wsum[lane];  // kPlanThreads / 32 = 32 warps
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(nrq::kFull, t, o);
+    if (lane >= o) t += y;
+  }
+  *all = __shfl_sync(nrq::kFull, t, 31);
+  const uint64_t before = __shfl_sync(nrq::kFull, t, w > 0 ? w - 1 : 0);
+  return x + (w > 0 ? before : 0);
+}
+
+// One CTA: the rounds of a span and the items of every query. Whole streams
+// (items_cap = nq) go longest first: the queries are bucketed by stream length
+// (1024 buckets scaled to the longest) and listed in decreasing bucket order,
+// so the persistent CTAs finish together instead of waiting on a long query
+// picked up last. Order inside a bucket is arbitrary; it does not affect any
+// result. Streams cut into spans keep the batch's order: their items are
+// short. Bound by latency: 5 us for 1 to 1,000 queries (scans by shuffles; the
+// serial 1,024-bucket scan it replaces made that 8).
+__global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
+  __shared__ uint64_t wsum[32];
   __shared__ unsigned int hist[kOrderBins];
   __shared__ unsigned int smax;
   const int tid = threadIdx.x;
+  const int64_t nq = a.nq;
+  const bool whole = a.items_cap <= nq;
+  const int64_t per = (nq + kPlanThreads - 1) / kPlanThreads;
+  const int64_t lo = min(nq, tid * per), hi = min(nq, lo + per);
+  uint64_t rounds = 0;
   if (tid == 0) smax = 1;
-  for (int i = tid; i < kOrderBins; i += blockDim.x) hist[i] = 0;
-  __syncthreads();
-  unsigned int m = 1;
-  for (int64_t q = tid; q < nq; q += blockDim.x) m = max(m, slen[q]);
-  atomicMax(&smax, m);
-  __syncthreads();
-  const uint64_t top = (uint64_t)smax + 1;
-  for (int64_t q = tid; q < nq; q += blockDim.x)
-    atomicAdd(&hist[kOrderBins - 1 - (int)((uint64_t)slen[q] * kOrderBins / top)], 1u);
-  __syncthreads();
-  if (tid == 0) {  // exclusive scan (1024 entries)
-    unsigned int run = 0;
-    for (int i = 0; i < kOrderBins; ++i) {
-      const unsigned int v = hist[i];
-      hist[i] = run;
-      run += v;
-    }
+  hist[tid] = 0;
+  static_assert(kOrderBins == kPlanThreads, "a bucket per thread");
+  if (!whole)
+    for (int64_t i = lo; i < hi; ++i) rounds += (a.slen[i] + (uint64_t)a.R - 1) / a.R;
+  uint64_t all;
+  plan_scan(rounds, wsum, &all);  // starts with a barrier
+  uint64_t S = 0;                 // rounds of a span; 0: whole streams
+  if (!whole) {
+    S = min((uint64_t)a.rounds_most, all / a.items_want);
+    const uint64_t room = a.items_cap - (uint64_t)nq;
+    S = max(S, (all + room - 1) / room);
+    S = max((S + a.align - 1) / a.align, (uint64_t)1) * a.align;
+    if (S * (uint64_t)a.R >= 0xffffffffull) S = 0;
   }
-  __syncthreads();
-  for (int64_t q = tid; q < nq; q += blockDim.x) {
-    const int bin = kOrderBins - 1 - (int)((uint64_t)slen[q] * kOrderBins / top);
-    perm[atomicAdd(&hist[bin], 1u)] = (int32_t)q;
+  const uint32_t span = S ? (uint32_t)(S * (uint64_t)a.R) : 0xffffffffu;
+  if (whole) {
+    unsigned int m = 1;
+    for (int64_t q = tid; q < nq; q += kPlanThreads) m = max(m, a.slen[q]);
+    m = __reduce_max_sync(nrq::kFull, m);
+    if ((tid & 31) == 0) atomicMax(&smax, m);
+    __syncthreads();
+    const uint64_t top = (uint64_t)smax + 1;
+    auto bin = [&](int64_t q) { return kOrderBins - 1 - (int)((uint64_t)a.slen[q] * kOrderBins / top); };
+    for (int64_t q = tid; q < nq; q += kPlanThreads) atomicAdd(&hist[bin(q)], 1u);
+    __syncthreads();
+    const unsigned int mine = hist[tid];
+    const uint64_t incl = plan_scan(mine, wsum, &all);
+    hist[tid] = (unsigned int)incl - mine;
+    __syncthreads();
+    for (int64_t q = tid; q < nq; q += kPlanThreads) a.perm[atomicAdd(&hist[bin(q)], 1u)] = (int32_t)q;
+    all = (uint64_t)nq;
+  } else {
+    uint64_t items = 0;
+    for (int64_t i = lo; i < hi; ++i) items += max(1u, (uint32_t)(((uint64_t)a.slen[i] + span - 1) / span));
+    const uint64_t incl = plan_scan(items, wsum, &all);
+    uint32_t at = (uint32_t)(incl - items);
+    for (int64_t i = lo; i < hi; ++i) {
+      a.pre[i] = at;
+      at += max(1u, (uint32_t)(((uint64_t)a.slen[i] + span - 1) / span));
+    }
+    if (tid == 0) a.pre[nq] = (uint32_t)all;
+  }
+  if (tid == 0) {
+    a.plan->ticket = 0u;
+    a.plan->nitems = (unsigned int)all;
+    a.plan->span_rows = span;
+    a.plan->pool_used = 0ull;
   }
 }
 
@@ -58,101 +138,260 @@ struct RefineArgs {
   int64_t nq;
   int64_t row_bytes;
   int Lmax;
+  // queries of a group: the first spans of a group's queries come before the
+  // rest of them, so that most later spans start with a committed threshold
+  int group;
   const nr_seg *seg;
   const int32_t *nL;
   const uint32_t *slen;
   int64_t *out_ids;
   float *out_d;
   int64_t *stats;
-  unsigned int *counter;
-  const int32_t *perm;  // processing order (null: index order)
+  nrq::RefinePlan *plan;
+  const uint32_t *pre;       // null: whole streams, in the order of perm
+  const int32_t *perm;
+  nrq::RefineQState *state;  // [nq]
+  uint32_t *ready;           // [items] 0: not finished, 1 + groups logged, or kSpanRedo
+  nrq::SpanHeader *hdr;      // [items]
+  uint64_t *heap;            // [nq x k] committed top-k
+  nrq::SpanEntry *pool;
+  uint32_t pool_cap;
 };
 
-template <int DT, int TR, int STAGES, int CPR, int MINB>
+// The item of ticket t: its query i and its span, by a whole warp. Tickets go group by group: the first spans of the group's
+// queries, then the other spans query by query.
+__device__ __forceinline__ void item_of(const RefineArgs &a, uint32_t t, int &i, uint32_t &span) {
+  const int nq = (int)a.nq;
+  const int g0 = nrq::warp_last_le(0, nq, t, [&](int x) { return __ldg(&a.pre[x]); }) / a.group * a.group;
+  const int ng = min(a.group, nq - g0);
+  const uint32_t first = __ldg(&a.pre[g0]), o = t - first;
+  if (o < (uint32_t)ng) {
+    i = g0 + (int)o;
+    span = 0;
+    return;
+  }
+  const uint32_t x = o - (uint32_t)ng;  // among the later spans of the group
+  i = nrq::warp_last_le(g0, g0 + ng, x,
+                        [&](int y) { return __ldg(&a.pre[y]) - first - (uint32_t)(y - g0); });
+  span = 1u + x - (__ldg(&a.pre[i]) - first - (uint32_t)(i - g0));
+}
+
+// sctl words of the kernel (1..3 are refine_span's)
+enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlCur, kCtlHn, kCtlRounds, kCtlLow, kCtlStop, kCtlNext, kCtlRedo };
+
+template <int DT, int TR, int CPR, int KCC, int MINB>
 __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int k = a.rf.k;
-  const nrq::RefineSmem m = nrq::refine_carve<TR, STAGES>(smem, a.row_bytes, k);
-  int *qslot = m.sctl + 4;
-  for (;;) {
-    if (tid == 0) {
-      const unsigned int slot = atomicAdd(a.counter, 1u);
-      *qslot = slot < a.nq ? (a.perm ? a.perm[slot] : (int)slot) : -1;
+  const nrq::RefineSmem m = nrq::refine_carve<TR, KCC>(smem, a.row_bytes, k);
+  volatile int *ctl = m.sctl;
+  const uint32_t nitems = a.plan->nitems, span_rows = a.plan->span_rows;
+  // spans a commit stages at once: what fits the stages (rows of 16 bytes at least)
+  constexpr int kFit = (int)(nrq::refine_stage_bytes<TR, KCC>(CPR > 0 ? CPR * 16 : 16) / (nrq::kStaged * 16));
+  constexpr int kStage = kFit < 32 ? kFit : 32;
+  for (bool first = true;; first = false) {
+    if (tid < 32) {  // the next item whose query has not stopped
+      int q = -1;
+      uint32_t sp = 0, base = 0, spans = 1;
+      for (uint32_t t = blockIdx.x;; first = false) {
+        if (!first) {
+          if (lane == 0) t = gridDim.x + atomicAdd(&a.plan->ticket, 1u);
+          t = __shfl_sync(nrq::kFull, t, 0);
+        }
+        if (t >= nitems) break;
+        if (!a.pre) {
+          q = a.perm[t];
+          break;
+        }
+        int i;
+        item_of(a, t, i, sp);
+        if (sp > 0 && __ldcg(&a.state[i].done)) continue;
+        q = i;
+        base = __ldg(&a.pre[i]);
+        spans = __ldg(&a.pre[i + 1]) - base;
+        break;
+      }
+      if (lane == 0) {
+        ctl[kCtlQuery] = q;
+        ctl[kCtlItem] = (int)base;
+        ctl[kCtlSpan] = (int)sp;
+        ctl[kCtlSpans] = (int)spans;
+      }
     }
     __syncthreads();
-    const int64_t q = *qslot;
+    const int64_t q = ctl[kCtlQuery];
     if (q < 0) break;
+    uint32_t sp = (uint32_t)ctl[kCtlSpan];
     for (int c = tid; c * 16 < a.row_bytes; c += TR)
       reinterpret_cast<uint4 *>(m.sq)[c] = reinterpret_cast<const uint4 *>(a.q + q * a.row_bytes)[c];
-    nrq::refine_block<DT, TR, STAGES, CPR>(a.rf, m, a.slen[q], a.nL[q], a.seg + (size_t)q * a.Lmax,
-                                           a.out_ids + q * k, a.out_d + q * k,
-                                           a.stats ? a.stats + q * NR_QSTATS : nullptr);
+    const uint32_t n = a.slen[q];
+    nrq::RefineQState *st = a.state + q;
+    bool held = sp == 0;  // this block owns the query's top-k
+    nrq::SpanRun r = {0, 0, 0, 0, false};
+    for (;;) {
+      const uint32_t p0 = sp * span_rows;  // span 0 when streams are whole
+      const uint32_t p1 = n - p0 > span_rows ? p0 + span_rows : n;
+      nrq::SpanLog lg;
+      lg.nthr = &st->nthr;
+      lg.pool_used = &a.plan->pool_used;
+      lg.pool = a.pool;
+      lg.pool_cap = a.pool_cap;
+      nrq::refine_span<DT, TR, CPR, KCC>(a.rf, m, p0, p1, a.nL[q], a.seg + (size_t)q * a.Lmax, held, r, lg);
+      const uint32_t base = (uint32_t)ctl[kCtlItem], spans = (uint32_t)ctl[kCtlSpans];
+      uint32_t next = sp + 1;  // the next span to commit, when held
+      bool redo = false;
+      if (!held && tid < 32) {  // publish the log
+        __syncwarp();
+        if (lane == 0) {
+          a.hdr[base + sp].minkey = r.hn > 0 ? m.hkey[r.cur * k] : nrq::kEmpty;
+          a.hdr[base + sp].off = lg.off;
+          __threadfence();
+          atomicExch(&a.ready[base + sp], lg.full ? nrq::kSpanRedo : lg.groups + 1u);
+          __threadfence();
+        }
+      }
+      for (;;) {
+        if (!held) {
+          if (!__syncthreads_or(tid == 0 && atomicCAS(&st->lock, 1, 2) == 1)) break;
+          __threadfence();
+          held = true;
+          r.cur = 0;
+          r.hn = __ldcg(&st->hn);
+          r.rounds = __ldcg(&st->rounds);
+          r.low = __ldcg(&st->low);
+          r.stop = false;
+          next = (uint32_t)__ldcg(&st->next);
+          for (int i = tid; i < r.hn; i += TR) {
+            m.hkey[i] = __ldcg(&a.heap[q * k + i]);
+            m.htag[i] = 0;
+          }
+          __syncthreads();
+        }
+        if (!r.stop && next < spans) {  // commit the finished spans that follow
+          if (tid < 32) {
+            // the stages are free between spans
+            redo = nrq::commit_ready(a.rf, m, r, a.pool, a.pool_cap, a.ready + base, a.hdr + base, next,
+                                     spans, n, span_rows, reinterpret_cast<uint4 *>(m.stage), kStage);
+            if (lane == 0) {
+              ctl[kCtlCur] = r.cur;
+              ctl[kCtlHn] = r.hn;
+              ctl[kCtlRounds] = r.rounds;
+              ctl[kCtlLow] = r.low;
+              ctl[kCtlStop] = r.stop ? 1 : 0;
+              ctl[kCtlNext] = (int)next;
+              ctl[kCtlRedo] = redo ? 1 : 0;
+            }
+          }
+          __syncthreads();
+          r.cur = ctl[kCtlCur];
+          r.hn = ctl[kCtlHn];
+          r.rounds = ctl[kCtlRounds];
+          r.low = ctl[kCtlLow];
+          r.stop = ctl[kCtlStop] != 0;
+          next = (uint32_t)ctl[kCtlNext];
+          redo = ctl[kCtlRedo] != 0;
+        }
+        const uint64_t *H = m.hkey + r.cur * k;
+        if (r.stop || next == spans) {  // the answer, sorted by (distance, id), padded
+          for (int i = tid; i < k; i += TR) {
+            int64_t id = -1;
+            float d = __int_as_float(0x7f800000);
+            if (i < r.hn) {
+              const uint64_t kk = H[i];
+              id = (int64_t)(uint32_t)kk;
+              const uint32_t db = (uint32_t)(kk >> 32);
+              d = DT == 0 ? (float)db : __uint_as_float(db);
+            }
+            a.out_ids[q * k + i] = id;
+            a.out_d[q * k + i] = d;
+          }
+          if (tid == 0) {
+            const uint64_t rows = (uint64_t)r.rounds * (uint64_t)a.rf.R;
+            if (a.stats) {
+              a.stats[q * NR_QSTATS] = (int64_t)(rows < n ? rows : n);  // rows of completed rounds
+              a.stats[q * NR_QSTATS + 1] = r.rounds;
+            }
+            if (spans > 1) atomicExch(&st->done, 1);
+          }
+          redo = false;
+          break;  // the lock stays taken: there is nothing more to commit
+        }
+        if (redo) break;
+        // hand the top-k back
+        for (int i = tid; i < r.hn; i += TR) a.heap[q * k + i] = H[i];
+        if (tid == 0) {
+          st->hn = r.hn;
+          st->rounds = r.rounds;
+          st->low = r.low;
+          st->next = (int)next;
+          if (r.hn == k) *reinterpret_cast<volatile unsigned long long *>(&st->nthr) = ~H[k - 1];
+        }
+        __syncthreads();
+        held = false;
+        bool again = false;
+        if (tid == 0) {
+          __threadfence();
+          atomicExch(&st->lock, 1);
+          __threadfence();
+          // a span finished meanwhile was left by its block to this one
+          again = nrq::ld_acquire(&a.ready[base + next]) != 0u;
+        }
+        if (!__syncthreads_or(again)) break;
+      }
+      if (!redo) break;
+      sp = next;  // its block had no room for the log: refined here on the query's top-k
+    }
+    __syncthreads();  // m and ctl are free for the next item
   }
 }
 
-// fp32 rows longer than 1 KB: tiles staged in pieces (refine_block_split)
-template <int TR, int STAGES, int KCC, int MINB>
-__global__ void __launch_bounds__(TR, MINB) refine_split_kernel(RefineArgs a) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const int tid = threadIdx.x;
-  const int k = a.rf.k;
-  const nrq::RefineSmem m = nrq::refine_split_carve<TR, STAGES, KCC>(smem, a.row_bytes, k);
-  int *qslot = m.sctl + 4;
-  for (;;) {
-    if (tid == 0) {
-      const unsigned int slot = atomicAdd(a.counter, 1u);
-      *qslot = slot < a.nq ? (a.perm ? a.perm[slot] : (int)slot) : -1;
-    }
-    __syncthreads();
-    const int64_t q = *qslot;
-    if (q < 0) break;
-    for (int c = tid; c * 16 < a.row_bytes; c += TR)
-      reinterpret_cast<uint4 *>(m.sq)[c] = reinterpret_cast<const uint4 *>(a.q + q * a.row_bytes)[c];
-    nrq::refine_block_split<TR, STAGES, KCC>(a.rf, m, a.slen[q], a.nL[q],
-                                             a.seg + (size_t)q * a.Lmax, a.out_ids + q * k,
-                                             a.out_d + q * k, a.stats ? a.stats + q * NR_QSTATS : nullptr);
-  }
+// Whether a batch keeps its streams whole (a block a query) when grid blocks
+// are resident. Few queries leave most blocks idle; many keep them busy, and
+// cutting their streams only adds work per span (about 7 us each: the item,
+// the segment search, the first tile's latency, the commit) and rows read
+// beyond an early stop. Measured (search us, cut / whole): u8-10m P 256, no
+// early stop, 912 blocks: 100 queries 237 / 379, 500 427 / 448, 700 521 / 503;
+// u8-30m P 1024 t_low 80: 300 537 / 657, 500 752 / 764, 700 975 / 910; f32-10m
+// t_low 16, 1,824 blocks: 500 620 / 944, 900 974 / 1022, 1400 1476 / 1177;
+// u8-10m P 64 t_low 4: 100 165 / 172, 500 261 / 196; 1536-value fp32 rows, 456
+// blocks: 30 1,109 / 11,860, 200 6,190 / 13,588. An early stop after few
+// rounds makes the later spans of a stream likely waste.
+bool whole_streams(int64_t nq, int64_t grid, int t_low, bool long_rows) {
+  if (long_rows) return nq >= grid;
+  const int64_t sixteenths = t_low == 0 || t_low >= 64 ? 9 : t_low >= 8 ? 6 : 2;
+  return nq * 16 >= grid * sixteenths;
 }
 
-template <typename K>
-cudaError_t persistent_launch(nr_index *ix, K kern, int threads, size_t smem, int64_t nq,
-                              const void *args, cudaStream_t s, void (*go)(K, int, int, size_t,
-                                                                           cudaStream_t, const void *)) {
+template <int DT, int TR, int CPR, int KCC, int MINB>
+cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s) {
+  const size_t smem = nrq::refine_smem_bytes<TR, KCC>(a.row_bytes, a.rf.k);
+  auto kern = refine_kernel<DT, TR, CPR, KCC, MINB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TR, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
   int64_t grid = (int64_t)per_sm * ix->num_sms;
-  if (grid > nq) grid = nq;
-  go(kern, (int)grid, threads, smem, s, args);
+  pa.align = a.rf.R < TR ? TR / a.rf.R : 1;
+  // two uint8 items a block, four of the slower fp32 ones (u8-10m, 100 queries:
+  // 237 us at two, 244 at four; long fp32 rows, 30 queries: 1,203 and 1,109)
+  pa.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
+  if (whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) pa.items_cap = (unsigned int)a.nq;
+  a.group = (int)grid;
+  if (pa.items_cap <= a.nq) {  // whole streams
+    a.pre = nullptr;
+    grid = std::min(grid, a.nq);
+  }
+  plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
+  ix->launches += 1;
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)grid, TR, smem, s>>>(a);
   ix->launches += 1;
   return cudaGetLastError();
-}
-
-template <int DT, int TR, int STAGES, int CPR, int MINB = 1>
-cudaError_t launch_refine(nr_index *ix, const RefineArgs &a, cudaStream_t s) {
-  const size_t smem = nrq::refine_smem_bytes<DT, TR, STAGES>(a.row_bytes, a.rf.k) + 16;
-  auto kern = refine_kernel<DT, TR, STAGES, CPR, MINB>;
-  return persistent_launch(ix, kern, TR, smem, a.nq, &a, s,
-                           +[](decltype(kern) kk, int g, int t, size_t sm, cudaStream_t st,
-                               const void *p) {
-                             kk<<<g, t, sm, st>>>(*static_cast<const RefineArgs *>(p));
-                           });
-}
-
-template <int TR, int STAGES, int KCC, int MINB>
-cudaError_t launch_refine_split(nr_index *ix, const RefineArgs &a, cudaStream_t s) {
-  const size_t smem = nrq::refine_split_smem_bytes<TR, STAGES, KCC>(a.row_bytes, a.rf.k) + 16;
-  auto kern = refine_split_kernel<TR, STAGES, KCC, MINB>;
-  return persistent_launch(ix, kern, TR, smem, a.nq, &a, s,
-                           +[](decltype(kern) kk, int g, int t, size_t sm, cudaStream_t st,
-                               const void *p) {
-                             kk<<<g, t, sm, st>>>(*static_cast<const RefineArgs *>(p));
-                           });
 }
 
 nrq::RefineParams refine_params(const nr_index *ix, int k) {
@@ -177,19 +416,56 @@ nrq::RefineParams refine_params(const nr_index *ix, int k) {
   return rf;
 }
 
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+// Scratch of a refine launch: [plan][order of whole streams], and where
+// streams may be cut into items spans: [item prefix][query states, ready flags
+// (zeroed together)][span headers][committed top-k][log entries]
+struct RefineScratch {
+  size_t plan, perm, pre, state, ready, zero_end, hdr, heap, pool, total;
+};
+RefineScratch refine_scratch(int64_t nq, int k, int64_t items, int64_t entries) {
+  RefineScratch l = {};
+  size_t o = 0;
+  l.plan = o; o = up256(o + sizeof(nrq::RefinePlan));
+  l.perm = o; o = up256(o + (size_t)nq * 4);
+  if (items > nq) {
+    l.pre = o;   o = up256(o + ((size_t)nq + 1) * 4);
+    l.state = o; o += (size_t)nq * sizeof(nrq::RefineQState);
+    l.ready = o; o += (size_t)items * 4;
+    l.zero_end = o;
+    o = up256(o);
+    l.hdr = o;   o = up256(o + (size_t)items * sizeof(nrq::SpanHeader));
+    l.heap = o;  o = up256(o + (size_t)nq * k * 8);
+    l.pool = o;  o = up256(o + (size_t)entries * sizeof(nrq::SpanEntry));
+  }
+  l.total = o;
+  return l;
+}
+
+// Items and log entries a batch of nq queries has room for.
+int64_t span_items(int64_t nq) { return nq + std::min<int64_t>(1 << 20, std::max<int64_t>(4096, nq * 64)); }
+int64_t span_entries(int64_t nq, int k) {
+  return std::min<int64_t>(16 << 20, (int64_t)k * std::max<int64_t>(4096, nq * 32));
+}
+
 }  // namespace
+
+size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least) {
+  return least ? refine_scratch(nq, k, nq, 0).total
+               : refine_scratch(nq, k, span_items(nq), span_entries(nq, k)).total;
+}
 
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
-                             int64_t *d_ids, float *d_dists, int64_t *d_stats,
-                             unsigned int *d_counter, int32_t *d_perm, cudaStream_t s) {
+                             int64_t *d_ids, float *d_dists, int64_t *d_stats, void *d_scratch,
+                             size_t scratch_bytes, cudaStream_t s) {
   if (nq <= 0) return cudaSuccess;
-  if (d_perm) {
-    order_kernel<<<1, 1024, 0, s>>>(d_slen, nq, d_perm);
-    ix->launches += 1;
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  char *w = static_cast<char *>(d_scratch);
+  const int64_t items = span_items(nq), entries = span_entries(nq, k);
+  RefineScratch l = refine_scratch(nq, k, items, entries);
+  const bool whole = l.total > scratch_bytes;  // no room to cut streams
+  if (whole) l = refine_scratch(nq, k, nq, 0);
   RefineArgs a;
   a.rf = refine_params(ix, k);
   a.q = static_cast<const uint8_t *>(d_q);
@@ -202,21 +478,41 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   a.out_ids = d_ids;
   a.out_d = d_dists;
   a.stats = d_stats;
-  a.counter = d_counter;
-  a.perm = d_perm;
-  cudaError_t e = cudaMemsetAsync(d_counter, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return e;
+  a.plan = reinterpret_cast<nrq::RefinePlan *>(w + l.plan);
+  a.pre = reinterpret_cast<uint32_t *>(w + l.pre);
+  a.perm = reinterpret_cast<int32_t *>(w + l.perm);
+  a.state = reinterpret_cast<nrq::RefineQState *>(w + l.state);
+  a.ready = reinterpret_cast<uint32_t *>(w + l.ready);
+  a.hdr = reinterpret_cast<nrq::SpanHeader *>(w + l.hdr);
+  a.heap = reinterpret_cast<uint64_t *>(w + l.heap);
+  a.pool = reinterpret_cast<nrq::SpanEntry *>(w + l.pool);
+  a.pool_cap = whole ? 0u : (uint32_t)entries;
+  PlanArgs pa;
+  pa.slen = d_slen;
+  pa.nq = nq;
+  pa.R = a.rf.R;
+  pa.align = 1;
+  pa.rounds_most = std::max(1, 8192 / a.rf.R);
+  pa.items_want = 1;
+  pa.items_cap = (unsigned int)(whole ? nq : items);
+  pa.plan = a.plan;
+  pa.pre = reinterpret_cast<uint32_t *>(w + l.pre);
+  pa.perm = reinterpret_cast<int32_t *>(w + l.perm);
+  if (!whole) {
+    const cudaError_t e = cudaMemsetAsync(w + l.state, 0, l.zero_end - l.state, s);
+    if (e != cudaSuccess) return e;
+  }
   if (ix->dtype == 0) {
-    if (a.rf.cpr == 8) return launch_refine<0, 128, 2, 8, 6>(ix, a, s);  // uint8, D = 128
-    if (ix->row_bytes <= 512) return launch_refine<0, 128, 2, 0, 4>(ix, a, s);
-    return launch_refine<0, 64, 2, 0, 4>(ix, a, s);
+    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 6>(ix, a, pa, s);  // uint8, D = 128
+    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 4>(ix, a, pa, s);
+    return launch_refine<0, 64, 0, 0, 4>(ix, a, pa, s);
   }
   if (ix->row_bytes > 1024) {  // fp32, D above 256: rows staged in pieces
-    if (ix->row_bytes % 256 == 0) return launch_refine_split<128, 2, 16, 3>(ix, a, s);
-    if (ix->row_bytes % 128 == 0) return launch_refine_split<128, 2, 8, 3>(ix, a, s);
-    return launch_refine_split<128, 2, 4, 3>(ix, a, s);  // row_bytes % 64 == 0 (load check)
+    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 3>(ix, a, pa, s);
+    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 3>(ix, a, pa, s);
+    return launch_refine<1, 128, 0, 4, 3>(ix, a, pa, s);  // row_bytes % 64 == 0 (load check)
   }
-  if (a.rf.cpr == 24) return launch_refine<1, 32, 2, 24, 12>(ix, a, s);  // fp32, D = 96
-  if (ix->row_bytes <= 512) return launch_refine<1, 64, 2, 0, 4>(ix, a, s);
-  return launch_refine<1, 32, 2, 0, 4>(ix, a, s);
+  if (a.rf.cpr == 24) return launch_refine<1, 32, 24, 0, 12>(ix, a, pa, s);  // fp32, D = 96
+  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 4>(ix, a, pa, s);
+  return launch_refine<1, 32, 0, 0, 4>(ix, a, pa, s);
 }

@@ -67,9 +67,9 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   if (nq == 0) return NR_OK;
   if (!d_queries || !d_out_ids || !d_out_dists) return NR_ERR_INVALID_ARG;
   // scratch layout: logits, codes, probe counts, cluster lists and their
-  // counts, segments, stream lengths, the refinement order, per-query stats,
-  // select's global sort slabs, the query counter, the activations of an
-  // encoder with several hidden layers. nq < 2^31 and every
+  // counts, segments, stream lengths, per-query stats, select's global sort
+  // slabs, the activations of an encoder with several hidden layers, the
+  // refinement's plan and order. nq < 2^31 and every
   // per-query size is bounded (P, C <= 4096, b <= 24, the slab <= 768 KiB),
   // so no product below overflows size_t.
   const size_t Lmax = (size_t)P + (size_t)C, q = (size_t)nq;
@@ -81,12 +81,12 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   const size_t o_nL = o;     o = up256(o + q * 4);
   const size_t o_seg = o;    o = up256(o + q * Lmax * sizeof(nr_seg));
   const size_t o_slen = o;   o = up256(o + q * 4);
-  const size_t o_perm = o;   o = up256(o + q * 4);
   const size_t o_stats = o;  o = up256(o + q * NR_QSTATS * 8);
   const size_t slab_q = nr_select_slab_bytes(P, ix->K_max);
   const size_t o_slab = o;   o = up256(o + nr_select_slab_total((int64_t)q, P, ix->K_max));
-  const size_t o_count = o;  o = up256(o + 16);
   const size_t o_enc = o;    o = up256(o + nr_encode_scratch_bytes(ix, (int64_t)q));
+  // the rest serves the refinement, which takes what it can use of it
+  const size_t o_refine = o; o += nr_refine_scratch_bytes(nq, k, true);
   if (o > NR_STATIC_SCRATCH_BYTES) return NR_ERR_INVALID_ARG;  // request too large for the array
   DeviceGuard g(ix->device);
   if (!g.ok) return NR_ERR_CUDA;
@@ -98,7 +98,7 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   float *logits = (float *)(w + o_logits);
   int64_t *stats = (int64_t *)(w + o_stats);
   // every buffer below is fully written before it is read, except the
-  // refine kernel's query counter, which its launcher clears on the stream
+  // refinement's flags, which its launcher clears on the stream
   cudaError_t e = nr_launch_encode(ix, d_queries, nq, logits, s, w + o_enc);
   if (e == cudaSuccess)
     e = nr_launch_route(ix, logits, nq, P, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), s);
@@ -109,7 +109,7 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   if (e == cudaSuccess)
     e = nr_launch_refine(ix, d_queries, nq, k, (int)Lmax, (nr_seg *)(w + o_seg),
                          (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), d_out_ids, d_out_dists,
-                         stats, (unsigned int *)(w + o_count), (int32_t *)(w + o_perm), s);
+                         stats, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine, s);
   // statistics of this call are read from the array by nr_last_stats / nr_query_stats
   ix->d_stats = stats;
   ix->last_nq = nq;

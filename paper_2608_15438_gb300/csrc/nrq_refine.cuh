@@ -1,5 +1,7 @@
-// refine_block: one block per query refines the candidate stream exactly
-// with round-based early stop (Sec. 3.4, Algorithm 2's T_low rule).
+// refine_span: one block refines a span of a query's candidate stream exactly,
+// with the round-based early stop (Sec. 3.4, Algorithm 2's T_low rule), and
+// the in-order commit that joins the spans of a query refined by several
+// blocks.
 #pragma once
 
 #include "nrq_common.cuh"
@@ -16,14 +18,21 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
 
 // ============================================================== refine
 // Candidate stream = rows of the kept clusters in list order, a list of
 // contiguous segments. Tiles of TR rows (one row per thread) are gathered by
 // 16-byte cp.async copies (each warp copies and later reads only its own 32
-// rows, so stage reuse needs no block barrier) into STAGES shared-memory
-// stages whose 16-byte chunks are XOR-swizzled by row, so one-row-per-thread
-// reads are bank-conflict free.
+// rows, so stage reuse needs no block barrier) into two shared-memory stages
+// whose 16-byte chunks are XOR-swizzled by row, so one-row-per-thread reads
+// are bank-conflict free. fp32 rows too long for whole-row stages (KCC > 0,
+// D above 256) are staged in pieces of KCC 16-byte chunks of every row, each
+// thread carrying its row's distance from piece to piece.
 // Distances: uint8 rows: per-byte |x - q| (__vabsdiffu4) squared and summed by
 // __dp4a in int32 (exact); fp32 rows: the sequential fmaf chain over j, so a
 // distance is bit-identical to a sequential CPU evaluation.
@@ -31,6 +40,21 @@ __device__ __forceinline__ void cp_async_wait() {
 // current k-th key are merged by rank, each member tagged with the round it
 // entered. After round t: updates = members entered in round t, front
 // updates = those within the first nfront slots.
+//
+// A query's stream is cut into spans of S whole rounds, refined by different
+// blocks at once (the plan kernel chooses S). The block of span 0 refines it
+// on the query's own top-k. A block of a later span does not know the top-k
+// that its rounds start from: it refines its span on an empty top-k of its
+// own and logs, per round, the members that entered (a row outside that local
+// top-k has k smaller rows before it in its own span, and a row at or above
+// the k-th key of the spans committed so far has k smaller ones there, so
+// neither can enter the query's). The spans are then committed in stream
+// order: each round's logged members are merged into the query's top-k and
+// the stop rule is evaluated round by round, which gives the top-k, the
+// rounds and the stop of one block refining the whole stream. Whichever block
+// finishes the next span to commit takes the query's lock and commits every
+// consecutive finished span; a block that does not get the lock moves on (the
+// holder looks again after it unlocks), so no block ever waits for another.
 struct RefineParams {
   const uint8_t *vec;
   const uint32_t *ids;
@@ -40,255 +64,71 @@ struct RefineParams {
   int t_low, u_min, f_min, r_min, nfront;
 };
 
-// Shared memory of refine_block beyond the stages.
+// What the plan kernel leaves for the refinement: work counters and the spans.
+struct RefinePlan {
+  unsigned int ticket;            // items handed out beyond each block's first
+  unsigned int nitems;            // spans of all queries
+  uint32_t span_rows;             // rows of a span (S R; 0xffffffff: whole streams)
+  unsigned int pad;
+  unsigned long long pool_used;   // log entries reserved
+};
+
+// A query's committed state, zeroed before the launch. lock: 0 = span 0 not
+// committed yet (its block owns the state), 1 = free, 2 = held.
+struct RefineQState {
+  int lock, next, done, hn, rounds, low;
+  unsigned long long nthr;  // ~(k-th key) of a full top-k, 0 before
+};
+struct SpanHeader {  // of a logged span
+  uint64_t minkey;   // its smallest key
+  uint32_t off, pad; // its first group of log entries
+};
+// The log: per round in which members entered a span's local top-k, a group of
+// 1 + count entries: first (next group of the span, round within the span,
+// count), then (key, 0, 0) per member.
+struct SpanEntry {
+  uint64_t key;  // of a group's first entry: the next group, kEmpty for none
+  uint32_t round, count;
+};
+constexpr uint32_t kSpanRedo = 0xffffffffu;  // ready value: not logged (the pool was full)
+
+// Rows that the stages hold as they are (see refine_span).
+template <int DT, int CPR>
+constexpr bool kRow128 = DT == 0 && CPR == 8;
+
+// Log entries of a span that the commit stages in shared memory: its first
+// group's first 32.
+constexpr int kStaged = 32;
+// Bytes of the stages: two tiles.
+template <int TR, int KCC>
+__host__ __device__ constexpr size_t refine_stage_bytes(int64_t row_bytes) {
+  return (size_t)2 * TR * (KCC > 0 ? KCC * 16 : row_bytes);
+}
+
+// Shared memory of refine_span.
 struct RefineSmem {
-  unsigned char *stage;  // STAGES x TR x row_bytes (16-byte aligned)
+  unsigned char *stage;  // refine_stage_bytes (16-byte aligned)
   unsigned char *sq;     // the query row (row_bytes)
-  uint32_t *srow;        // STAGES x TR
+  uint32_t *srow;        // 2 x TR: rows of the open tiles
   uint64_t *hkey;        // 2 x k
   uint64_t *skey;        // 2 x TR
   int *htag;             // 2 x k
-  int *sctl;             // 4 ints: survivor counters [1..3]
+  int *sctl;             // 16 ints: [1..3] survivor counters, [4..15] the kernel's
 };
 
-template <int DT, int TR, int STAGES>
+template <int TR, int KCC>
 __host__ __device__ inline size_t refine_smem_bytes(int64_t row_bytes, int k) {
-  return (size_t)STAGES * TR * row_bytes + (size_t)row_bytes + (size_t)STAGES * TR * 4 +
-         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)2 * k * 4 + 16;
+  return refine_stage_bytes<TR, KCC>(row_bytes) + (size_t)row_bytes + (size_t)2 * TR * 4 +
+         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)2 * k * 4 + 16 * 4;
 }
 
 // Carve RefineSmem from base (16-byte aligned).
-template <int TR, int STAGES>
+template <int TR, int KCC>
 __device__ __forceinline__ RefineSmem refine_carve(unsigned char *base, int64_t row_bytes, int k) {
   RefineSmem m;
   m.stage = base;
-  m.sq = base + (size_t)STAGES * TR * row_bytes;
+  m.sq = base + refine_stage_bytes<TR, KCC>(row_bytes);
   m.srow = reinterpret_cast<uint32_t *>(m.sq + row_bytes);
-  m.hkey = reinterpret_cast<uint64_t *>(m.srow + STAGES * TR);
-  m.skey = m.hkey + 2 * k;
-  m.htag = reinterpret_cast<int *>(m.skey + 2 * TR);
-  m.sctl = m.htag + 2 * k;
-  return m;
-}
-
-// One query. The caller has written the query row into m.sq (block-visible
-// after this function's first barrier).
-// segs: nl segments (any address space) of a stream of n positions. Writes
-// out_ids/out_d [k] and stats[0..1]. Whole block (TR threads) calls.
-template <int DT, int TR, int STAGES, int CPR>
-__device__ __forceinline__ void refine_block(const RefineParams &a, const RefineSmem &m, uint32_t n,
-                                             int nl, const nr_seg *segs, int64_t *out_ids,
-                                             float *out_d, int64_t *stats) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cpr = CPR > 0 ? CPR : a.cpr;
-  const int swz = CPR > 0 ? ((CPR % 8 == 0) ? 7 : (CPR % 4 == 0) ? 3 : (CPR % 2 == 0) ? 1 : 0)
-                          : a.swz_mask;
-  const int64_t RB = (int64_t)cpr * 16;
-  const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(m.stage);
-  const int k = a.k;
-  const int chunk = a.R < TR ? a.R : TR;
-  const uint32_t ntiles = (uint32_t)(((uint64_t)n + TR - 1) / TR);
-  if (tid == 0) m.sctl[1] = m.sctl[2] = m.sctl[3] = 0;
-  __syncthreads();  // the caller's copy of the query row into m.sq is visible after this
-  uint4 qreg[DT == 0 && CPR > 0 && CPR <= 8 ? CPR : 1];
-  if (DT == 0 && CPR > 0 && CPR <= 8) {
-#pragma unroll
-    for (int c = 0; c < (CPR > 0 && CPR <= 8 ? CPR : 1); ++c) qreg[c] = reinterpret_cast<const uint4 *>(m.sq)[c];
-  }
-
-  int seg_i = 0;  // this thread's segment cursor (positions only grow)
-  auto issue = [&](uint32_t t, int st) {
-    if (t < ntiles) {
-      const uint32_t p = t * TR + tid;
-      uint32_t grow = 0;
-      if (p < n) {
-        // last segment starting at or before p: exponential search from the cursor
-        int step = 1;
-        while (seg_i + step < nl && segs[seg_i + step].pos <= p) {
-          seg_i += step;
-          step <<= 1;
-        }
-        for (step >>= 1; step > 0; step >>= 1)
-          if (seg_i + step < nl && segs[seg_i + step].pos <= p) seg_i += step;
-        grow = segs[seg_i].row0 + (p - segs[seg_i].pos);
-        m.srow[st * TR + tid] = grow;
-      }
-      const uint32_t wbase = t * TR + warp * 32;
-      const uint32_t sbase = stage_s + (uint32_t)((size_t)st * TR * RB);
-#pragma unroll 4
-      for (int f = lane; f < 32 * cpr; f += 32) {
-        const int rr = f / cpr;
-        const int c = f - rr * cpr;
-        const uint32_t gr = __shfl_sync(kFull, grow, rr);
-        if (wbase + rr < n) {
-          const int r = warp * 32 + rr;
-          const uint32_t dst = sbase + (uint32_t)(r * RB) + (uint32_t)((c ^ (r & swz)) << 4);
-          cp_async16(dst, a.vec + (size_t)gr * RB + ((size_t)c << 4));
-        }
-      }
-    }
-    cp_async_commit();
-  };
-
-  for (int s = 0; s < STAGES - 1; ++s) issue((uint32_t)s, s);
-  int cur = 0, hn = 0, rounds = 0, low = 0, ci = 0;
-  bool stop = false;
-  uint32_t done = 0;                                 // positions in completed rounds
-  const uint32_t rmask_round = (uint32_t)a.R - 1u;  // R is a power of two
-  int st = 0;                                        // stage of tile t
-  for (uint32_t t = 0; t < ntiles && !stop; ++t) {
-    issue(t + STAGES - 1, st == 0 ? STAGES - 1 : st - 1);
-    cp_async_wait<STAGES - 1>();
-    __syncwarp();
-    const uint32_t p = t * TR + tid;
-    uint32_t dkey = 0xffffffffu;
-    if (p < n) {
-      const unsigned char *row = m.stage + (size_t)st * TR * RB + (size_t)tid * RB;
-      if (DT == 0) {
-        unsigned a0 = 0, a1 = 0, a2 = 0, a3 = 0;  // integer sums: any order is exact
-#pragma unroll 8
-        for (int c = 0; c < cpr; ++c) {
-          const uint4 v = *reinterpret_cast<const uint4 *>(row + ((c ^ (tid & swz)) << 4));
-          uint4 w;
-          if (CPR > 0 && CPR <= 8) w = qreg[c < (CPR > 0 && CPR <= 8 ? CPR : 1) ? c : 0];
-          else w = reinterpret_cast<const uint4 *>(m.sq)[c];
-          unsigned d;
-          d = __vabsdiffu4(v.x, w.x); a0 = __dp4a(d, d, a0);
-          d = __vabsdiffu4(v.y, w.y); a1 = __dp4a(d, d, a1);
-          d = __vabsdiffu4(v.z, w.z); a2 = __dp4a(d, d, a2);
-          d = __vabsdiffu4(v.w, w.w); a3 = __dp4a(d, d, a3);
-        }
-        dkey = (a0 + a1) + (a2 + a3);
-      } else {
-        float acc = 0.0f;  // sequential over j: the order fixes the rounding
-#pragma unroll 4
-        for (int c = 0; c < cpr; ++c) {
-          const float4 v = *reinterpret_cast<const float4 *>(row + ((c ^ (tid & swz)) << 4));
-          const float4 w = reinterpret_cast<const float4 *>(m.sq)[c];
-          float d;
-          d = __fsub_rn(v.x, w.x); acc = __fmaf_rn(d, d, acc);
-          d = __fsub_rn(v.y, w.y); acc = __fmaf_rn(d, d, acc);
-          d = __fsub_rn(v.z, w.z); acc = __fmaf_rn(d, d, acc);
-          d = __fsub_rn(v.w, w.w); acc = __fmaf_rn(d, d, acc);
-        }
-        dkey = __float_as_uint(acc);
-      }
-    }
-    // Merge chunk by chunk; a round ends every R stream positions. One block
-    // barrier per chunk (two when the top-k changes): survivor counters
-    // rotate over three slots and survivor buffers over two, and every warp
-    // evaluates the stop rule itself from the shared top-k.
-    for (int cs = 0; cs < TR && !stop; cs += chunk, ++ci) {
-      const uint32_t cstart = t * TR + cs;
-      if (cstart >= n) break;
-      int *cnt = &m.sctl[1 + ci % 3];
-      uint64_t *sk_buf = m.skey + (ci & 1) * TR;
-      const uint64_t thr = hn == k ? m.hkey[cur * k + k - 1] : kEmpty;
-      const uint32_t thr_hi = (uint32_t)(thr >> 32);
-      if (tid >= cs && tid < cs + chunk && p < n && dkey <= thr_hi) {
-        const uint32_t id = __ldg(&a.ids[m.srow[st * TR + tid]]);
-        const uint64_t key = ((uint64_t)dkey << 32) | id;
-        if (key < thr) sk_buf[atomicAdd(cnt, 1)] = key;
-      }
-      if (tid == 0) m.sctl[1 + (ci + 1) % 3] = 0;  // counter of the next chunk
-      __syncthreads();
-      const int ns = *cnt;
-      const int roundno = rounds + 1;
-      if (ns > 0) {
-        const int nxt = cur ^ 1;
-        const uint64_t *H = m.hkey + cur * k;
-        // merged order: by key; on equal keys (possible only when an index
-        // stores a row twice) H before S, and S by slot, so ranks are unique
-        for (int i = tid; i < ns; i += TR) {
-          const uint64_t sk = sk_buf[i];
-          int lo = 0, hi = hn;  // # of H at or below sk
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (H[mid] <= sk) lo = mid + 1; else hi = mid;
-          }
-          int r = lo;
-          for (int j = 0; j < ns; ++j) r += (sk_buf[j] < sk || (sk_buf[j] == sk && j < i)) ? 1 : 0;
-          if (r < k) {
-            m.hkey[nxt * k + r] = sk;
-            m.htag[nxt * k + r] = roundno;
-          }
-        }
-        for (int j = tid; j < hn; j += TR) {
-          const uint64_t hk = H[j];
-          int r = j;
-          for (int i = 0; i < ns; ++i) r += sk_buf[i] < hk ? 1 : 0;
-          if (r < k) {
-            m.hkey[nxt * k + r] = hk;
-            m.htag[nxt * k + r] = m.htag[cur * k + j];
-          }
-        }
-        __syncthreads();
-        cur = nxt;
-        hn = hn + ns < k ? hn + ns : k;
-      }
-      const uint32_t cend = n - cstart > (uint32_t)chunk ? cstart + chunk : n;
-      if ((cend & rmask_round) == 0 || cend >= n) {  // round complete
-        rounds = roundno;
-        done = cend;
-        int newc = 0, frontc = 0;
-        for (int i = lane; i < hn; i += 32) {
-          const bool nw = m.htag[cur * k + i] == roundno;
-          newc += nw ? 1 : 0;
-          frontc += (nw && i < a.nfront) ? 1 : 0;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          newc += __shfl_xor_sync(kFull, newc, o);
-          frontc += __shfl_xor_sync(kFull, frontc, o);
-        }
-        const bool lowq = newc < a.u_min && frontc < a.f_min;
-        low = lowq ? low + 1 : 0;
-        stop = a.t_low > 0 && hn == k && roundno >= a.r_min && low >= a.t_low;
-      }
-    }
-    st = st + 1 == STAGES ? 0 : st + 1;
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  // output, sorted by (distance, id), padded
-  const uint64_t *H = m.hkey + cur * k;
-  for (int i = tid; i < k; i += TR) {
-    int64_t id = -1;
-    float d = __int_as_float(0x7f800000);
-    if (i < hn) {
-      const uint64_t kk = H[i];
-      id = (int64_t)(uint32_t)kk;
-      const uint32_t db = (uint32_t)(kk >> 32);
-      d = DT == 0 ? (float)db : __uint_as_float(db);
-    }
-    out_ids[i] = id;
-    out_d[i] = d;
-  }
-  if (tid == 0 && stats) {
-    stats[0] = (int64_t)done;
-    stats[1] = rounds;
-  }
-  __syncthreads();
-}
-
-// ============================================================== refine, long rows
-// fp32 rows too long for whole-row stages (D above 256): each tile of TR rows
-// is staged in pieces of KCC 16-byte chunks of every row (TR x 16 KCC bytes a
-// stage), and each thread carries its row's distance from piece to piece, so
-// the sum over j stays the sequential fmaf chain of refine_block; the merge,
-// rounds and stop rule are refine_block's. row_bytes is a multiple of 16 KCC.
-template <int TR, int STAGES, int KCC>
-__host__ __device__ inline size_t refine_split_smem_bytes(int64_t row_bytes, int k) {
-  return (size_t)STAGES * TR * KCC * 16 + (size_t)row_bytes + (size_t)2 * TR * 4 +
-         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)2 * k * 4 + 16;
-}
-
-template <int TR, int STAGES, int KCC>
-__device__ __forceinline__ RefineSmem refine_split_carve(unsigned char *base, int64_t row_bytes,
-                                                         int k) {
-  RefineSmem m;
-  m.stage = base;
-  m.sq = base + (size_t)STAGES * TR * KCC * 16;
-  m.srow = reinterpret_cast<uint32_t *>(m.sq + row_bytes);  // 2 x TR: rows of the open tiles
   m.hkey = reinterpret_cast<uint64_t *>(m.srow + 2 * TR);
   m.skey = m.hkey + 2 * k;
   m.htag = reinterpret_cast<int *>(m.skey + 2 * TR);
@@ -296,178 +136,514 @@ __device__ __forceinline__ RefineSmem refine_split_carve(unsigned char *base, in
   return m;
 }
 
-template <int TR, int STAGES, int KCC>
-__device__ __forceinline__ void refine_block_split(const RefineParams &a, const RefineSmem &m,
-                                                   uint32_t n, int nl, const nr_seg *segs,
-                                                   int64_t *out_ids, float *out_d, int64_t *stats) {
-  constexpr int swz = KCC % 8 == 0 ? 7 : KCC % 4 == 0 ? 3 : KCC % 2 == 0 ? 1 : 0;
-  constexpr uint32_t PB = KCC * 16;  // bytes of one row in one stage
+// Top-k state of a block (uniform in the block): which buffer, members,
+// rounds done, consecutive low-quality rounds, stopped.
+struct SpanRun {
+  int cur, hn, rounds, low;
+  bool stop;
+};
+
+// The stop rule after round `roundno` with newc members entered in it, frontc
+// of them in the front slots.
+__device__ __forceinline__ void round_done(const RefineParams &a, SpanRun &r, int roundno, int newc,
+                                           int frontc) {
+  r.rounds = roundno;
+  r.low = newc < a.u_min && frontc < a.f_min ? r.low + 1 : 0;
+  r.stop = a.t_low > 0 && r.hn == a.k && roundno >= a.r_min && r.low >= a.t_low;
+}
+// The same after m rounds that changed nothing.
+__device__ __forceinline__ void rounds_unchanged(const RefineParams &a, SpanRun &r, int m) {
+  if (m <= 0) return;
+  const bool lowq = 0 < a.u_min && 0 < a.f_min;
+  if (a.t_low > 0 && r.hn == a.k && lowq) {
+    const int j = max(1, max(a.r_min - r.rounds, a.t_low - r.low));  // the round that stops
+    if (j <= m) {
+      r.rounds += j;
+      r.low += j;
+      r.stop = true;
+      return;
+    }
+  }
+  r.rounds += m;
+  r.low = lowq ? r.low + m : 0;
+}
+
+// The members that entered the top-k in round `roundno` (all of them, those in
+// the front slots), counted by a warp.
+__device__ __forceinline__ void count_new(const RefineSmem &m, const SpanRun &r, int k, int nfront,
+                                          int roundno, int &newc, int &frontc) {
+  newc = frontc = 0;
+  for (int i = threadIdx.x & 31; i < r.hn; i += 32) {
+    const bool nw = m.htag[r.cur * k + i] == roundno;
+    newc += nw ? 1 : 0;
+    frontc += (nw && i < nfront) ? 1 : 0;
+  }
+  newc = __reduce_add_sync(kFull, newc);
+  frontc = __reduce_add_sync(kFull, frontc);
+}
+
+// Last index in [lo, hi) with f(index) <= x, by a whole warp, 32 probes a
+// step; f nondecreasing, f(lo) <= x.
+template <class F>
+__device__ __forceinline__ int warp_last_le(int lo, int hi, uint32_t x, F f) {
+  const int lane = threadIdx.x & 31;
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) / 32, i = lo + lane * step;
+    const unsigned b = __ballot_sync(kFull, i < hi && f(i) <= x);
+    lo += (__popc(b) - 1) * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// Where a span that is not refined on the query's own top-k is logged.
+struct SpanLog {
+  const unsigned long long *nthr;  // the query's committed threshold
+  unsigned long long *pool_used;
+  SpanEntry *pool;
+  uint32_t pool_cap;
+  // out (warp 0): groups logged, the first and the last one, and whether the
+  // pool was full
+  uint32_t groups, off, last;
+  bool full;
+};
+
+// Positions [p0, p1) of a query's stream of nl segments, p0 a whole number of
+// rounds and of tiles, p1 the stream's end or a whole number of rounds. The
+// caller has written the query row into m.sq (block-visible after this
+// function's first barrier). direct: r is the query's top-k, and the stop rule
+// ends the span; else r is the span's own, empty at first, and the members
+// that enter are logged. Whole block (TR threads) calls; ends with a barrier.
+template <int DT, int TR, int CPR, int KCC>
+__device__ __forceinline__ void refine_span(const RefineParams &a, const RefineSmem &m, uint32_t p0,
+                                            uint32_t p1, int nl, const nr_seg *segs, bool direct,
+                                            SpanRun &r, SpanLog &lg) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t RB = (int64_t)a.cpr * 16;
-  const int nk = a.cpr / KCC;  // pieces per row
-  const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(m.stage);
   const int k = a.k;
   const int chunk = a.R < TR ? a.R : TR;
-  const uint32_t ntiles = (uint32_t)(((uint64_t)n + TR - 1) / TR);
-  const uint32_t nitems = ntiles * (uint32_t)nk;
+  const uint32_t ntiles = (uint32_t)(((uint64_t)(p1 - p0) + TR - 1) / TR);
   if (tid == 0) m.sctl[1] = m.sctl[2] = m.sctl[3] = 0;
   __syncthreads();  // the caller's copy of the query row into m.sq is visible after this
 
-  int seg_i = 0;       // this thread's segment cursor (positions only grow)
-  uint32_t grow = 0;   // this thread's row in the tile being issued
-  auto issue = [&](uint32_t it, int st) {
-    if (it < nitems) {
-      const uint32_t t = it / (uint32_t)nk;
-      const int kk = (int)(it - t * (uint32_t)nk);
-      if (kk == 0) {  // a new tile: find this thread's row
-        const uint32_t p = t * TR + tid;
-        grow = 0;
-        if (p < n) {
-          int step = 1;
-          while (seg_i + step < nl && segs[seg_i + step].pos <= p) {
-            seg_i += step;
-            step <<= 1;
-          }
-          for (step >>= 1; step > 0; step >>= 1)
-            if (seg_i + step < nl && segs[seg_i + step].pos <= p) seg_i += step;
-          grow = segs[seg_i].row0 + (p - segs[seg_i].pos);
-          m.srow[(t & 1) * TR + tid] = grow;
-        }
-      }
-      const uint32_t wbase = t * TR + warp * 32;
-      const uint32_t sbase = stage_s + (uint32_t)((size_t)st * TR * PB);
-#pragma unroll 4
-      for (int f = lane; f < 32 * KCC; f += 32) {
-        const int rr = f / KCC;
-        const int c = f - rr * KCC;
-        const uint32_t gr = __shfl_sync(kFull, grow, rr);
-        if (wbase + rr < n) {
-          const int r = warp * 32 + rr;
-          const uint32_t dst = sbase + (uint32_t)(r * PB) + (uint32_t)((c ^ (r & swz)) << 4);
-          cp_async16(dst, a.vec + (size_t)gr * RB + (size_t)kk * PB + ((size_t)c << 4));
-        }
-      }
+  // The warp's window of 32 segments, one a lane: where it begins in the
+  // stream and the stored row less that (positions past the list: none).
+  // Positions only grow, so a window serves many tiles.
+  int wseg = 0;
+  uint32_t wpos = 0xffffffffu, wdelta = 0;
+  auto window = [&](int at) {
+    wseg = at;
+    const nr_seg sg = segs[min(at + lane, nl - 1)];
+    wpos = at + lane < nl ? sg.pos : 0xffffffffu;
+    wdelta = sg.row0 - sg.pos;
+  };
+  if (p0 < p1)
+    window(p0 == 0 ? 0
+                   : warp_last_le(0, nl, min(p0 + (uint32_t)warp * 32u, p1 - 1u),
+                                  [&](int i) { return segs[i].pos; }));
+  // the stored row of this thread in tile t (row 0 past the span); whole warp
+  auto row_of = [&](uint32_t t) {
+    const uint32_t first = p0 + t * TR + warp * 32u, p = first + lane;
+    if (first >= p1) return 0u;
+    const uint32_t last = min(first + 31u, p1 - 1u);
+    int head;  // segments of the window that begin at or before the first row
+    for (;;) {
+      head = __popc(__ballot_sync(kFull, wpos <= first));
+      if (__shfl_sync(kFull, wpos, 31) > last || head <= 1) break;
+      window(wseg + head - 1);
     }
-    cp_async_commit();
+    // a bit for each row of the warp that begins a segment after the first's
+    const bool starts = wpos > first && wpos <= last;
+    const unsigned bits = __reduce_or_sync(kFull, starts ? 1u << (wpos - first) : 0u);
+    if (__popc(__ballot_sync(kFull, starts)) == __popc(bits)) {
+      const int i = head - 1 + __popc(bits & (0xffffffffu >> (31 - lane)));
+      const uint32_t row = __shfl_sync(kFull, wdelta, i) + p;
+      return p < p1 ? row : 0u;
+    }
+    // segments without rows share their place with the next: the last one counts
+    int i = wseg;
+    while (i + 1 < nl && segs[i + 1].pos <= min(p, last)) ++i;
+    return p < p1 ? segs[i].row0 + (p - segs[i].pos) : 0u;
   };
 
-  for (int s = 0; s < STAGES - 1; ++s) issue((uint32_t)s, s);
-  int cur = 0, hn = 0, rounds = 0, low = 0, ci = 0;
-  bool stop = false;
-  uint32_t done = 0;
-  const uint32_t rmask_round = (uint32_t)a.R - 1u;
-  int st = 0;
-  float acc = 0.0f;  // sequential over j across the pieces of a row
-  for (uint32_t it = 0; it < nitems && !stop; ++it) {
-    issue(it + STAGES - 1, st == 0 ? STAGES - 1 : st - 1);
-    cp_async_wait<STAGES - 1>();
-    __syncwarp();
-    const uint32_t t = it / (uint32_t)nk;
-    const int kk = (int)(it - t * (uint32_t)nk);
-    const uint32_t p = t * TR + tid;
-    if (p < n) {
-      const unsigned char *row = m.stage + (size_t)st * TR * PB + (size_t)tid * PB;
-      const float4 *q4 = reinterpret_cast<const float4 *>(m.sq + (size_t)kk * PB);
-#pragma unroll 4
-      for (int c = 0; c < KCC; ++c) {
-        const float4 v = *reinterpret_cast<const float4 *>(row + ((c ^ (tid & swz)) << 4));
-        const float4 w = q4[c];
-        float d;
-        d = __fsub_rn(v.x, w.x); acc = __fmaf_rn(d, d, acc);
-        d = __fsub_rn(v.y, w.y); acc = __fmaf_rn(d, d, acc);
-        d = __fsub_rn(v.z, w.z); acc = __fmaf_rn(d, d, acc);
-        d = __fsub_rn(v.w, w.w); acc = __fmaf_rn(d, d, acc);
-      }
-    }
-    st = st + 1 == STAGES ? 0 : st + 1;
-    if (kk + 1 < nk) continue;  // the row is not complete yet
-    const uint32_t dkey = p < n ? __float_as_uint(acc) : 0xffffffffu;
-    acc = 0.0f;
-    for (int cs = 0; cs < TR && !stop; cs += chunk, ++ci) {
-      const uint32_t cstart = t * TR + cs;
-      if (cstart >= n) break;
+  int ci = 0;
+  bool changed = false;  // the top-k in this round
+  const uint32_t rmask_round = (uint32_t)a.R - 1u;  // R is a power of two
+  lg.groups = 0;
+  lg.full = false;
+  // The committed threshold of the query, as the load of the previous tile
+  // found it: a stale one only keeps more rows than it need, and waiting for
+  // the load here would add an L2 latency to every tile.
+  unsigned long long nthr = direct ? 0ull : __ldcg(lg.nthr);
+  // Merges a tile (dkey: this thread's distance, row: its stored row) chunk by
+  // chunk; a round ends every R stream positions. One block barrier per chunk
+  // (two when the top-k changes): survivor counters rotate over three slots
+  // and survivor buffers over two, and every warp evaluates the stop rule
+  // itself from the shared top-k.
+  auto merge = [&](uint32_t t, uint32_t dkey, uint32_t row, uint64_t ext) {
+    const uint32_t p = p0 + t * TR + tid;
+    for (int cs = 0; cs < TR && !r.stop; cs += chunk, ++ci) {
+      const uint32_t cstart = p0 + t * TR + cs;
+      if (cstart >= p1) break;
       int *cnt = &m.sctl[1 + ci % 3];
       uint64_t *sk_buf = m.skey + (ci & 1) * TR;
-      const uint64_t thr = hn == k ? m.hkey[cur * k + k - 1] : kEmpty;
+      uint64_t thr = r.hn == k ? m.hkey[r.cur * k + k - 1] : kEmpty;
+      if (ext < thr) thr = ext;
       const uint32_t thr_hi = (uint32_t)(thr >> 32);
-      if (tid >= cs && tid < cs + chunk && p < n && dkey <= thr_hi) {
-        const uint32_t id = __ldg(&a.ids[m.srow[(t & 1) * TR + tid]]);
+      if (tid >= cs && tid < cs + chunk && p < p1 && dkey <= thr_hi) {
+        const uint32_t id = __ldg(&a.ids[row]);
         const uint64_t key = ((uint64_t)dkey << 32) | id;
         if (key < thr) sk_buf[atomicAdd(cnt, 1)] = key;
       }
-      if (tid == 0) m.sctl[1 + (ci + 1) % 3] = 0;
+      if (tid == 0) m.sctl[1 + (ci + 1) % 3] = 0;  // counter of the next chunk
       __syncthreads();
       const int ns = *cnt;
-      const int roundno = rounds + 1;
+      const int roundno = r.rounds + 1;
       if (ns > 0) {
-        const int nxt = cur ^ 1;
-        const uint64_t *H = m.hkey + cur * k;
+        const int nxt = r.cur ^ 1;
+        const uint64_t *H = m.hkey + r.cur * k;
+        // merged order: by key; on equal keys (possible only when an index
+        // stores a row twice) H before S, and S by slot, so ranks are unique
         for (int i = tid; i < ns; i += TR) {
           const uint64_t sk = sk_buf[i];
-          int lo = 0, hi = hn;
+          int lo = 0, hi = r.hn;  // # of H at or below sk
           while (lo < hi) {
             const int mid = (lo + hi) >> 1;
             if (H[mid] <= sk) lo = mid + 1; else hi = mid;
           }
-          int r = lo;
-          for (int j = 0; j < ns; ++j) r += (sk_buf[j] < sk || (sk_buf[j] == sk && j < i)) ? 1 : 0;
-          if (r < k) {
-            m.hkey[nxt * k + r] = sk;
-            m.htag[nxt * k + r] = roundno;
+          int rk = lo;
+          for (int j = 0; j < ns; ++j) rk += (sk_buf[j] < sk || (sk_buf[j] == sk && j < i)) ? 1 : 0;
+          if (rk < k) {
+            m.hkey[nxt * k + rk] = sk;
+            m.htag[nxt * k + rk] = roundno;
           }
         }
-        for (int j = tid; j < hn; j += TR) {
+        for (int j = tid; j < r.hn; j += TR) {
           const uint64_t hk = H[j];
-          int r = j;
-          for (int i = 0; i < ns; ++i) r += sk_buf[i] < hk ? 1 : 0;
-          if (r < k) {
-            m.hkey[nxt * k + r] = hk;
-            m.htag[nxt * k + r] = m.htag[cur * k + j];
+          int rk = j;
+          for (int i = 0; i < ns; ++i) rk += sk_buf[i] < hk ? 1 : 0;
+          if (rk < k) {
+            m.hkey[nxt * k + rk] = hk;
+            m.htag[nxt * k + rk] = m.htag[r.cur * k + j];
           }
         }
         __syncthreads();
-        cur = nxt;
-        hn = hn + ns < k ? hn + ns : k;
+        r.cur = nxt;
+        r.hn = r.hn + ns < k ? r.hn + ns : k;
+        changed = true;
       }
-      const uint32_t cend = n - cstart > (uint32_t)chunk ? cstart + chunk : n;
-      if ((cend & rmask_round) == 0 || cend >= n) {
-        rounds = roundno;
-        done = cend;
+      const uint32_t cend = p1 - cstart > (uint32_t)chunk ? cstart + chunk : p1;
+      if ((cend & rmask_round) == 0 || cend >= p1) {  // round complete
         int newc = 0, frontc = 0;
-        for (int i = lane; i < hn; i += 32) {
-          const bool nw = m.htag[cur * k + i] == roundno;
-          newc += nw ? 1 : 0;
-          frontc += (nw && i < a.nfront) ? 1 : 0;
+        if (changed) count_new(m, r, k, a.nfront, roundno, newc, frontc);
+        changed = false;
+        if (direct) {
+          round_done(a, r, roundno, newc, frontc);
+        } else {
+          r.rounds = roundno;
+          if (warp == 0 && newc > 0 && !lg.full) {  // log the members that entered
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(lg.pool_used, (unsigned long long)newc + 1ull);
+            at = __shfl_sync(kFull, at, 0);
+            lg.full = at + (unsigned)newc + 1u > lg.pool_cap;
+            if (!lg.full) {
+              SpanEntry *g = lg.pool + at;
+              if (lane == 0) {
+                *reinterpret_cast<ulonglong2 *>(g) = make_ulonglong2(
+                    kEmpty, (unsigned long long)(roundno - 1) | ((unsigned long long)newc << 32));
+                if (lg.groups > 0) lg.pool[lg.last].key = at;
+              }
+              int e = 1;
+              for (int i0 = 0; i0 < r.hn; i0 += 32) {
+                const bool nw = i0 + lane < r.hn && m.htag[r.cur * k + i0 + lane] == roundno;
+                const unsigned b = __ballot_sync(kFull, nw);
+                if (nw) g[e + __popc(b & ((1u << lane) - 1u))].key = m.hkey[r.cur * k + i0 + lane];
+                e += __popc(b);
+              }
+              if (lg.groups == 0) lg.off = (uint32_t)at;
+              lg.last = (uint32_t)at;
+              ++lg.groups;
+            }
+          }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-          newc += __shfl_xor_sync(kFull, newc, o);
-          frontc += __shfl_xor_sync(kFull, frontc, o);
-        }
-        const bool lowq = newc < a.u_min && frontc < a.f_min;
-        low = lowq ? low + 1 : 0;
-        stop = a.t_low > 0 && hn == k && roundno >= a.r_min && low >= a.t_low;
       }
     }
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  const uint64_t *H = m.hkey + cur * k;
-  for (int i = tid; i < k; i += TR) {
-    int64_t id = -1;
-    float d = __int_as_float(0x7f800000);
-    if (i < hn) {
-      const uint64_t kk2 = H[i];
-      id = (int64_t)(uint32_t)kk2;
-      d = __uint_as_float((uint32_t)(kk2 >> 32));
+  };
+
+  if constexpr (kRow128<DT, CPR>) {
+    // uint8 rows of 128 bytes lie in the stages as they are (eight lanes copy
+    // a row, so a copy's place is the lane's plus a constant); thread i reads
+    // its row's pieces in the order c ^ (i & 7), without bank conflicts, and
+    // holds the query's pieces in registers in that order. With the segment
+    // window this takes 373 warp instructions per 32 rows where swizzled
+    // stages and a search per tile took 523: 4-15% of a batch of 300 to 1,300
+    // queries (1,000 queries x 30,000 rows 672 -> 625 us); at 10,000 queries
+    // HBM binds either way.
+    uint4 w[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) w[c] = reinterpret_cast<const uint4 *>(m.sq)[c ^ (lane & 7)];
+    const uint8_t *piece = a.vec + (lane & 7) * 16;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(m.stage) + (uint32_t)(warp * 4096 + lane * 16);
+    const uint32_t mine = (uint32_t)(tid * 128 + (lane & 7) * 16);
+    uint32_t row = 0, next = 0;
+    auto issue = [&](uint32_t t, uint32_t st) {
+      if (t < ntiles) {
+        next = row_of(t);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint32_t gr = __shfl_sync(kFull, next, i * 4 + (lane >> 3));
+          cp_async16(dst + st * (TR * 128u) + i * 512u, piece + (size_t)gr * 128);
+        }
+      }
+      cp_async_commit();
+    };
+    issue(0u, 0u);
+    for (uint32_t t = 0; t < ntiles && !r.stop; ++t) {
+      row = next;
+      issue(t + 1, (t + 1) & 1u);
+      const uint64_t ext = ~nthr;
+      if (!direct) nthr = __ldcg(lg.nthr);
+      cp_async_wait<1>();
+      __syncwarp();
+      const uint32_t at = mine + (t & 1u) * (TR * 128u);
+      unsigned a0 = 0, a1 = 0, a2 = 0, a3 = 0;  // integer sums: any order is exact
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(m.stage + (at ^ (c * 16u)));
+        unsigned d;
+        d = __vabsdiffu4(v.x, w[c].x); a0 = __dp4a(d, d, a0);
+        d = __vabsdiffu4(v.y, w[c].y); a1 = __dp4a(d, d, a1);
+        d = __vabsdiffu4(v.z, w[c].z); a2 = __dp4a(d, d, a2);
+        d = __vabsdiffu4(v.w, w[c].w); a3 = __dp4a(d, d, a3);
+      }
+      merge(t, (a0 + a1) + (a2 + a3), row, ext);
     }
-    out_ids[i] = id;
-    out_d[i] = d;
-  }
-  if (tid == 0 && stats) {
-    stats[0] = (int64_t)done;
-    stats[1] = rounds;
+    cp_async_wait<0>();
+  } else {
+    const int cpr = CPR > 0 ? CPR : a.cpr;
+    constexpr int swz_c = KCC > 0 ? KCC : CPR;
+    const int swz = swz_c > 0 ? ((swz_c % 8 == 0) ? 7 : (swz_c % 4 == 0) ? 3 : (swz_c % 2 == 0) ? 1 : 0)
+                              : a.swz_mask;
+    const int64_t RB = (int64_t)cpr * 16;
+    const int pc = KCC > 0 ? KCC : cpr;       // chunks of a row in a stage
+    const uint32_t PB = (uint32_t)pc * 16u;   // bytes of a row in a stage
+    const uint32_t nk = KCC > 0 ? (uint32_t)(cpr / KCC) : 1u;  // pieces per row
+    const uint32_t nitems = ntiles * nk;
+    const uint32_t stage_s = (uint32_t)__cvta_generic_to_shared(m.stage);
+    uint32_t grow = 0;  // this thread's row in the tile being issued
+    auto issue = [&](uint32_t it, int st) {
+      if (it < nitems) {
+        const uint32_t t = KCC > 0 ? it / nk : it;
+        const uint32_t kk = KCC > 0 ? it - t * nk : 0u;
+        if (KCC == 0 || kk == 0) {  // a new tile
+          grow = row_of(t);
+          m.srow[(t & 1u) * TR + tid] = grow;
+        }
+        const uint32_t wbase = p0 + t * TR + warp * 32;
+        const uint32_t sbase = stage_s + (uint32_t)((size_t)st * TR * PB);
+#pragma unroll 4
+        for (int f = lane; f < 32 * pc; f += 32) {
+          const int rr = f / pc;
+          const int c = f - rr * pc;
+          const uint32_t gr = __shfl_sync(kFull, grow, rr);
+          if (wbase + rr < p1) {
+            const int row = warp * 32 + rr;
+            const uint32_t dst = sbase + (uint32_t)(row * PB) + (uint32_t)((c ^ (row & swz)) << 4);
+            cp_async16(dst, a.vec + (size_t)gr * RB + (size_t)kk * PB + ((size_t)c << 4));
+          }
+        }
+      }
+      cp_async_commit();
+    };
+    issue(0u, 0);
+    float acc = 0.0f;  // a long row's distance so far
+    for (uint32_t it = 0; it < nitems && !r.stop; ++it) {
+      issue(it + 1, (int)((it + 1) & 1u));
+      const uint64_t ext = ~nthr;
+      if (!direct) nthr = __ldcg(lg.nthr);
+      cp_async_wait<1>();
+      __syncwarp();
+      const uint32_t t = KCC > 0 ? it / nk : it;
+      const uint32_t kk = KCC > 0 ? it - t * nk : 0u;
+      uint32_t dkey = 0xffffffffu;
+      if (p0 + t * TR + tid < p1) {
+        const unsigned char *row = m.stage + (size_t)(it & 1u) * TR * PB + (size_t)tid * PB;
+        if (DT == 0) {
+          unsigned a0 = 0, a1 = 0, a2 = 0, a3 = 0;  // integer sums: any order is exact
+#pragma unroll 8
+          for (int c = 0; c < cpr; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(row + ((c ^ (tid & swz)) << 4));
+            const uint4 w = reinterpret_cast<const uint4 *>(m.sq)[c];
+            unsigned d;
+            d = __vabsdiffu4(v.x, w.x); a0 = __dp4a(d, d, a0);
+            d = __vabsdiffu4(v.y, w.y); a1 = __dp4a(d, d, a1);
+            d = __vabsdiffu4(v.z, w.z); a2 = __dp4a(d, d, a2);
+            d = __vabsdiffu4(v.w, w.w); a3 = __dp4a(d, d, a3);
+          }
+          dkey = (a0 + a1) + (a2 + a3);
+        } else {
+          const float4 *q4 = reinterpret_cast<const float4 *>(m.sq + (size_t)kk * PB);
+          if (KCC == 0) acc = 0.0f;  // sequential over j: the order fixes the rounding
+#pragma unroll 4
+          for (int c = 0; c < pc; ++c) {
+            const float4 v = *reinterpret_cast<const float4 *>(row + ((c ^ (tid & swz)) << 4));
+            const float4 w = q4[c];
+            float d;
+            d = __fsub_rn(v.x, w.x); acc = __fmaf_rn(d, d, acc);
+            d = __fsub_rn(v.y, w.y); acc = __fmaf_rn(d, d, acc);
+            d = __fsub_rn(v.z, w.z); acc = __fmaf_rn(d, d, acc);
+            d = __fsub_rn(v.w, w.w); acc = __fmaf_rn(d, d, acc);
+          }
+          dkey = __float_as_uint(acc);
+        }
+      }
+      if (KCC > 0) {
+        if (kk + 1 < nk) continue;  // the row is not complete yet
+        acc = 0.0f;
+      }
+      merge(t, dkey, m.srow[(t & 1u) * TR + tid], ext);
+    }
+    cp_async_wait<0>();
   }
   __syncthreads();
+}
+
+// Merges the keys of the lanes in `group` into the top-k, tagged with round
+// `roundno`, by one warp: the same merged order as refine_span's.
+__device__ __forceinline__ void warp_insert(const RefineSmem &m, SpanRun &r, int k, uint64_t key,
+                                            unsigned group, int roundno) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t *H = m.hkey + r.cur * k;
+  const bool in = ((group >> lane) & 1u) && (r.hn < k || key < H[k - 1]);
+  const unsigned sv = __ballot_sync(kFull, in);
+  if (!sv) return;
+  const int nxt = r.cur ^ 1;
+  int rk = 0;
+  if (in) {
+    int lo = 0, hi = r.hn;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (H[mid] <= key) lo = mid + 1; else hi = mid;
+    }
+    rk = lo;
+  }
+  for (unsigned b = sv; b; b &= b - 1) {
+    const int src = __ffs(b) - 1;
+    const uint64_t o = __shfl_sync(kFull, key, src);
+    rk += (o < key || (o == key && src < lane)) ? 1 : 0;
+  }
+  if (in && rk < k) {
+    m.hkey[nxt * k + rk] = key;
+    m.htag[nxt * k + rk] = roundno;
+  }
+  for (int j0 = 0; j0 < r.hn; j0 += 32) {
+    const int j = j0 + lane;
+    const uint64_t hk = j < r.hn ? H[j] : kEmpty;
+    int hr = j;
+    for (unsigned b = sv; b; b &= b - 1) {
+      const uint64_t o = __shfl_sync(kFull, key, __ffs(b) - 1);
+      hr += o < hk ? 1 : 0;
+    }
+    if (j < r.hn && hr < k) {
+      m.hkey[nxt * k + hr] = hk;
+      m.htag[nxt * k + hr] = m.htag[r.cur * k + j];
+    }
+  }
+  __syncwarp();
+  r.cur = nxt;
+  r.hn = min(k, r.hn + __popc(sv));
+}
+
+// Commits a logged span of nr rounds to the query's top-k, by one warp: its
+// first group of log entries starts at off of the pool, with its first kStaged
+// entries in shared memory.
+__device__ __forceinline__ void commit_span(const RefineParams &a, const RefineSmem &m, SpanRun &r,
+                                            const SpanEntry *pool, uint64_t off,
+                                            const uint4 *staged, int nr) {
+  const int lane = threadIdx.x & 31, k = a.k;
+  int done = 0;  // rounds of the span committed
+  uint4 v = staged[lane];
+  for (uint64_t at = off;;) {
+    const uint64_t key = ((uint64_t)v.y << 32) | v.x;
+    const uint64_t nextat = __shfl_sync(kFull, key, 0);
+    const int round = (int)__shfl_sync(kFull, v.z, 0), cnt = (int)__shfl_sync(kFull, v.w, 0);
+    rounds_unchanged(a, r, round - done);
+    if (r.stop) return;
+    const int roundno = r.rounds + 1;
+    warp_insert(m, r, k, key, __ballot_sync(kFull, lane >= 1 && lane <= cnt), roundno);
+    for (int e0 = 32; e0 <= cnt; e0 += 32) {
+      const int e = e0 + lane;
+      const uint64_t kk = e <= cnt ? __ldcg(&pool[at + e].key) : kEmpty;
+      warp_insert(m, r, k, kk, __ballot_sync(kFull, e <= cnt), roundno);
+    }
+    int newc, frontc;
+    count_new(m, r, k, a.nfront, roundno, newc, frontc);
+    round_done(a, r, roundno, newc, frontc);
+    if (r.stop) return;
+    done = round + 1;
+    if (nextat == kEmpty) break;
+    at = nextat;
+    // the next group's first entry, then its members
+    const uint4 h = __ldcg(reinterpret_cast<const uint4 *>(pool + at));
+    v = lane <= (int)h.w ? __ldcg(reinterpret_cast<const uint4 *>(pool + at + lane)) : h;
+  }
+  rounds_unchanged(a, r, nr - done);
+}
+
+// Commits the finished spans from `next` on, in order, to the query's top-k,
+// by one warp: until one is not finished, was not logged (returns true), or
+// the stop. Spans are looked at 32 at a time: those whose smallest key is
+// below the current k-th have their first group's entries staged in shared
+// memory together, so a batch costs two memory latencies and not one a span.
+__device__ __forceinline__ bool commit_ready(const RefineParams &a, const RefineSmem &m, SpanRun &r,
+                                             const SpanEntry *pool, uint32_t cap,
+                                             const uint32_t *ready, const SpanHeader *hdr,
+                                             uint32_t &next, uint32_t spans, uint32_t n,
+                                             uint32_t span_rows, uint4 *stage, int most) {
+  const int lane = threadIdx.x & 31, k = a.k;
+  while (next < spans) {
+    const uint32_t x = next + lane;
+    const uint32_t rdy = lane < most && x < spans ? ld_acquire(&ready[x]) : 0u;
+    const bool logged = rdy > 1u && rdy != kSpanRedo;
+    uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);  // min key, first group
+    if (logged) h = __ldcg(reinterpret_cast<const uint4 *>(hdr + x));
+    const uint64_t mk = ((uint64_t)h.y << 32) | h.x;
+    const unsigned idle = __ballot_sync(kFull, rdy == 0u || rdy == kSpanRedo);
+    const int nb = idle ? __ffs(idle) - 1 : 32;  // finished spans of this batch
+    const bool redo = nb < 32 && __shfl_sync(kFull, rdy, nb) == kSpanRedo;
+    auto below = [&]() {  // spans that can change the top-k
+      const uint64_t kth = r.hn == k ? m.hkey[r.cur * k + k - 1] : kEmpty;
+      return __ballot_sync(kFull, lane < nb && logged && (r.hn < k || mk < kth));
+    };
+    const unsigned want = below();
+    for (unsigned b = want; b; b &= b - 1) {
+      const int j = __ffs(b) - 1;
+      const uint32_t at = __shfl_sync(kFull, h.z, j);
+      if (at + lane < cap)
+        cp_async16((uint32_t)__cvta_generic_to_shared(stage + j * kStaged + lane), pool + at + lane);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncwarp();
+    const int rounds_span = (int)((span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+    int at = 0;  // spans of the batch committed
+    while (at < nb && !r.stop) {
+      const unsigned b = want & below() & (kFull << at);
+      const int j = b ? __ffs(b) - 1 : nb;  // the next one that can change it
+      const bool last = next + nb == spans && j == nb;  // the stream's last span may be short
+      const int tail = (int)((n - (spans - 1u) * span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+      if (j > at) rounds_unchanged(a, r, (j - at - (last ? 1 : 0)) * rounds_span + (last ? tail : 0));
+      at = j;
+      if (r.stop || j == nb) break;
+      commit_span(a, m, r, pool, __shfl_sync(kFull, h.z, j), stage + j * kStaged,
+                  next + j + 1 == spans ? tail : rounds_span);
+      at = j + 1;
+    }
+    next += (uint32_t)at;
+    if (r.stop) return false;
+    if (redo) return true;
+    if (nb < (most < 32 ? most : 32)) return false;  // the next one is not finished
+  }
+  return false;
 }
 
 }  // namespace nrq
