@@ -16,6 +16,7 @@
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -28,8 +29,17 @@ namespace {
 constexpr int kBMax = 24;          // code bits
 constexpr int kKMax = 64;          // clusters per bucket
 constexpr int kMaxSample = 4096;   // sample_per_cluster
-constexpr int64_t kWarpRows = 4096;  // buckets up to this size: one warp; larger: one CTA
-constexpr int kCtaThreads = 256;
+// Buckets up to kWarpRows rows: one warp; up to kCtaRows: one CTA; larger: one
+// CTA of more threads. A bucket's passes follow one another, so the longest
+// bucket of each kind bounds the whole step: with warps up to 4,096 rows one
+// warp's largest bucket took 12.1 ms of a build of 2e6 rows (and the 8 larger
+// ones 2.2 ms in CTAs of 256 threads before it).
+constexpr int64_t kWarpRows = 256;
+constexpr int64_t kCtaRows = 1024;
+constexpr int kCtaThreads = 128;
+constexpr int kHugeThreads = 512;
+// Rows whose fixed-point sums two 32-bit words hold (see add_fixed).
+constexpr int64_t kSumRows = 65536;
 
 // ---------------------------------------------------------------------------
 // Arithmetic of the build definition (identical on the host builder)
@@ -69,9 +79,24 @@ __device__ __forceinline__ int64_t uniform_pick(uint64_t draw, int64_t m) {
   const int64_t p = (int64_t)__dmul_rn(u, (double)m);
   return p < m ? p : m - 1;
 }
-// fp32 squared distance, each product and sum rounded, j ascending
+// fp32 squared distance, each product and sum rounded, j ascending; c 16-byte
+// aligned when b is a multiple of 4
 __device__ __forceinline__ float dist_rn(const float (&l)[kBMax], const float *c, int b) {
   float s = 0.0f;
+  if ((b & 3) == 0) {
+#pragma unroll
+    for (int j = 0; j < kBMax; j += 4)
+      if (j < b) {
+        const float4 v = *reinterpret_cast<const float4 *>(c + j);
+        const float t0 = __fsub_rn(l[j], v.x), t1 = __fsub_rn(l[j + 1], v.y);
+        const float t2 = __fsub_rn(l[j + 2], v.z), t3 = __fsub_rn(l[j + 3], v.w);
+        s = __fadd_rn(s, __fmul_rn(t0, t0));
+        s = __fadd_rn(s, __fmul_rn(t1, t1));
+        s = __fadd_rn(s, __fmul_rn(t2, t2));
+        s = __fadd_rn(s, __fmul_rn(t3, t3));
+      }
+    return s;
+  }
 #pragma unroll
   for (int j = 0; j < kBMax; ++j)
     if (j < b) {
@@ -80,11 +105,39 @@ __device__ __forceinline__ float dist_rn(const float (&l)[kBMax], const float *c
     }
   return s;
 }
+// a row's logits (16-byte loads when b is a multiple of 4: rows are aligned)
 __device__ __forceinline__ void load_logits(const float *__restrict__ L, uint32_t r, int b,
                                             float (&l)[kBMax]) {
   const float *p = L + (size_t)r * b;
+  if ((b & 3) == 0) {
+#pragma unroll
+    for (int j = 0; j < kBMax; j += 4) {
+      const float4 v = j < b ? __ldg(reinterpret_cast<const float4 *>(p + j)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      l[j] = v.x;
+      l[j + 1] = v.y;
+      l[j + 2] = v.z;
+      l[j + 3] = v.w;
+    }
+    return;
+  }
 #pragma unroll
   for (int j = 0; j < kBMax; ++j) l[j] = j < b ? __ldg(p + j) : 0.0f;
+}
+// llrint(x 2^G), |x 2^G| < 2^30: in fp32 where 2^G is one of its normal
+// numbers (the product is exact then, or below 2^-126 and rounds to 0 either
+// way), else in double
+__device__ __forceinline__ int32_t fixed_of(float x, float scalef, double scale) {
+  return scalef != 0.0f ? __float2int_rn(__fmul_rn(x, scalef))
+                        : (int32_t)__double2ll_rn(__dmul_rn((double)x, scale));
+}
+// trunc(d 2^(50 - e)) for 0 <= d <= f 2^e, f < 1 (d below 2^e: the result is
+// below 2^50): the 24-bit significand shifted
+__device__ __forceinline__ unsigned long long weight_of(float d, int e) {
+  const uint32_t u = __float_as_uint(d);
+  const int ex = (int)(u >> 23);
+  const unsigned long long m = ex ? (u & 0x7FFFFFu) | 0x800000u : u & 0x7FFFFFu;
+  const int sh = (ex ? ex : 1) - 150 + 50 - e;  // d = m 2^(max(ex, 1) - 150)
+  return sh >= 0 ? m << sh : sh > -64 ? m >> -sh : 0ull;
 }
 
 // ---------------------------------------------------------------------------
@@ -194,7 +247,8 @@ __global__ void flag_kernel(const uint32_t *__restrict__ cnt, int64_t nb, uint32
     flag[u] = (u < nb && cnt[u] > 0) ? 1u : 0u;
 }
 
-// non-empty codes in order; clusters per bucket K_B; the large-bucket list
+// non-empty codes in order; clusters per bucket K_B; the large-bucket list (nbig[0]
+// of them, nbig[1] above kCtaRows rows)
 __global__ void bucket_list_kernel(const uint32_t *__restrict__ cnt, const uint32_t *__restrict__ pos,
                                    int64_t nb, int K_max, int t, uint32_t *ne_code, uint32_t *kcount,
                                    uint32_t *big_e, uint32_t *big_n, unsigned int *nbig) {
@@ -210,9 +264,10 @@ __global__ void bucket_list_kernel(const uint32_t *__restrict__ cnt, const uint3
     if (K < 1) K = 1;
     kcount[e] = (uint32_t)K;
     if ((int64_t)n > kWarpRows) {
-      const unsigned int i = atomicAdd(nbig, 1u);
+      const unsigned int i = atomicAdd(&nbig[0], 1u);
       big_e[i] = e;
       big_n[i] = n;
+      if ((int64_t)n > kCtaRows) atomicAdd(&nbig[1], 1u);
     }
   }
 }
@@ -236,16 +291,19 @@ struct KmArgs {
   uint32_t *ncl;           // [ne] kept clusters per bucket
   float *dmin;             // [groups x mcap] seeding scratch
   int64_t mcap;
-  unsigned int *counter;   // [2] work counters (warp buckets, CTA buckets)
+  unsigned int *counter;   // [3] work counters (warps, CTAs, large CTAs)
+  int64_t nhuge;           // of the large buckets, those of the large CTAs
   int b, K_max, t, iters, S;
   uint64_t seed;
   double scale, inv_scale;
+  float scalef;            // the scale where fp32 has it, else 0
 };
 
 // shared memory of one group
 struct KmSmem {
-  float *cent;                // [K_max * b]
-  unsigned long long *sum;    // [K_max * b] fixed-point sums
+  float *cent;                // [K_max * b] (16-byte aligned when b is a multiple of 4)
+  uint32_t *sum;              // [2][K_max * b] fixed-point sums, low and high parts
+  long long *total;           // [K_max * b] sums of earlier chunks (CTAs only)
   uint32_t *cnt;              // [K_max]
   int32_t *remap;             // [K_max] kept index or -1
   uint32_t *off;              // [K_max] placement cursor
@@ -257,6 +315,8 @@ struct KmSmem {
 __host__ __device__ inline size_t km_smem_bytes(int K_max, int b, int nw) {
   size_t o = 0;
   o += (size_t)K_max * b * 8;   // sum
+  if (nw > 1) o += (size_t)K_max * b * 8;  // total
+  o = (o + 15) & ~(size_t)15;
   o += (size_t)K_max * b * 4;   // cent
   o += (size_t)K_max * 4 * 3;   // cnt, remap, off
   o += (size_t)nw * K_max * 4;  // wcnt
@@ -267,8 +327,11 @@ __host__ __device__ inline size_t km_smem_bytes(int K_max, int b, int nw) {
 
 __device__ inline KmSmem km_carve(unsigned char *p, int K_max, int b, int nw) {
   KmSmem m;
-  m.sum = reinterpret_cast<unsigned long long *>(p);
+  m.sum = reinterpret_cast<uint32_t *>(p);
   p += (size_t)K_max * b * 8;
+  m.total = reinterpret_cast<long long *>(p);
+  if (nw > 1) p += (size_t)K_max * b * 8;
+  p = reinterpret_cast<unsigned char *>(((uintptr_t)p + 15) & ~(uintptr_t)15);
   m.cent = reinterpret_cast<float *>(p);
   p += (size_t)K_max * b * 4;
   m.cnt = reinterpret_cast<uint32_t *>(p);
@@ -384,9 +447,9 @@ __device__ void kmeans_bucket(const KmArgs &a, int64_t e, const KmSmem &m, float
       gsync<NT>();
       const uint64_t draw = (uint64_t)m.misc[1];
       if (mx > 0.0f) {
-        const double mult = pow2(50 - exponent_of((double)mx));
+        const int top = exponent_of((double)mx);
         unsigned long long local = 0;
-        for (int64_t i = i0; i < i1; ++i) local += (unsigned long long)__dmul_rn((double)dmin[i], mult);
+        for (int64_t i = i0; i < i1; ++i) local += weight_of(dmin[i], top);
         unsigned long long tot;
         const unsigned long long ex = group_excl_scan<NT>(local, m, &tot);
         if (tot > 0) {
@@ -394,7 +457,7 @@ __device__ void kmeans_bucket(const KmArgs &a, int64_t e, const KmSmem &m, float
           if (ex <= r && r < ex + local) {
             unsigned long long acc = ex;
             for (int64_t i = i0; i < i1; ++i) {
-              acc += (unsigned long long)__dmul_rn((double)dmin[i], mult);
+              acc += weight_of(dmin[i], top);
               if (acc > r) {
                 m.misc[0] = i;
                 break;
@@ -411,39 +474,75 @@ __device__ void kmeans_bucket(const KmArgs &a, int64_t e, const KmSmem &m, float
     }
   }
   // Lloyd passes (K = 1: one pass, the mean)
+  const int kb = K * b;
+  uint32_t *lo_sum = m.sum, *hi_sum = m.sum + (size_t)a.K_max * b;
+  auto add_fixed = [&](int at, int32_t v) {
+    // v = 2^15 (v >> 15) + (v & 0x7fff): two native 32-bit adds, which
+    // kSumRows rows cannot overflow, for one 64-bit add (a compare-and-swap
+    // loop in shared memory)
+    atomicAdd(&lo_sum[at], (uint32_t)v & 0x7FFFu);
+    atomicAdd(&hi_sum[at], (uint32_t)(v >> 15));
+  };
   const int iters = K > 1 ? (a.iters > 0 ? a.iters : 1) : 1;
   for (int it = 0; it < iters; ++it) {
-    gsync<NT>();
-    for (int i = g; i < K * b; i += NT) m.sum[i] = 0ull;
-    for (int i = g; i < K; i += NT) m.cnt[i] = 0u;
-    gsync<NT>();
-    for (int64_t i = g; i < n; i += NT) {
-      load_logits(a.L, mem[i], b, l);
-      int best = 0;
-      if (K > 1) {
-        float bd = dist_rn(l, m.cent, b);
-        for (int k = 1; k < K; ++k) {
-          const float d = dist_rn(l, m.cent + (size_t)k * b, b);
-          if (d < bd) {
-            bd = d;
-            best = k;
-          }
+    for (int64_t r0 = 0; r0 < n; r0 += kSumRows) {  // one chunk for most buckets
+      const int64_t r1 = n - r0 < kSumRows ? n : r0 + kSumRows;
+      gsync<NT>();
+      for (int i = g; i < kb; i += NT) {
+        if (NT > 32) {
+          const long long part = r0 == 0 ? 0ll : m.total[i];
+          m.total[i] = r0 == 0 ? 0ll : part + (((long long)(int32_t)hi_sum[i] << 15) + (long long)lo_sum[i]);
         }
-        lab[i] = (uint8_t)best;
+        lo_sum[i] = hi_sum[i] = 0u;
       }
-      atomicAdd(&m.cnt[best], 1u);
+      if (r0 == 0)
+        for (int i = g; i < K; i += NT) m.cnt[i] = 0u;
+      gsync<NT>();
+      if (K == 1) {
+        // every row adds to the same b sums: b threads a row, each its column,
+        // the sums of a thread's rows kept in a register
+        const int per = NT / b, col = g % b, row = g / b;
+        long long acc = 0;
+        if (row < per)
+#pragma unroll 4
+          for (int64_t i = r0 + row; i < r1; i += per)
+            acc += fixed_of(__ldg(a.L + (size_t)mem[i] * b + col), a.scalef, a.scale);
+        if (row < per) {
+          // several rows' sums: in 64 bits, split as add_fixed splits one (the
+          // parts of all threads of a column stay within kSumRows rows' range)
+          atomicAdd(&lo_sum[col], (uint32_t)acc & 0x7FFFu);
+          atomicAdd(&hi_sum[col], (uint32_t)(acc >> 15));
+        }
+        if (g == 0 && r0 == 0) m.cnt[0] = (uint32_t)n;
+      } else {
+        for (int64_t i = r0 + g; i < r1; i += NT) {
+          load_logits(a.L, mem[i], b, l);
+          int best = 0;
+          float bd = dist_rn(l, m.cent, b);
+          for (int k = 1; k < K; ++k) {
+            const float d = dist_rn(l, m.cent + (size_t)k * b, b);
+            if (d < bd) {
+              bd = d;
+              best = k;
+            }
+          }
+          lab[i] = (uint8_t)best;
+          atomicAdd(&m.cnt[best], 1u);
 #pragma unroll
-      for (int j = 0; j < kBMax; ++j)
-        if (j < b)
-          atomicAdd(&m.sum[best * b + j],
-                    (unsigned long long)__double2ll_rn(__dmul_rn((double)l[j], a.scale)));
+          for (int j = 0; j < kBMax; ++j)
+            if (j < b) add_fixed(best * b + j, fixed_of(l[j], a.scalef, a.scale));
+        }
+      }
     }
     gsync<NT>();
-    for (int i = g; i < K * b; i += NT) {
+    for (int i = g; i < kb; i += NT) {
       const uint32_t c = m.cnt[i / b];
-      if (c > 0)
-        m.cent[i] = __double2float_rn(__ddiv_rn(
-            __dmul_rn(__ll2double_rn((long long)m.sum[i]), a.inv_scale), (double)c));
+      if (c > 0) {
+        long long v = ((long long)(int32_t)hi_sum[i] << 15) + (long long)lo_sum[i];
+        if (NT > 32) v += m.total[i];
+        m.cent[i] = __double2float_rn(
+            __ddiv_rn(__dmul_rn(__ll2double_rn(v), a.inv_scale), (double)c));
+      }
     }
   }
   gsync<NT>();
@@ -522,20 +621,23 @@ __global__ void kmeans_warp_kernel(KmArgs a) {
   }
 }
 
-// one CTA per large bucket, largest first; persistent CTAs
-__global__ void __launch_bounds__(kCtaThreads) kmeans_cta_kernel(KmArgs a) {
+// one CTA of NT threads per large bucket [first, last) of the list, largest
+// first; persistent CTAs
+template <int NT>
+__global__ void __launch_bounds__(NT) kmeans_cta_kernel(KmArgs a, int64_t first, int64_t last,
+                                                         unsigned int *counter) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const KmSmem m = km_carve(smem, a.K_max, a.b, kCtaThreads / 32);
+  const KmSmem m = km_carve(smem, a.K_max, a.b, NT / 32);
   float *dmin = a.dmin + (int64_t)blockIdx.x * a.mcap;
   __shared__ long long item;
   for (;;) {
-    for (int k = threadIdx.x; k < (kCtaThreads / 32) * a.K_max; k += kCtaThreads) m.wcnt[k] = 0;
-    if (threadIdx.x == 0) item = (long long)atomicAdd(&a.counter[1], 1u);
+    for (int k = threadIdx.x; k < (NT / 32) * a.K_max; k += NT) m.wcnt[k] = 0;
+    if (threadIdx.x == 0) item = first + (long long)atomicAdd(counter, 1u);
     __syncthreads();
     const int64_t it = item;
     __syncthreads();
-    if (it >= a.nbig) break;
-    kmeans_bucket<kCtaThreads>(a, a.big_e[it], m, dmin);
+    if (it >= last) break;
+    kmeans_bucket<NT>(a, a.big_e[it], m, dmin);
     __syncthreads();
   }
 }
@@ -629,6 +731,32 @@ struct Scratch {
         cudaFree(q);
         q = nullptr;
       }
+  }
+};
+
+// two streams beside the build's, closed (their work done) on every exit
+struct SideStreams {
+  cudaStream_t s[2] = {nullptr, nullptr};
+  cudaError_t open() {
+    for (auto &x : s) {
+      const cudaError_t e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  cudaError_t wait() {
+    cudaError_t r = cudaSuccess;
+    for (auto &x : s)
+      if (x) {
+        const cudaError_t e = cudaStreamSynchronize(x);
+        if (r == cudaSuccess) r = e;
+      }
+    return r;
+  }
+  ~SideStreams() {
+    wait();
+    for (auto &x : s)
+      if (x) cudaStreamDestroy(x);
   }
 };
 
@@ -758,9 +886,10 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
     sc.release(tmp);
   }
   sc.release(flag);
-  uint32_t nslots = 0, nbig = 0;
+  uint32_t nslots = 0, nbig2[2] = {0, 0};
   NRB_TRY(cudaMemcpy(&nslots, kslot + ne, 4, cudaMemcpyDeviceToHost));
-  NRB_TRY(cudaMemcpy(&nbig, d_small, 4, cudaMemcpyDeviceToHost));
+  NRB_TRY(cudaMemcpy(nbig2, d_small, 8, cudaMemcpyDeviceToHost));
+  const uint32_t nbig = nbig2[0], nhuge = nbig2[1];
   // large buckets largest first (the order only balances the load)
   NRB_TRY(sc.alloc(&big_e_s, (size_t)nbig + 1));
   NRB_TRY(sc.alloc(&big_n_s, (size_t)nbig + 1));
@@ -791,8 +920,10 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   a.iters = bd->cfg.lloyd_iters;
   a.S = bd->cfg.sample_per_cluster;
   a.seed = bd->cfg.seed;
+  a.nhuge = nhuge;
   a.scale = pow2(G);
   a.inv_scale = pow2(-G);
+  a.scalef = G >= -126 && G <= 127 ? (float)pow2(G) : 0.0f;
   uint32_t *out_ids;
   NRB_TRY(cudaMalloc((void **)&out_ids, (size_t)N * 4));
   ix->ids = out_ids;  // owned by the index from here on
@@ -806,34 +937,53 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   const int wpb = 8;
   const size_t wsm = km_smem_bytes(ix->K_max, b, 1) * wpb;
   const size_t csm = km_smem_bytes(ix->K_max, b, kCtaThreads / 32);
+  const size_t hsm = km_smem_bytes(ix->K_max, b, kHugeThreads / 32);
+  auto cta = kmeans_cta_kernel<kCtaThreads>;
+  auto huge = kmeans_cta_kernel<kHugeThreads>;
   NRB_TRY(cudaFuncSetAttribute(kmeans_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
-  NRB_TRY(cudaFuncSetAttribute(kmeans_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-  int occ_w = 0, occ_c = 0;
+  NRB_TRY(cudaFuncSetAttribute(cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+  NRB_TRY(cudaFuncSetAttribute(huge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hsm));
+  int occ_w = 0, occ_c = 0, occ_h = 0;
   NRB_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_w, kmeans_warp_kernel, 32 * wpb, wsm));
-  NRB_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, kmeans_cta_kernel, kCtaThreads, csm));
-  if (occ_w < 1 || occ_c < 1) return NR_ERR_INVALID_ARG;
+  NRB_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, cta, kCtaThreads, csm));
+  NRB_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_h, huge, kHugeThreads, hsm));
+  if (occ_w < 1 || occ_c < 1 || occ_h < 1) return NR_ERR_INVALID_ARG;
   const int grid_w = occ_w * nsm;
-  const int grid_c = (int)(nbig < (uint32_t)(occ_c * nsm) ? (nbig > 0 ? nbig : 1) : occ_c * nsm);
-  // seeding scratch: a warp's bucket has at most kWarpRows members; a CTA's
-  // sample at most sample_per_cluster * K_max
-  const int64_t mcap_c = (int64_t)a.S * ix->K_max;
-  const int64_t mcap_w = kWarpRows;
-  float *dmin_w, *dmin_c;
+  const int grid_c = (int)std::min<int64_t>(nbig - nhuge, (int64_t)occ_c * nsm);
+  const int grid_h = (int)std::min<int64_t>(nhuge, (int64_t)occ_h * nsm);
+  // seeding scratch: at most a bucket's rows and sample_per_cluster * K_max
+  const int64_t sample = (int64_t)a.S * ix->K_max;
+  const int64_t mcap_w = std::min(sample, kWarpRows), mcap_c = std::min(sample, kCtaRows);
+  float *dmin_w, *dmin_c, *dmin_h;
   NRB_TRY(sc.alloc(&dmin_w, (size_t)grid_w * wpb * mcap_w));
   NRB_TRY(sc.alloc(&dmin_c, (size_t)grid_c * mcap_c));
-  if (nbig > 0) {
+  NRB_TRY(sc.alloc(&dmin_h, (size_t)grid_h * sample));
+  // the three kinds side by side, each on its own stream: the largest buckets
+  // are the longest chain and start first
+  NRB_TRY(cudaStreamSynchronize(s));  // the lists and counters are written
+  SideStreams side;
+  NRB_TRY(side.open());
+  if (grid_h > 0) {
+    a.dmin = dmin_h;
+    a.mcap = sample;
+    huge<<<grid_h, kHugeThreads, hsm, side.s[0]>>>(a, 0, nhuge, a.counter + 2);
+    NRB_TRY(cudaGetLastError());
+  }
+  if (grid_c > 0) {
     a.dmin = dmin_c;
     a.mcap = mcap_c;
-    kmeans_cta_kernel<<<grid_c, kCtaThreads, csm, s>>>(a);
+    cta<<<grid_c, kCtaThreads, csm, side.s[1]>>>(a, nhuge, nbig, a.counter + 1);
     NRB_TRY(cudaGetLastError());
   }
   a.dmin = dmin_w;
   a.mcap = mcap_w;
   kmeans_warp_kernel<<<grid_w, 32 * wpb, wsm, s>>>(a);
   NRB_TRY(cudaGetLastError());
+  NRB_TRY(side.wait());
   NRB_TRY(cudaStreamSynchronize(s));
   sc.release(dmin_w);
   sc.release(dmin_c);
+  sc.release(dmin_h);
   sc.release(a.labels);
   sc.release(ids_s);
   // bucket -> cluster CSR level: exclusive sum of kept clusters over all codes
