@@ -144,71 +144,87 @@ __device__ __forceinline__ unsigned long long weight_of(float d, int e) {
 // Step 1/2: fixed-point scale and medians
 // ---------------------------------------------------------------------------
 
-__global__ void absmax_kernel(const float *__restrict__ L, int64_t n, unsigned int *out) {
-  unsigned int m = 0;
-  const uint32_t *u = reinterpret_cast<const uint32_t *>(L);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned int v = __ldg(u + i) & 0x7FFFFFFFu;
-    m = v > m ? v : m;
-  }
-  for (int o = 16; o; o >>= 1) {
-    const unsigned int w = __shfl_xor_sync(0xffffffffu, m, o);
-    m = w > m ? w : m;
-  }
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
-}
-
-// histogram of key digit (key >> shift) & 255 per column, over the elements
-// whose higher digits equal prefix[j]
-__global__ void median_hist_kernel(const float *__restrict__ L, int64_t N, int b, int shift,
-                                   const uint32_t *__restrict__ prefix, uint32_t *hist) {
+// Histogram of key digit (key >> shift) & 255 per column, over the elements
+// whose higher digits equal prefix[j]; the first pass (FIRST) also takes the
+// largest |logit|'s bits. The threads taking part are a multiple of b, so each
+// stays in one column: reads are coalesced, and a warp's adds fall on
+// different columns' bins (a warp reading 32 rows of one column needed a
+// __match_any_sync an element: 64 to 146 us a pass over 2e6 x 16 logits, and
+// 32 us for the largest; 27 to 40 us a pass now, bound by the 128 MB read).
+template <bool FIRST>
+__global__ void __launch_bounds__(256) median_hist_kernel(const float *__restrict__ L, int64_t n, int b,
+                                                          int shift, const uint32_t *__restrict__ prefix,
+                                                          uint32_t *hist, unsigned int *amax) {
   extern __shared__ uint32_t sh[];  // [b][256]
-  __shared__ uint32_t spre[kBMax];
   for (int i = threadIdx.x; i < b * 256; i += blockDim.x) sh[i] = 0;
-  if (threadIdx.x < b) spre[threadIdx.x] = prefix[threadIdx.x];
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t base = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; base < N;
-       base += nwarps * 32) {
-    const int64_t r = base + lane;
-    const bool valid = r < N;
-    for (int j = 0; j < b; ++j) {
-      const uint32_t key = valid ? float_key(__ldg(L + (size_t)r * b + j)) : 0u;
-      const bool match = valid && (shift == 24 || (key >> (shift + 8)) == spre[j]);
-      const int bin = match ? j * 256 + (int)((key >> shift) & 255u) : -1;
-      const unsigned peers = __match_any_sync(0xffffffffu, bin);
-      if (match && lane == __ffs(peers) - 1) atomicAdd(&sh[bin], (uint32_t)__popc(peers));
+  const int64_t T = (int64_t)gridDim.x * blockDim.x / b * b;
+  const int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t *u = reinterpret_cast<const uint32_t *>(L);
+  unsigned int m = 0;
+  if (e0 < T) {
+    const int col = (int)(e0 % b);
+    const uint32_t pre = FIRST ? 0u : prefix[col];
+    uint32_t *h = sh + col * 256;
+    auto add = [&](uint32_t x) {
+      const uint32_t key = (x & 0x80000000u) ? ~x : (x | 0x80000000u);  // float_key
+      if (FIRST) m = max(m, x & 0x7FFFFFFFu);
+      if (FIRST || (key >> (shift + 8)) == pre) atomicAdd(&h[(key >> shift) & 255u], 1u);
+    };
+    int64_t e = e0;
+    for (; e + 7 * T < n; e += 8 * T) {
+      uint32_t x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = __ldg(u + e + i * T);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) add(x[i]);
     }
+    for (; e < n; e += T) add(__ldg(u + e));
+  }
+  if (FIRST) {
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(amax, m);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < b * 256; i += blockDim.x)
     if (sh[i]) atomicAdd(&hist[i], sh[i]);
 }
 
-// per column: the digit holding rank[j]; rank and prefix move to it; the
-// column's histogram is cleared for the next pass. After the last digit the
-// prefix is the whole key: tau[j].
-__global__ void median_pick_kernel(uint32_t *hist, uint32_t *prefix, uint32_t *rank, int b,
-                                   int shift, float *tau) {
-  const int j = threadIdx.x;
-  if (j >= b) return;
-  uint32_t *h = hist + j * 256;
+// per column (a warp each): the digit holding rank[j]; rank and prefix move to
+// it; the column's histogram is cleared for the next pass. After the last
+// digit the prefix is the whole key: tau[j]. (Latency: one thread a column
+// walking 256 bins took 20 us a digit.)
+__global__ void median_pick_kernel(uint32_t *hist, uint32_t *prefix, uint32_t *rank, int shift,
+                                   float *tau) {
+  const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t *h = hist + j * 256 + lane * 8;
+  uint32_t c[8], sum = 0;
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    c[d] = h[d];
+    h[d] = 0;
+    sum += c[d];
+  }
+  uint32_t incl = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
   const uint32_t r = rank[j];
-  uint32_t cum = 0;
-  int digit = 255;
-  for (int d = 0; d < 256; ++d) {
-    if (cum + h[d] > r) {
-      digit = d;
-      break;
-    }
-    cum += h[d];
+  const unsigned hit = __ballot_sync(0xffffffffu, incl > r);  // not empty: the bins hold more than r
+  if (hit == 0 || lane != __ffs(hit) - 1) return;
+  uint32_t cum = incl - sum;
+  int digit = lane * 8;
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    if (cum + c[d] > r) break;
+    cum += c[d];
+    ++digit;
   }
   rank[j] = r - cum;
-  prefix[j] = shift == 24 ? (uint32_t)digit : ((prefix[j] << 8) | (uint32_t)digit);
-  for (int d = 0; d < 256; ++d) h[d] = 0;
-  if (shift == 0) tau[j] = key_float(prefix[j]);
+  const uint32_t p = shift == 24 ? (uint32_t)digit : ((prefix[j] << 8) | (uint32_t)digit);
+  prefix[j] = p;
+  if (shift == 0) tau[j] = key_float(p);
 }
 
 // ---------------------------------------------------------------------------
@@ -223,8 +239,19 @@ __global__ void codes_kernel(const float *__restrict__ L, int64_t N, int b,
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < N;
        r += (int64_t)gridDim.x * blockDim.x) {
     uint32_t u = 0;
-    for (int j = 0; j < b; ++j)
-      if (__ldg(L + (size_t)r * b + j) >= st[j]) u |= 1u << j;
+    if ((b & 3) == 0) {
+      const float4 *p = reinterpret_cast<const float4 *>(L + (size_t)r * b);
+#pragma unroll
+      for (int j = 0; j < kBMax; j += 4)
+        if (j < b) {
+          const float4 v = __ldg(p + j / 4);
+          u |= (v.x >= st[j] ? 1u << j : 0u) | (v.y >= st[j + 1] ? 2u << j : 0u) |
+               (v.z >= st[j + 2] ? 4u << j : 0u) | (v.w >= st[j + 3] ? 8u << j : 0u);
+        }
+    } else {
+      for (int j = 0; j < b; ++j)
+        if (__ldg(L + (size_t)r * b + j) >= st[j]) u |= 1u << j;
+    }
     codes[r] = u;
     ids[r] = (uint32_t)r;
   }
@@ -781,36 +808,35 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   const int64_t nb = (int64_t)1 << b;
   const float *L = bd->logits;
   Scratch sc;
-  // fixed-point scale from the largest |logit|; rejects NaN and infinities
+  // medians: 4 radix passes of 8 bits; the first also finds the largest
+  // |logit| for the fixed-point scale, which rejects NaN and infinities
   unsigned int *d_small = nullptr;
   NRB_TRY(sc.alloc(&d_small, 16));
   NRB_TRY(cudaMemsetAsync(d_small, 0, 64, s));
-  absmax_kernel<<<grid_for(N * b, 256, nsm), 256, 0, s>>>(L, N * b, d_small);
+  uint32_t *hist, *prefix, *rank;
+  NRB_TRY(sc.alloc(&hist, (size_t)b * 256));
+  NRB_TRY(sc.alloc(&prefix, kBMax));
+  NRB_TRY(sc.alloc(&rank, kBMax));
+  NRB_TRY(cudaMemsetAsync(hist, 0, (size_t)b * 256 * 4, s));
+  NRB_TRY(cudaMemsetAsync(prefix, 0, kBMax * 4, s));
+  const int hist_blocks = std::min(grid_for(N * b, 256, nsm), nsm * 8);
+  const size_t hist_bytes = (size_t)b * 256 * 4;
+  median_hist_kernel<true><<<hist_blocks, 256, hist_bytes, s>>>(L, N * b, b, 24, prefix, hist, d_small);
   NRB_TRY(cudaGetLastError());
   unsigned int amax = 0;
+  std::vector<uint32_t> r0(kBMax, (uint32_t)((N - 1) / 2));
+  NRB_TRY(cudaMemcpyAsync(rank, r0.data(), kBMax * 4, cudaMemcpyHostToDevice, s));
   NRB_TRY(cudaMemcpyAsync(&amax, d_small, 4, cudaMemcpyDeviceToHost, s));
   NRB_TRY(cudaStreamSynchronize(s));
   if (amax >= 0x7F800000u) return NR_ERR_INVALID_ARG;
   float am;
   memcpy(&am, &amax, 4);
   const int G = 30 - (am > 0.0f ? exponent_of((double)am) : 0);
-  // medians: 4 radix passes of 8 bits
-  uint32_t *hist, *prefix, *rank;
-  NRB_TRY(sc.alloc(&hist, (size_t)b * 256));
-  NRB_TRY(sc.alloc(&prefix, kBMax));
-  NRB_TRY(sc.alloc(&rank, kBMax));
-  NRB_TRY(cudaMemsetAsync(hist, 0, (size_t)b * 256 * 4, s));
-  {
-    std::vector<uint32_t> r0(kBMax, (uint32_t)((N - 1) / 2));
-    NRB_TRY(cudaMemcpyAsync(rank, r0.data(), kBMax * 4, cudaMemcpyHostToDevice, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-  }
-  NRB_TRY(cudaMemsetAsync(prefix, 0, kBMax * 4, s));
-  const int hist_blocks = grid_for(N, 256, nsm) < nsm * 4 ? grid_for(N, 256, nsm) : nsm * 4;
   for (int shift = 24; shift >= 0; shift -= 8) {
-    median_hist_kernel<<<hist_blocks, 256, (size_t)b * 256 * 4, s>>>(L, N, b, shift, prefix, hist);
+    if (shift < 24)
+      median_hist_kernel<false><<<hist_blocks, 256, hist_bytes, s>>>(L, N * b, b, shift, prefix, hist, d_small);
     NRB_TRY(cudaGetLastError());
-    median_pick_kernel<<<1, 32, 0, s>>>(hist, prefix, rank, b, shift, ix->tau);
+    median_pick_kernel<<<1, 32 * b, 0, s>>>(hist, prefix, rank, shift, ix->tau);
     NRB_TRY(cudaGetLastError());
   }
   // codes and the stable sort of ids by code
