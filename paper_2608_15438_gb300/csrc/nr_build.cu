@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256) median_hist_kernel(const float *__restric
     const uint32_t pre = FIRST ? 0u : prefix[col];
     uint32_t *h = sh + col * 256;
     auto add = [&](uint32_t x) {
-      const uint32_t key = (x & 0x80000000u) ? ~x : (x | 0x80000000u);  // float_key
+      const uint32_t key = float_key(__uint_as_float(x));
       if (FIRST) m = max(m, x & 0x7FFFFFFFu);
       if (FIRST || (key >> (shift + 8)) == pre) atomicAdd(&h[(key >> shift) & 255u], 1u);
     };
@@ -735,29 +735,42 @@ struct nr_builder {
 
 namespace {
 
-// device buffers of one finish call, released on every exit
+// Device buffers of one finish call, released on every exit. reserve() takes
+// one block for the buffers that follow (an allocation and its release cost
+// about 70 us of host time together, and a build has some thirty buffers).
 struct Scratch {
   std::vector<void *> ptrs;
-  ~Scratch() {
+  char *block = nullptr;
+  size_t left = 0;
+  ~Scratch() { drop(); }
+  void drop() {
     for (void *p : ptrs)
       if (p) cudaFree(p);
+    ptrs.clear();
+    left = 0;
+  }
+  static size_t up(size_t v) { return (v + 255) & ~(size_t)255; }
+  cudaError_t reserve(size_t bytes) {
+    void *v = nullptr;
+    const cudaError_t e = cudaMalloc(&v, bytes > 0 ? bytes : 16);
+    if (e != cudaSuccess) return e;
+    ptrs.push_back(v);
+    block = static_cast<char *>(v);
+    left = bytes;
+    return cudaSuccess;
   }
   template <class T>
   cudaError_t alloc(T **p, size_t count) {
     *p = nullptr;
-    void *v = nullptr;
-    const cudaError_t e = cudaMalloc(&v, count * sizeof(T) > 0 ? count * sizeof(T) : 16);
-    if (e != cudaSuccess) return e;
-    ptrs.push_back(v);
-    *p = static_cast<T *>(v);
+    const size_t n = up(count * sizeof(T) > 0 ? count * sizeof(T) : 16);
+    if (n > left) {
+      const cudaError_t e = reserve(n);
+      if (e != cudaSuccess) return e;
+    }
+    *p = reinterpret_cast<T *>(block);
+    block += n;
+    left -= n;
     return cudaSuccess;
-  }
-  void release(void *p) {
-    for (auto &q : ptrs)
-      if (q == p) {
-        cudaFree(q);
-        q = nullptr;
-      }
   }
 };
 
@@ -807,7 +820,29 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   const int nsm = ix->num_sms;
   const int64_t nb = (int64_t)1 << b;
   const float *L = bd->logits;
-  Scratch sc;
+  // buffers kept to the end, and those of the sort; the scans share one
+  // temporary (of the longest, over all codes)
+  Scratch sc, sort;
+  size_t scan_bytes = 0, sort_bytes = 0;
+  const uint32_t *cnull = nullptr;
+  uint32_t *wnull = nullptr;
+  NRB_TRY(cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, cnull, wnull, nb + 1, s));
+  NRB_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, cnull, wnull, cnull, wnull, N, 0, b, s));
+  const size_t U = 256;
+  NRB_TRY(sc.reserve((size_t)N * 4 + 4 * ((size_t)nb + 1) * 4 + scan_bytes + (size_t)b * 1024 + 16 * U));
+  void *scan_tmp;
+  NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&scan_tmp), scan_bytes));
+  auto scan = [&](const uint32_t *in, uint32_t *out, int64_t n) -> cudaError_t {
+    size_t tb = 0;
+    const cudaError_t e = cub::DeviceScan::ExclusiveSum(nullptr, tb, in, out, n, s);
+    if (e != cudaSuccess) return e;
+    void *tmp = scan_tmp;
+    if (tb > scan_bytes) {  // a shorter scan never needs more, but it is cub's to say
+      const cudaError_t e2 = sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb);
+      if (e2 != cudaSuccess) return e2;
+    }
+    return cub::DeviceScan::ExclusiveSum(tmp, tb, in, out, n, s);
+  };
   // medians: 4 radix passes of 8 bits; the first also finds the largest
   // |logit| for the fixed-point scale, which rejects NaN and infinities
   unsigned int *d_small = nullptr;
@@ -841,57 +876,36 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   }
   // codes and the stable sort of ids by code
   uint32_t *codes, *ids, *codes_s, *ids_s;
-  NRB_TRY(sc.alloc(&codes, N));
-  NRB_TRY(sc.alloc(&ids, N));
-  NRB_TRY(sc.alloc(&codes_s, N));
   NRB_TRY(sc.alloc(&ids_s, N));
+  NRB_TRY(sort.reserve((size_t)N * 12 + sort_bytes + 4 * U));
+  NRB_TRY(sort.alloc(&codes, N));
+  NRB_TRY(sort.alloc(&ids, N));
+  NRB_TRY(sort.alloc(&codes_s, N));
+  void *sort_tmp;
+  NRB_TRY(sort.alloc(reinterpret_cast<unsigned char **>(&sort_tmp), sort_bytes));
   codes_kernel<<<grid_for(N, 256, nsm), 256, 0, s>>>(L, N, b, ix->tau, codes, ids);
   NRB_TRY(cudaGetLastError());
-  {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, codes, codes_s, ids, ids_s, N, 0, b, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceRadixSort::SortPairs(tmp, tb, codes, codes_s, ids, ids_s, N, 0, b, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
-  sc.release(codes);
-  sc.release(ids);
+  NRB_TRY(cub::DeviceRadixSort::SortPairs(sort_tmp, sort_bytes, codes, codes_s, ids, ids_s, N, 0, b, s));
   // bucket sizes, row starts, the non-empty list
   uint32_t *cnt, *bstart, *flag, *pos;
   NRB_TRY(sc.alloc(&cnt, nb + 1));
   NRB_TRY(sc.alloc(&bstart, nb + 1));
+  NRB_TRY(sc.alloc(&flag, nb + 1));
+  NRB_TRY(sc.alloc(&pos, nb + 1));
   NRB_TRY(cudaMemsetAsync(cnt, 0, (size_t)(nb + 1) * 4, s));
   count_kernel<<<grid_for(N, 256, nsm), 256, 0, s>>>(codes_s, N, cnt);
   NRB_TRY(cudaGetLastError());
-  {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt, bstart, nb + 1, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, cnt, bstart, nb + 1, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
-  sc.release(codes_s);
-  NRB_TRY(sc.alloc(&flag, nb + 1));
-  NRB_TRY(sc.alloc(&pos, nb + 1));
+  NRB_TRY(scan(cnt, bstart, nb + 1));
   flag_kernel<<<grid_for(nb + 1, 256, nsm), 256, 0, s>>>(cnt, nb, flag);
   NRB_TRY(cudaGetLastError());
-  {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, flag, pos, nb + 1, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, flag, pos, nb + 1, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
+  NRB_TRY(scan(flag, pos, nb + 1));
   uint32_t ne32 = 0;
-  NRB_TRY(cudaMemcpy(&ne32, pos + nb, 4, cudaMemcpyDeviceToHost));
+  NRB_TRY(cudaMemcpyAsync(&ne32, pos + nb, 4, cudaMemcpyDeviceToHost, s));
+  NRB_TRY(cudaStreamSynchronize(s));
+  sort.drop();
   const int64_t ne = ne32;
   uint32_t *ne_code, *kcount, *kslot, *big_e, *big_n, *big_e_s, *big_n_s;
+  NRB_TRY(sc.reserve(5 * (((size_t)ne + 1) * 4 + U)));
   NRB_TRY(sc.alloc(&ne_code, ne + 1));
   NRB_TRY(sc.alloc(&kcount, ne + 1));
   NRB_TRY(sc.alloc(&kslot, ne + 1));
@@ -902,34 +916,12 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   bucket_list_kernel<<<grid_for(nb, 256, nsm), 256, 0, s>>>(cnt, pos, nb, ix->K_max, ix->t, ne_code,
                                                             kcount, big_e, big_n, d_small);
   NRB_TRY(cudaGetLastError());
-  {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, kcount, kslot, ne + 1, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, kcount, kslot, ne + 1, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
-  sc.release(flag);
+  NRB_TRY(scan(kcount, kslot, ne + 1));
   uint32_t nslots = 0, nbig2[2] = {0, 0};
-  NRB_TRY(cudaMemcpy(&nslots, kslot + ne, 4, cudaMemcpyDeviceToHost));
-  NRB_TRY(cudaMemcpy(nbig2, d_small, 8, cudaMemcpyDeviceToHost));
+  NRB_TRY(cudaMemcpyAsync(&nslots, kslot + ne, 4, cudaMemcpyDeviceToHost, s));
+  NRB_TRY(cudaMemcpyAsync(nbig2, d_small, 8, cudaMemcpyDeviceToHost, s));
+  NRB_TRY(cudaStreamSynchronize(s));
   const uint32_t nbig = nbig2[0], nhuge = nbig2[1];
-  // large buckets largest first (the order only balances the load)
-  NRB_TRY(sc.alloc(&big_e_s, (size_t)nbig + 1));
-  NRB_TRY(sc.alloc(&big_n_s, (size_t)nbig + 1));
-  if (nbig > 0) {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, big_n, big_n_s, big_e, big_e_s,
-                                                      (int64_t)nbig, 0, 32, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceRadixSort::SortPairsDescending(tmp, tb, big_n, big_n_s, big_e, big_e_s,
-                                                      (int64_t)nbig, 0, 32, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
   // k-means
   KmArgs a;
   a.L = L;
@@ -937,7 +929,6 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   a.bstart = bstart;
   a.ne_code = ne_code;
   a.kslot = kslot;
-  a.big_e = big_e_s;
   a.ne = ne;
   a.nbig = nbig;
   a.b = b;
@@ -953,12 +944,6 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   uint32_t *out_ids;
   NRB_TRY(cudaMalloc((void **)&out_ids, (size_t)N * 4));
   ix->ids = out_ids;  // owned by the index from here on
-  NRB_TRY(sc.alloc(&a.labels, N));
-  NRB_TRY(sc.alloc(&a.slot_cent, (size_t)nslots * b + 1));
-  NRB_TRY(sc.alloc(&a.slot_cnt, (size_t)nslots + 1));
-  NRB_TRY(sc.alloc(&a.ncl, ne + 1));
-  NRB_TRY(sc.alloc(&a.counter, 4));
-  NRB_TRY(cudaMemsetAsync(a.counter, 0, 16, s));
   a.out_ids = out_ids;
   const int wpb = 8;
   const size_t wsm = km_smem_bytes(ix->K_max, b, 1) * wpb;
@@ -980,10 +965,34 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   // seeding scratch: at most a bucket's rows and sample_per_cluster * K_max
   const int64_t sample = (int64_t)a.S * ix->K_max;
   const int64_t mcap_w = std::min(sample, kWarpRows), mcap_c = std::min(sample, kCtaRows);
+  const size_t n_w = (size_t)grid_w * wpb * mcap_w, n_c = (size_t)grid_c * mcap_c,
+               n_h = (size_t)grid_h * sample;
+  size_t big_bytes = 0;
+  if (nbig > 0)
+    NRB_TRY(cub::DeviceRadixSort::SortPairsDescending(nullptr, big_bytes, cnull, wnull, cnull, wnull,
+                                                      (int64_t)nbig, 0, 32, s));
+  NRB_TRY(sc.reserve((size_t)N + ((size_t)nslots * (b + 1) + 2) * 4 + ((size_t)ne + 1) * 4 +
+                     2 * ((size_t)nbig + 1) * 4 + big_bytes + (n_w + n_c + n_h) * 4 + 16 * U));
   float *dmin_w, *dmin_c, *dmin_h;
-  NRB_TRY(sc.alloc(&dmin_w, (size_t)grid_w * wpb * mcap_w));
-  NRB_TRY(sc.alloc(&dmin_c, (size_t)grid_c * mcap_c));
-  NRB_TRY(sc.alloc(&dmin_h, (size_t)grid_h * sample));
+  NRB_TRY(sc.alloc(&a.labels, N));
+  NRB_TRY(sc.alloc(&a.slot_cent, (size_t)nslots * b + 1));
+  NRB_TRY(sc.alloc(&a.slot_cnt, (size_t)nslots + 1));
+  NRB_TRY(sc.alloc(&a.ncl, ne + 1));
+  NRB_TRY(sc.alloc(&a.counter, 4));
+  NRB_TRY(sc.alloc(&dmin_w, n_w));
+  NRB_TRY(sc.alloc(&dmin_c, n_c));
+  NRB_TRY(sc.alloc(&dmin_h, n_h));
+  NRB_TRY(cudaMemsetAsync(a.counter, 0, 16, s));
+  // large buckets largest first (the order only balances the load)
+  NRB_TRY(sc.alloc(&big_e_s, (size_t)nbig + 1));
+  NRB_TRY(sc.alloc(&big_n_s, (size_t)nbig + 1));
+  if (nbig > 0) {
+    void *tmp;
+    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), big_bytes));
+    NRB_TRY(cub::DeviceRadixSort::SortPairsDescending(tmp, big_bytes, big_n, big_n_s, big_e, big_e_s,
+                                                      (int64_t)nbig, 0, 32, s));
+  }
+  a.big_e = big_e_s;
   // the three kinds side by side, each on its own stream: the largest buckets
   // are the longest chain and start first
   NRB_TRY(cudaStreamSynchronize(s));  // the lists and counters are written
@@ -1007,28 +1016,15 @@ nr_status finish_impl(nr_builder *bd, int64_t *info, cudaStream_t s) {
   NRB_TRY(cudaGetLastError());
   NRB_TRY(side.wait());
   NRB_TRY(cudaStreamSynchronize(s));
-  sc.release(dmin_w);
-  sc.release(dmin_c);
-  sc.release(dmin_h);
-  sc.release(a.labels);
-  sc.release(ids_s);
   // bucket -> cluster CSR level: exclusive sum of kept clusters over all codes
-  uint32_t *clc;
-  NRB_TRY(sc.alloc(&clc, nb + 1));
+  uint32_t *clc = flag;  // no longer needed
   NRB_TRY(cudaMemsetAsync(clc, 0, (size_t)(nb + 1) * 4, s));
   scatter_ncl_kernel<<<grid_for(ne, 256, nsm), 256, 0, s>>>(ne_code, a.ncl, ne, clc);
   NRB_TRY(cudaGetLastError());
-  {
-    size_t tb = 0;
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, clc, ix->bkt_off, nb + 1, s));
-    void *tmp;
-    NRB_TRY(sc.alloc(reinterpret_cast<unsigned char **>(&tmp), tb));
-    NRB_TRY(cub::DeviceScan::ExclusiveSum(tmp, tb, clc, ix->bkt_off, nb + 1, s));
-    NRB_TRY(cudaStreamSynchronize(s));
-    sc.release(tmp);
-  }
+  NRB_TRY(scan(clc, ix->bkt_off, nb + 1));
   uint32_t ncl_total = 0;
-  NRB_TRY(cudaMemcpy(&ncl_total, ix->bkt_off + nb, 4, cudaMemcpyDeviceToHost));
+  NRB_TRY(cudaMemcpyAsync(&ncl_total, ix->bkt_off + nb, 4, cudaMemcpyDeviceToHost, s));
+  NRB_TRY(cudaStreamSynchronize(s));
   ix->n_cl = ncl_total;
   if (ix->n_cl >= ((int64_t)1 << 31)) return NR_ERR_INVALID_ARG;  // cluster indices fill 31 bits of a sort key
   NRB_TRY(cudaMalloc((void **)&ix->cl_off, ((size_t)ix->n_cl + 1) * 4));
