@@ -1,0 +1,35 @@
+"""nr_index_locate with few ids (found through the filters) and many (searched
+directly): repeats, ids that are not stored, negative and 2^32-range ids."""
+import numpy as np
+import pytest
+
+from gpu_util import build_small, need_cuda
+from nrix_reader import read_nrix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 33, 7_499, 7_500, 40_000])
+def test_locate_matches_the_stored_order(tmp_path, n):
+    torch = need_cuda()
+    from paper_2608_15438_gb300 import neuroute as nr
+
+    path, _, _ = build_small(tmp_path, "tiny", n=30_000, bits=10, name="loc")
+    a = read_nrix(path)
+    rng = np.random.default_rng(n)
+    ids = rng.integers(0, 30_000, n)
+    odd = rng.random(n) < 0.2
+    ids[odd] = rng.choice(np.array([-1, -5, 30_000, 2**19, 2**19 + 3, 2**27 + 7, 2**32 - 1, 2**33 + 1]), odd.sum())
+    ix = nr.Index(path, 0)
+    got = ix.locate(torch.from_numpy(ids).cuda()).cpu().numpy()
+    ix.close()
+    pos = np.full(30_000, -1)
+    pos[a["ids"].astype(np.int64)] = np.arange(30_000)
+    ok = (ids >= 0) & (ids < 30_000)
+    p = pos[np.where(ok, ids, 0)]
+    c = np.searchsorted(a["cl_off"], p, side="right") - 1
+    u = np.searchsorted(a["bkt_off"], c, side="right") - 1
+    first, last = a["bkt_off"][u].astype(np.int64), a["bkt_off"][u + 1].astype(np.int64)
+    exp = np.stack([c, u, first, last - first], 1)
+    exp[~ok] = (-1, -1, -1, 0)
+    assert np.array_equal(got, exp)
