@@ -892,7 +892,8 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     }
     ev = tstart(3, sb);
     e = nr_launch_refine(ix, qp, n, k, P + C, (nr_seg *)(cw + l.seg), (int32_t *)(cw + l.nL),
-                         (uint32_t *)(cw + l.slen), d_ids + q0 * k, d_d + q0 * k, stats + q0 * NR_QSTATS,
+                         (uint32_t *)(cw + l.slen), (uint32_t *)(cw + l.codes), P, d_ids + q0 * k,
+                         d_d + q0 * k, stats + q0 * NR_QSTATS,
                          cw + l.refine, l.total - l.refine, sb);
     tend(ev, sb);
     if (pipe && e == cudaSuccess) e = cudaEventRecord(ps.ref[slot], sb);

@@ -162,8 +162,9 @@ cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t
 // scratch of a refine launch over nq queries: room to refine one query's
 // stream by several blocks at once, or (least) only whole streams a block
 size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least);
-// scratch: at least the least bytes; whole streams a block below the others
+// d_codes: the probe codes [nq x P], the base code first. scratch: at least the
+// least bytes; whole streams a block below the others
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
-                             int64_t *d_ids, float *d_dists, int64_t *d_stats, void *d_scratch,
-                             size_t scratch_bytes, cudaStream_t s);
+                             const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
+                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s);

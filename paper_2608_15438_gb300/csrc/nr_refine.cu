@@ -4,18 +4,21 @@
 // nrq::refine_span on the segments K3 wrote to global memory and commit the
 // spans of a query in stream order.
 //
-// Bound by HBM at large batches (10,000 queries of the 3e7-row uint8 index:
-// 8.48 ms for 63.8 GB of candidate rows, DRAM at 7.31 TB/s), by latency at
-// small ones: one block a query left a single query to one SM (one uint8 query
+// Bound by HBM at large batches, less what queries share in L2, and by latency
+// at small ones: one block a query left a single query to one SM (one uint8 query
 // of 31,000 candidates 523 us, four fp32 queries of 154 MB each 7.8 ms; cut
 // into spans 60 us and 0.12 ms).
 //
-// Launch shapes measured on GB300 (u8-10m / f32-10m operating points): the
-// scan is limited by how many rows are in flight per SM, so tiles are small
-// (128 uint8 rows, 32-64 fp32 rows), two stages deep, and registers are capped
-// for many CTAs per SM. Tiles held in registers (eight lanes a 128-byte row,
-// no shared memory) had fewer bytes in flight: 14.8 ms against 9.1 for that
-// batch.
+// Launch shapes measured on GB300: the scan is limited by the bytes in flight
+// per SM, so tiles are small (128 uint8 rows, 32-64 fp32 rows). uint8, D = 128:
+// 3 stages and 4 CTAs an SM hold 8 tiles in flight, 2 stages and 6 CTAs 6 (with
+// nearby codes side by side 7,780 and 8,318 us a batch of 10,000; 4 stages and
+// 3 CTAs 8,754, 6 and 2 11,815). fp32, D = 96: 2 stages of 64
+// rows and 4 CTAs of two warps (4,473 us a batch of 10,000; 32 rows and 9 CTAs
+// 4,805, 3 stages and 6 CTAs 4,905: fewer queries side by side share more,
+// but a row's chain is serial and needs the warps).
+// Tiles held in registers (eight lanes a 128-byte row, no shared memory) had
+// fewer bytes in flight: 14.8 ms for 9.1.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -40,6 +43,9 @@ struct PlanArgs {
   nrq::RefinePlan *plan;
   uint32_t *pre;        // [nq + 1] first item of the i-th query (not of whole streams)
   int32_t *perm;        // processing order of whole streams
+  const uint32_t *codes;    // [nq x P] probe codes, the base code first
+  int P, b;
+  int64_t last;         // whole streams kept for the end, longest first
 };
 
 // inclusive prefix of v over the block's threads; *all = the sum
@@ -63,18 +69,21 @@ __device__ __forceinline__ uint64_t plan_scan(uint64_t v, uint64_t *wsum, uint64
   return x + (w > 0 ? before : 0);
 }
 
-// One CTA: the rounds of a span and the items of every query. Whole streams
-// (items_cap = nq) go longest first: the queries are bucketed by stream length
-// (1024 buckets scaled to the longest) and listed in decreasing bucket order,
-// so the persistent CTAs finish together instead of waiting on a long query
-// picked up last. Order inside a bucket is arbitrary; it does not affect any
-// result. Streams cut into spans keep the batch's order: their items are
-// short. Bound by latency: 5 us for 1 to 1,000 queries (scans by shuffles; the
-// serial 1,024-bucket scan it replaces made that 8).
+// One CTA: the rounds of a span and the items of every query, bound by latency
+// (5 us for 1 to 1,000 queries).
+// Whole streams (items_cap = nq): the queries with the `last` shortest streams
+// go at the end, longest first (1024 buckets scaled to the longest stream), so
+// that the persistent CTAs finish together; the others go by the top bits of
+// their base code, since queries of nearby codes have many clusters in common
+// and those that run at the same time read them from L2. Against longest first
+// throughout: 10,000 queries of the 3e7-row uint8 index 9,016 -> 7,792 us, of
+// the 1e7-row fp32 one 5,130 -> 4,796 (tiles of 32 rows). Order inside a bucket is arbitrary; no
+// order affects any result. Streams cut into spans keep the batch's order:
+// their items are short.
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
   __shared__ uint64_t wsum[32];
-  __shared__ unsigned int hist[kOrderBins];
-  __shared__ unsigned int smax;
+  __shared__ unsigned int hist[kOrderBins], hcode[kOrderBins];
+  __shared__ unsigned int smax, cut;
   const int tid = threadIdx.x;
   const int64_t nq = a.nq;
   const bool whole = a.items_cap <= nq;
@@ -108,10 +117,30 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
     for (int64_t q = tid; q < nq; q += kPlanThreads) atomicAdd(&hist[bin(q)], 1u);
     __syncthreads();
     const unsigned int mine = hist[tid];
-    const uint64_t incl = plan_scan(mine, wsum, &all);
-    hist[tid] = (unsigned int)incl - mine;
+    const unsigned int at = (unsigned int)(plan_scan(mine, wsum, &all) - mine);
+    // the buckets before the shortest `last` queries' first: by base code
+    if (tid == 0) cut = 0;
     __syncthreads();
-    for (int64_t q = tid; q < nq; q += kPlanThreads) a.perm[atomicAdd(&hist[bin(q)], 1u)] = (int32_t)q;
+    if ((int64_t)at + mine <= nq - a.last) atomicMax(&cut, (unsigned int)tid + 1u);
+    hist[tid] = at;
+    __syncthreads();
+    const int nc = (int)cut;
+    const int shift = a.b > 10 ? a.b - 10 : 0;  // 1024 ranges of codes
+    hcode[tid] = 0;
+    __syncthreads();
+    if (nc > 0)
+      for (int64_t q = tid; q < nq; q += kPlanThreads)
+        if (bin(q) < nc) atomicAdd(&hcode[a.codes[q * a.P] >> shift & (kOrderBins - 1)], 1u);
+    __syncthreads();
+    const unsigned int mc = hcode[tid];
+    const unsigned int ac = (unsigned int)(plan_scan(mc, wsum, &all) - mc);
+    hcode[tid] = ac;
+    __syncthreads();
+    for (int64_t q = tid; q < nq; q += kPlanThreads) {
+      const int z = bin(q);
+      unsigned int *h = z < nc ? &hcode[a.codes[q * a.P] >> shift & (kOrderBins - 1)] : &hist[z];
+      a.perm[atomicAdd(h, 1u)] = (int32_t)q;
+    }
     all = (uint64_t)nq;
   } else {
     uint64_t items = 0;
@@ -179,16 +208,16 @@ __device__ __forceinline__ void item_of(const RefineArgs &a, uint32_t t, int &i,
 // sctl words of the kernel (1..3 are refine_span's)
 enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlCur, kCtlHn, kCtlRounds, kCtlLow, kCtlStop, kCtlNext, kCtlRedo };
 
-template <int DT, int TR, int CPR, int KCC, int MINB>
+template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31;
   const int k = a.rf.k;
-  const nrq::RefineSmem m = nrq::refine_carve<TR, KCC>(smem, a.row_bytes, k);
+  const nrq::RefineSmem m = nrq::refine_carve<TR, KCC, ST>(smem, a.row_bytes, k);
   volatile int *ctl = m.sctl;
   const uint32_t nitems = a.plan->nitems, span_rows = a.plan->span_rows;
   // spans a commit stages at once: what fits the stages (rows of 16 bytes at least)
-  constexpr int kFit = (int)(nrq::refine_stage_bytes<TR, KCC>(CPR > 0 ? CPR * 16 : 16) / (nrq::kStaged * 16));
+  constexpr int kFit = (int)(nrq::refine_stage_bytes<TR, KCC, ST>(CPR > 0 ? CPR * 16 : 16) / (nrq::kStaged * 16));
   constexpr int kStage = kFit < 32 ? kFit : 32;
   for (bool first = true;; first = false) {
     if (tid < 32) {  // the next item whose query has not stopped
@@ -237,7 +266,7 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
       lg.pool_used = &a.plan->pool_used;
       lg.pool = a.pool;
       lg.pool_cap = a.pool_cap;
-      nrq::refine_span<DT, TR, CPR, KCC>(a.rf, m, p0, p1, a.nL[q], a.seg + (size_t)q * a.Lmax, held, r, lg);
+      nrq::refine_span<DT, TR, CPR, KCC, ST>(a.rf, m, p0, p1, a.nL[q], a.seg + (size_t)q * a.Lmax, held, r, lg);
       const uint32_t base = (uint32_t)ctl[kCtlItem], spans = (uint32_t)ctl[kCtlSpans];
       uint32_t next = sp + 1;  // the next span to commit, when held
       bool redo = false;
@@ -351,22 +380,23 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
 // cutting their streams only adds work per span (about 7 us each: the item,
 // the segment search, the first tile's latency, the commit) and rows read
 // beyond an early stop. Measured (search us, cut / whole): u8-10m P 256, no
-// early stop, 912 blocks: 100 queries 237 / 379, 500 427 / 448, 700 521 / 503;
-// u8-30m P 1024 t_low 80: 300 537 / 657, 500 752 / 764, 700 975 / 910; f32-10m
-// t_low 16, 1,824 blocks: 500 620 / 944, 900 974 / 1022, 1400 1476 / 1177;
-// u8-10m P 64 t_low 4: 100 165 / 172, 500 261 / 196; 1536-value fp32 rows, 456
-// blocks: 30 1,109 / 11,860, 200 6,190 / 13,588. An early stop after few
-// rounds makes the later spans of a stream likely waste.
+// early stop, 608 blocks: 100 queries 240 / 343, 400 368 / 381, 600 485 / 432;
+// u8-30m P 1024 t_low 80: 300 546 / 593, 400 651 / 639; f32-10m, 1,368 blocks,
+// no early stop: 400 462 / 1,016, t_low 16: 400 462 / 569, 700 710 / 645;
+// u8-10m k 100 t_low 16: 100 471 / 507, 300 584 / 524; P 64 t_low 4: 1 query
+// 81 / 103, 100 167 / 163; 1536-value fp32 rows, 456 blocks: 30 1,075 / 7,909,
+// 440 13,058 / 16,062. An early stop after few rounds makes the later spans of
+// a stream likely waste.
 bool whole_streams(int64_t nq, int64_t grid, int t_low, bool long_rows) {
   if (long_rows) return nq >= grid;
-  const int64_t sixteenths = t_low == 0 || t_low >= 64 ? 9 : t_low >= 8 ? 6 : 2;
+  const int64_t sixteenths = t_low == 0 || t_low >= 64 ? 10 : t_low >= 8 ? 5 : 2;
   return nq * 16 >= grid * sixteenths;
 }
 
-template <int DT, int TR, int CPR, int KCC, int MINB>
+template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s) {
-  const size_t smem = nrq::refine_smem_bytes<TR, KCC>(a.row_bytes, a.rf.k);
-  auto kern = refine_kernel<DT, TR, CPR, KCC, MINB>;
+  const size_t smem = nrq::refine_smem_bytes<TR, KCC, ST>(a.row_bytes, a.rf.k);
+  auto kern = refine_kernel<DT, TR, CPR, KCC, ST, MINB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
@@ -376,14 +406,16 @@ cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t 
   if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
   int64_t grid = (int64_t)per_sm * ix->num_sms;
   pa.align = a.rf.R < TR ? TR / a.rf.R : 1;
-  // two uint8 items a block, four of the slower fp32 ones (u8-10m, 100 queries:
-  // 237 us at two, 244 at four; long fp32 rows, 30 queries: 1,203 and 1,109)
+  // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
+  // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
+  // 1,075)
   pa.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
   if (whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) pa.items_cap = (unsigned int)a.nq;
   a.group = (int)grid;
   if (pa.items_cap <= a.nq) {  // whole streams
     a.pre = nullptr;
     grid = std::min(grid, a.nq);
+    pa.last = std::min(grid, a.nq);
   }
   plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
   ix->launches += 1;
@@ -458,8 +490,8 @@ size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least) {
 
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
-                             int64_t *d_ids, float *d_dists, int64_t *d_stats, void *d_scratch,
-                             size_t scratch_bytes, cudaStream_t s) {
+                             const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
+                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s) {
   if (nq <= 0) return cudaSuccess;
   char *w = static_cast<char *>(d_scratch);
   const int64_t items = span_items(nq), entries = span_entries(nq, k);
@@ -489,6 +521,10 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   a.pool_cap = whole ? 0u : (uint32_t)entries;
   PlanArgs pa;
   pa.slen = d_slen;
+  pa.codes = d_codes;
+  pa.P = P;
+  pa.b = ix->b;
+  pa.last = nq;
   pa.nq = nq;
   pa.R = a.rf.R;
   pa.align = 1;
@@ -503,16 +539,16 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
     if (e != cudaSuccess) return e;
   }
   if (ix->dtype == 0) {
-    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 6>(ix, a, pa, s);  // uint8, D = 128
-    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 4>(ix, a, pa, s);
-    return launch_refine<0, 64, 0, 0, 4>(ix, a, pa, s);
+    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s);  // uint8, D = 128
+    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s);
+    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s);
   }
   if (ix->row_bytes > 1024) {  // fp32, D above 256: rows staged in pieces
-    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 3>(ix, a, pa, s);
-    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 3>(ix, a, pa, s);
-    return launch_refine<1, 128, 0, 4, 3>(ix, a, pa, s);  // row_bytes % 64 == 0 (load check)
+    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s);
+    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s);
+    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s);  // row_bytes % 64 == 0 (load check)
   }
-  if (a.rf.cpr == 24) return launch_refine<1, 32, 24, 0, 12>(ix, a, pa, s);  // fp32, D = 96
-  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 4>(ix, a, pa, s);
-  return launch_refine<1, 32, 0, 0, 4>(ix, a, pa, s);
+  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s);  // fp32, D = 96
+  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s);
+  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s);
 }

@@ -108,7 +108,8 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
                          (uint32_t *)(w + o_slen), stats, slab_q ? w + o_slab : nullptr, s);
   if (e == cudaSuccess)
     e = nr_launch_refine(ix, d_queries, nq, k, (int)Lmax, (nr_seg *)(w + o_seg),
-                         (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), d_out_ids, d_out_dists,
+                         (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), (uint32_t *)(w + o_codes), P,
+                         d_out_ids, d_out_dists,
                          stats, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine, s);
   // statistics of this call are read from the array by nr_last_stats / nr_query_stats
   ix->d_stats = stats;
