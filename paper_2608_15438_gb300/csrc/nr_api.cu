@@ -780,7 +780,7 @@ nr_status nr_debug_clusters(nr_index *ix, const float *d_logits, int64_t nq, int
   if (e == cudaSuccess)
     e = nr_launch_select(ix, d_logits, (uint32_t *)(w + l.codes), (int32_t *)(w + l.nprobe), nq,
                          P, C, d_clusters, d_ncl, (nr_seg *)(w + l.seg), (uint32_t *)(w + l.slen),
-                         nullptr, nr_select_slab_bytes(P, ix->K_max) ? w + l.slab : nullptr, s);
+                         nullptr, nr_select_slab_bytes(P, ix->K_max) ? w + l.slab : nullptr, {nullptr, 0}, s);
   return cuda_status(e);
 }
 
@@ -882,7 +882,8 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     e = nr_launch_select(ix, lg, (uint32_t *)(cw + l.codes), (int32_t *)(cw + l.nprobe), n, P, C,
                          (int32_t *)(cw + l.L), (int32_t *)(cw + l.nL), (nr_seg *)(cw + l.seg),
                          (uint32_t *)(cw + l.slen), stats + q0 * NR_QSTATS,
-                         nr_select_slab_bytes(P, ix->K_max) ? cw + l.slab : nullptr, sa);
+                         nr_select_slab_bytes(P, ix->K_max) ? cw + l.slab : nullptr,
+                         nr_refine_zero(n, k, cw + l.refine, l.total - l.refine), sa);
     tend(ev, sa);
     if (e != cudaSuccess) break;
     if (pipe) {

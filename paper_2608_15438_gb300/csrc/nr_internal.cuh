@@ -155,15 +155,25 @@ size_t nr_select_slab_bytes(int P, int K_max);
 // the global scratch of a select launch over nq queries: their slabs and the
 // list of the queries deferred to its overflow kernel (0: none needed)
 size_t nr_select_slab_total(int64_t nq, int P, int K_max);
+// n 16-byte words at p that a launch clears for a later one
+struct nr_zero {
+  void *p;
+  size_t n;
+};
+// zero: cleared beside the selection (see nr_refine_zero)
 cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t *d_codes,
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
-                             void *d_slab, cudaStream_t s);
+                             void *d_slab, nr_zero zero, cudaStream_t s);
+// the flags of a refine launch's scratch that have to be zero: the select
+// launch before it clears them
+nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes);
 // scratch of a refine launch over nq queries: room to refine one query's
 // stream by several blocks at once, or (least) only whole streams a block
 size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least);
 // d_codes: the probe codes [nq x P], the base code first. scratch: at least the
-// least bytes; whole streams a block below the others
+// least bytes, nr_refine_zero of it cleared; whole streams a block below the
+// others
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
                              const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,

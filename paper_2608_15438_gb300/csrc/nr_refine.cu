@@ -32,14 +32,19 @@ namespace {
 constexpr int kPlanThreads = 1024;
 constexpr int kOrderBins = 1024;
 
+// How streams are cut.
+struct SpanRule {
+  int R;
+  int align;                // rounds of a span: a multiple of this (whole tiles)
+  int rounds_most;          // its rounds when there are items enough
+  unsigned int items_want;  // items that keep every CTA busy
+  unsigned int items_cap;   // items there is room for (nq: whole streams only)
+};
+
 struct PlanArgs {
   const uint32_t *slen;
   int64_t nq;
-  int R;
-  int align;            // rounds of a span: a multiple of this (whole tiles)
-  int rounds_most;      // its rounds when there are items enough
-  unsigned int items_want;  // items that keep every CTA busy
-  unsigned int items_cap;   // items there is room for (nq: whole streams only)
+  SpanRule rule;
   nrq::RefinePlan *plan;
   uint32_t *pre;        // [nq + 1] first item of the i-th query (not of whole streams)
   int32_t *perm;        // processing order of whole streams
@@ -69,6 +74,22 @@ __device__ __forceinline__ uint64_t plan_scan(uint64_t v, uint64_t *wsum, uint64
   return x + (w > 0 ? before : 0);
 }
 
+// Rows of a span (0xffffffff: whole streams) when the streams have `all` rounds
+// in total: rounds that leave the items wanted and fit the room for them, whole
+// tiles.
+__device__ __forceinline__ uint32_t span_length(uint64_t all, int64_t nq, const SpanRule &r) {
+  uint64_t S = min((uint64_t)r.rounds_most, all / r.items_want);
+  const uint64_t room = r.items_cap - (uint64_t)nq;
+  S = max(S, (all + room - 1) / room);
+  S = max((S + r.align - 1) / r.align, (uint64_t)1) * r.align;
+  const uint64_t rows = S * (uint64_t)r.R;
+  return rows < 0xffffffffull ? (uint32_t)rows : 0xffffffffu;
+}
+// Items of a stream of n rows.
+__device__ __forceinline__ uint32_t spans_of(uint32_t n, uint32_t span) {
+  return max(1u, (uint32_t)(((uint64_t)n + span - 1) / span));
+}
+
 // One CTA: the rounds of a span and the items of every query, bound by latency
 // (5 us for 1 to 1,000 queries).
 // Whole streams (items_cap = nq): the queries with the `last` shortest streams
@@ -86,7 +107,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
   __shared__ unsigned int smax, cut;
   const int tid = threadIdx.x;
   const int64_t nq = a.nq;
-  const bool whole = a.items_cap <= nq;
+  const bool whole = a.rule.items_cap <= nq;
   const int64_t per = (nq + kPlanThreads - 1) / kPlanThreads;
   const int64_t lo = min(nq, tid * per), hi = min(nq, lo + per);
   uint64_t rounds = 0;
@@ -94,18 +115,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
   hist[tid] = 0;
   static_assert(kOrderBins == kPlanThreads, "a bucket per thread");
   if (!whole)
-    for (int64_t i = lo; i < hi; ++i) rounds += (a.slen[i] + (uint64_t)a.R - 1) / a.R;
+    for (int64_t i = lo; i < hi; ++i) rounds += (a.slen[i] + (uint64_t)a.rule.R - 1) / a.rule.R;
   uint64_t all;
   plan_scan(rounds, wsum, &all);  // starts with a barrier
-  uint64_t S = 0;                 // rounds of a span; 0: whole streams
-  if (!whole) {
-    S = min((uint64_t)a.rounds_most, all / a.items_want);
-    const uint64_t room = a.items_cap - (uint64_t)nq;
-    S = max(S, (all + room - 1) / room);
-    S = max((S + a.align - 1) / a.align, (uint64_t)1) * a.align;
-    if (S * (uint64_t)a.R >= 0xffffffffull) S = 0;
-  }
-  const uint32_t span = S ? (uint32_t)(S * (uint64_t)a.R) : 0xffffffffu;
+  const uint32_t span = whole ? 0xffffffffu : span_length(all, nq, a.rule);
   if (whole) {
     unsigned int m = 1;
     for (int64_t q = tid; q < nq; q += kPlanThreads) m = max(m, a.slen[q]);
@@ -144,12 +157,12 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
     all = (uint64_t)nq;
   } else {
     uint64_t items = 0;
-    for (int64_t i = lo; i < hi; ++i) items += max(1u, (uint32_t)(((uint64_t)a.slen[i] + span - 1) / span));
+    for (int64_t i = lo; i < hi; ++i) items += spans_of(a.slen[i], span);
     const uint64_t incl = plan_scan(items, wsum, &all);
     uint32_t at = (uint32_t)(incl - items);
     for (int64_t i = lo; i < hi; ++i) {
       a.pre[i] = at;
-      at += max(1u, (uint32_t)(((uint64_t)a.slen[i] + span - 1) / span));
+      at += spans_of(a.slen[i], span);
     }
     if (tid == 0) a.pre[nq] = (uint32_t)all;
   }
@@ -160,6 +173,10 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
     a.plan->pool_used = 0ull;
   }
 }
+
+// Batches up to this size need no plan kernel: a block's first warp works out
+// the spans while the others start (one uint8 query: 5 us less, and a launch).
+constexpr int kOwnPlan = 128;
 
 struct RefineArgs {
   nrq::RefineParams rf;
@@ -178,9 +195,11 @@ struct RefineArgs {
   int64_t *stats;
   nrq::RefinePlan *plan;
   const uint32_t *pre;       // null: whole streams, in the order of perm
+  bool own_plan;             // every block works the plan out itself (at most kOwnPlan queries)
+  SpanRule rule;
   const int32_t *perm;
   nrq::RefineQState *state;  // [nq]
-  uint32_t *ready;           // [items] 0: not finished, 1 + groups logged, or kSpanRedo
+  uint32_t *ready;           // [items] 0: not finished, 1: nothing logged, 2: logged, or kSpanRedo
   nrq::SpanHeader *hdr;      // [items]
   uint64_t *heap;            // [nq x k] committed top-k
   nrq::SpanEntry *pool;
@@ -189,11 +208,12 @@ struct RefineArgs {
 
 // The item of ticket t: its query i and its span, by a whole warp. Tickets go group by group: the first spans of the group's
 // queries, then the other spans query by query.
-__device__ __forceinline__ void item_of(const RefineArgs &a, uint32_t t, int &i, uint32_t &span) {
+template <class F>
+__device__ __forceinline__ void item_of(const RefineArgs &a, F pre, uint32_t t, int &i, uint32_t &span) {
   const int nq = (int)a.nq;
-  const int g0 = nrq::warp_last_le(0, nq, t, [&](int x) { return __ldg(&a.pre[x]); }) / a.group * a.group;
+  const int g0 = nrq::warp_last_le(0, nq, t, pre) / a.group * a.group;
   const int ng = min(a.group, nq - g0);
-  const uint32_t first = __ldg(&a.pre[g0]), o = t - first;
+  const uint32_t first = pre(g0), o = t - first;
   if (o < (uint32_t)ng) {
     i = g0 + (int)o;
     span = 0;
@@ -201,12 +221,15 @@ __device__ __forceinline__ void item_of(const RefineArgs &a, uint32_t t, int &i,
   }
   const uint32_t x = o - (uint32_t)ng;  // among the later spans of the group
   i = nrq::warp_last_le(g0, g0 + ng, x,
-                        [&](int y) { return __ldg(&a.pre[y]) - first - (uint32_t)(y - g0); });
-  span = 1u + x - (__ldg(&a.pre[i]) - first - (uint32_t)(i - g0));
+                        [&](int y) { return pre(y) - first - (uint32_t)(y - g0); });
+  span = 1u + x - (pre(i) - first - (uint32_t)(i - g0));
 }
 
+// Looks of about a microsecond each.
+constexpr int kPolls = 64;
+
 // sctl words of the kernel (1..3 are refine_span's)
-enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlCur, kCtlHn, kCtlRounds, kCtlLow, kCtlStop, kCtlNext, kCtlRedo };
+enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlRun, kCtlHn, kCtlRounds, kCtlLow, kCtlNext };
 
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
@@ -215,10 +238,47 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
   const int k = a.rf.k;
   const nrq::RefineSmem m = nrq::refine_carve<TR, KCC, ST>(smem, a.row_bytes, k);
   volatile int *ctl = m.sctl;
-  const uint32_t nitems = a.plan->nitems, span_rows = a.plan->span_rows;
-  // spans a commit stages at once: what fits the stages (rows of 16 bytes at least)
-  constexpr int kFit = (int)(nrq::refine_stage_bytes<TR, KCC, ST>(CPR > 0 ? CPR * 16 : 16) / (nrq::kStaged * 16));
-  constexpr int kStage = kFit < 32 ? kFit : 32;
+  uint32_t *spre = reinterpret_cast<uint32_t *>(m.sctl + 16);  // [kOwnPlan + 1], then the span's rows
+  if (a.own_plan && tid < 32) {
+    constexpr int per = kOwnPlan / 32;
+    uint32_t n[per], rounds = 0, items = 0;
+#pragma unroll
+    for (int e = 0; e < per; ++e) {
+      const int i = lane * per + e;
+      n[e] = i < a.nq ? a.slen[i] : 0u;
+      rounds += (uint32_t)(((uint64_t)n[e] + a.rule.R - 1) / a.rule.R);
+    }
+    uint64_t all = rounds;
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(nrq::kFull, all, o);
+    const uint32_t span = span_length(all, a.nq, a.rule);
+#pragma unroll
+    for (int e = 0; e < per; ++e)
+      if (lane * per + e < a.nq) items += spans_of(n[e], span);
+    uint32_t at = items;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(nrq::kFull, at, o);
+      if (lane >= o) at += v;
+    }
+    at -= items;
+#pragma unroll
+    for (int e = 0; e < per; ++e) {
+      spre[lane * per + e] = at;
+      if (lane * per + e < a.nq) at += spans_of(n[e], span);
+    }
+    if (lane == 31) spre[kOwnPlan] = at;  // (queries past the batch have no items)
+    if (lane == 0) spre[kOwnPlan + 1] = span;
+  }
+  if (a.own_plan) __syncthreads();
+  const uint32_t nitems = a.own_plan ? spre[kOwnPlan] : a.plan->nitems;
+  const uint32_t span_rows = a.own_plan ? spre[kOwnPlan + 1] : a.plan->span_rows;
+  auto pre = [&](int i) { return a.own_plan ? spre[i] : __ldg(&a.pre[i]); };
+  // spans a commit stages at once: what fits the stages beside its view (rows
+  // of 16 bytes at least)
+  constexpr int kRoom = (int)nrq::refine_stage_bytes<TR, KCC, ST>(CPR > 0 ? CPR * 16 : 16) - TR * 16 - 256;
+  constexpr int kFit = kRoom / (nrq::kStagedEntries * 16);
+  constexpr int kSlots = kFit < 0 ? 0 : kFit < 32 ? kFit : 32;
+  constexpr int kWarpFit = (int)nrq::refine_stage_bytes<TR, KCC, ST>(CPR > 0 ? CPR * 16 : 16) / 512;
+  constexpr int kWarpSlots = kWarpFit < 32 ? kWarpFit : 32;
   for (bool first = true;; first = false) {
     if (tid < 32) {  // the next item whose query has not stopped
       int q = -1;
@@ -234,11 +294,11 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
           break;
         }
         int i;
-        item_of(a, t, i, sp);
+        item_of(a, pre, t, i, sp);
         if (sp > 0 && __ldcg(&a.state[i].done)) continue;
         q = i;
-        base = __ldg(&a.pre[i]);
-        spans = __ldg(&a.pre[i + 1]) - base;
+        base = pre(i);
+        spans = pre(i + 1) - base;
         break;
       }
       if (lane == 0) {
@@ -271,12 +331,13 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
       uint32_t next = sp + 1;  // the next span to commit, when held
       bool redo = false;
       if (!held && tid < 32) {  // publish the log
+        nrq::log_flush(m, lg);
         __syncwarp();
         if (lane == 0) {
           a.hdr[base + sp].minkey = r.hn > 0 ? m.hkey[r.cur * k] : nrq::kEmpty;
-          a.hdr[base + sp].off = lg.off;
+          a.hdr[base + sp].off = (uint32_t)lg.first;
           __threadfence();
-          atomicExch(&a.ready[base + sp], lg.full ? nrq::kSpanRedo : lg.groups + 1u);
+          atomicExch(&a.ready[base + sp], lg.full ? nrq::kSpanRedo : lg.first != nrq::kEmpty ? 2u : 1u);
           __threadfence();
         }
       }
@@ -298,28 +359,38 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
           __syncthreads();
         }
         if (!r.stop && next < spans) {  // commit the finished spans that follow
-          if (tid < 32) {
-            // the stages are free between spans
-            redo = nrq::commit_ready(a.rf, m, r, a.pool, a.pool_cap, a.ready + base, a.hdr + base, next,
-                                     spans, n, span_rows, reinterpret_cast<uint4 *>(m.stage), kStage);
-            if (lane == 0) {
-              ctl[kCtlCur] = r.cur;
-              ctl[kCtlHn] = r.hn;
-              ctl[kCtlRounds] = r.rounds;
-              ctl[kCtlLow] = r.low;
-              ctl[kCtlStop] = r.stop ? 1 : 0;
-              ctl[kCtlNext] = (int)next;
-              ctl[kCtlRedo] = redo ? 1 : 0;
+          // With no item left for this block it waits a little for spans in
+          // flight (at most kPolls looks) instead of handing the top-k over to
+          // the block that finishes one.
+          const bool idle = __syncthreads_or(tid == 0 && gridDim.x + __ldcg(&a.plan->ticket) >= nitems);
+          // By the block, or for a small top-k by its first warp, whose turns
+          // are shorter (k = 100, 16 queries: 139 us a refinement by the
+          // block, 195 by a warp).
+          const int polls = idle ? kPolls : 0;
+          if (k <= 32) {
+            if (tid < 32) {
+              redo = nrq::commit_warp<kWarpSlots>(a.rf, m, r, a.pool, a.pool_cap, a.ready + base,
+                                                   a.hdr + base, next, spans, n, span_rows, polls);
+              if (lane == 0) {
+                ctl[kCtlRun] = r.cur | (r.stop ? 2 : 0) | (redo ? 4 : 0);
+                ctl[kCtlHn] = r.hn;
+                ctl[kCtlRounds] = r.rounds;
+                ctl[kCtlLow] = r.low;
+                ctl[kCtlNext] = (int)next;
+              }
             }
+            __syncthreads();
+            r.cur = ctl[kCtlRun] & 1;
+            r.stop = (ctl[kCtlRun] & 2) != 0;
+            redo = (ctl[kCtlRun] & 4) != 0;
+            r.hn = ctl[kCtlHn];
+            r.rounds = ctl[kCtlRounds];
+            r.low = ctl[kCtlLow];
+            next = (uint32_t)ctl[kCtlNext];
+          } else {
+            redo = nrq::commit_block<TR, kSlots>(a.rf, m, r, a.pool, a.pool_cap, a.ready + base,
+                                                 a.hdr + base, next, spans, n, span_rows, polls);
           }
-          __syncthreads();
-          r.cur = ctl[kCtlCur];
-          r.hn = ctl[kCtlHn];
-          r.rounds = ctl[kCtlRounds];
-          r.low = ctl[kCtlLow];
-          r.stop = ctl[kCtlStop] != 0;
-          next = (uint32_t)ctl[kCtlNext];
-          redo = ctl[kCtlRedo] != 0;
         }
         const uint64_t *H = m.hkey + r.cur * k;
         if (r.stop || next == spans) {  // the answer, sorted by (distance, id), padded
@@ -405,22 +476,26 @@ cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t 
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
   int64_t grid = (int64_t)per_sm * ix->num_sms;
-  pa.align = a.rf.R < TR ? TR / a.rf.R : 1;
+  pa.rule.align = a.rf.R < TR ? TR / a.rf.R : 1;
   // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
   // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
   // 1,075)
-  pa.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
-  if (whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) pa.items_cap = (unsigned int)a.nq;
+  pa.rule.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
+  if (whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) pa.rule.items_cap = (unsigned int)a.nq;
   a.group = (int)grid;
-  if (pa.items_cap <= a.nq) {  // whole streams
+  a.rule = pa.rule;
+  a.own_plan = pa.rule.items_cap > a.nq && a.nq <= kOwnPlan;
+  if (pa.rule.items_cap <= a.nq) {  // whole streams
     a.pre = nullptr;
     grid = std::min(grid, a.nq);
     pa.last = std::min(grid, a.nq);
   }
-  plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
-  ix->launches += 1;
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (!a.own_plan) {
+    plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
+    ix->launches += 1;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   kern<<<(unsigned)grid, TR, smem, s>>>(a);
   ix->launches += 1;
   return cudaGetLastError();
@@ -451,22 +526,22 @@ nrq::RefineParams refine_params(const nr_index *ix, int k) {
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // Scratch of a refine launch: [plan][order of whole streams], and where
-// streams may be cut into items spans: [item prefix][query states, ready flags
-// (zeroed together)][span headers][committed top-k][log entries]
+// streams may be cut into items spans: [item prefix][plan, query states, ready
+// flags (zeroed together)][span headers][committed top-k][log entries]
 struct RefineScratch {
   size_t plan, perm, pre, state, ready, zero_end, hdr, heap, pool, total;
 };
 RefineScratch refine_scratch(int64_t nq, int k, int64_t items, int64_t entries) {
   RefineScratch l = {};
   size_t o = 0;
-  l.plan = o; o = up256(o + sizeof(nrq::RefinePlan));
   l.perm = o; o = up256(o + (size_t)nq * 4);
+  l.plan = o; o = up256(o + sizeof(nrq::RefinePlan));
   if (items > nq) {
     l.pre = o;   o = up256(o + ((size_t)nq + 1) * 4);
+    l.plan = o;  o = up256(o + sizeof(nrq::RefinePlan));
     l.state = o; o += (size_t)nq * sizeof(nrq::RefineQState);
     l.ready = o; o += (size_t)items * 4;
-    l.zero_end = o;
-    o = up256(o);
+    l.zero_end = o = up256(o);
     l.hdr = o;   o = up256(o + (size_t)items * sizeof(nrq::SpanHeader));
     l.heap = o;  o = up256(o + (size_t)nq * k * 8);
     l.pool = o;  o = up256(o + (size_t)entries * sizeof(nrq::SpanEntry));
@@ -486,6 +561,12 @@ int64_t span_entries(int64_t nq, int k) {
 size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least) {
   return least ? refine_scratch(nq, k, nq, 0).total
                : refine_scratch(nq, k, span_items(nq), span_entries(nq, k)).total;
+}
+
+nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes) {
+  const RefineScratch l = refine_scratch(nq, k, span_items(nq), span_entries(nq, k));
+  if (nq <= 0 || l.total > scratch_bytes) return {nullptr, 0};  // whole streams
+  return {static_cast<char *>(scratch) + l.plan, (l.zero_end - l.plan) / 16};
 }
 
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
@@ -526,18 +607,10 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   pa.b = ix->b;
   pa.last = nq;
   pa.nq = nq;
-  pa.R = a.rf.R;
-  pa.align = 1;
-  pa.rounds_most = std::max(1, 8192 / a.rf.R);
-  pa.items_want = 1;
-  pa.items_cap = (unsigned int)(whole ? nq : items);
+  pa.rule = {a.rf.R, 1, std::max(1, 8192 / a.rf.R), 1u, (unsigned int)(whole ? nq : items)};
   pa.plan = a.plan;
   pa.pre = reinterpret_cast<uint32_t *>(w + l.pre);
   pa.perm = reinterpret_cast<int32_t *>(w + l.perm);
-  if (!whole) {
-    const cudaError_t e = cudaMemsetAsync(w + l.state, 0, l.zero_end - l.state, s);
-    if (e != cudaSuccess) return e;
-  }
   if (ix->dtype == 0) {
     if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s);  // uint8, D = 128
     if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s);

@@ -31,9 +31,14 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 6 : 1)
     select_kernel(nrq::SelectParams sp, const float *__restrict__ logits,
                   const uint32_t *__restrict__ codes, const int32_t *__restrict__ nprobe,
                   int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen, int64_t *stats,
-                  unsigned char *slab, size_t slab_bytes, unsigned *ovf) {
+                  unsigned char *slab, size_t slab_bytes, unsigned *ovf, nr_zero zero) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int q = blockIdx.x, tid = threadIdx.x;
+  // the block's share of the refinement's flags (in place of a memset between
+  // the kernels)
+  const size_t zper = (zero.n + gridDim.x - 1) / gridDim.x;
+  for (size_t i = q * zper + tid, e = min(zero.n, (q + 1) * zper); i < e; i += blockDim.x)
+    static_cast<uint4 *>(zero.p)[i] = make_uint4(0u, 0u, 0u, 0u);
   const int Lmax = sp.P + sp.C;
   unsigned char *scratch = smem;
   const size_t sbytes = MODE == 1 ? nrq::select_seq_bytes(sp.P, sp.C, sp.b_batch)
@@ -166,7 +171,7 @@ size_t nr_select_smem_bytes(const nr_index *ix, int P, int C) {
 cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t *d_codes,
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
-                             void *d_slab, cudaStream_t s) {
+                             void *d_slab, nr_zero zero, cudaStream_t s) {
   if (nq <= 0) return cudaSuccess;
   const size_t smem = nr_select_smem_bytes(ix, P, C);
   const nrq::SelectParams sp = nr_select_params(ix, P, C);  // before the launch configuration
@@ -184,13 +189,13 @@ cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t
     if (e != cudaSuccess) return e;
     select_kernel<1><<<(unsigned)nq, kThreads, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL,
                                                           d_seg, d_slen, d_stats, slab, slab_bytes,
-                                                          nullptr);
+                                                          nullptr, zero);
   } else {
     e = cudaFuncSetAttribute(select_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     select_kernel<0><<<(unsigned)nq, kThreads, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL,
                                                           d_seg, d_slen, d_stats, slab, slab_bytes,
-                                                          ovf);
+                                                          ovf, zero);
     ix->launches += 1;
     e = cudaGetLastError();
     if (e != cudaSuccess || !ovf) return e;

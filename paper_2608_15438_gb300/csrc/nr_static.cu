@@ -105,7 +105,8 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   if (e == cudaSuccess)
     e = nr_launch_select(ix, logits, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), nq, P, C,
                          (int32_t *)(w + o_L), (int32_t *)(w + o_nL), (nr_seg *)(w + o_seg),
-                         (uint32_t *)(w + o_slen), stats, slab_q ? w + o_slab : nullptr, s);
+                         (uint32_t *)(w + o_slen), stats, slab_q ? w + o_slab : nullptr,
+                         nr_refine_zero(nq, k, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine), s);
   if (e == cudaSuccess)
     e = nr_launch_refine(ix, d_queries, nq, k, (int)Lmax, (nr_seg *)(w + o_seg),
                          (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), (uint32_t *)(w + o_codes), P,

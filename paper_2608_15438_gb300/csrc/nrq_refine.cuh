@@ -81,15 +81,16 @@ struct RefineQState {
 };
 struct SpanHeader {  // of a logged span
   uint64_t minkey;   // its smallest key
-  uint32_t off, pad; // its first group of log entries
+  uint32_t off, pad; // its first block of log entries
 };
-// The log: per round in which members entered a span's local top-k, a group of
-// 1 + count entries: first (next group of the span, round within the span,
-// count), then (key, 0, 0) per member.
+// The log: the members that entered a span's local top-k in its rounds, in
+// round order, in blocks of 1 + count entries: first (next block of the span or
+// kEmpty, count), then (key, round within the span) per member.
 struct SpanEntry {
-  uint64_t key;  // of a group's first entry: the next group, kEmpty for none
-  uint32_t round, count;
+  uint64_t key;
+  uint32_t round, pad;
 };
+constexpr int kLogBlock = 128;  // members of a block at most
 constexpr uint32_t kSpanRedo = 0xffffffffu;  // ready value: not logged (the pool was full)
 
 // Rows that the stages hold as they are (see refine_span).
@@ -112,14 +113,17 @@ struct RefineSmem {
   uint32_t *srow;        // ST x TR: rows of the open tiles
   uint64_t *hkey;        // 2 x k
   uint64_t *skey;        // 2 x TR
+  uint64_t *logk;        // kLogBlock: members logged and not yet written, and
+  uint32_t *logr;        // their rounds
   int *htag;             // 2 x k
-  int *sctl;             // 16 ints: [1..3] survivor counters, [4..15] the kernel's
+  int *sctl;             // 16 ints: [1..3] survivor counters, [4..15] the kernel's; then its plan (132 ints)
 };
 
 template <int TR, int KCC, int ST>
 __host__ __device__ inline size_t refine_smem_bytes(int64_t row_bytes, int k) {
   return refine_stage_bytes<TR, KCC, ST>(row_bytes) + (size_t)row_bytes + (size_t)ST * TR * 4 +
-         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)2 * k * 4 + 16 * 4;
+         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)kLogBlock * 12 + (size_t)2 * k * 4 + 16 * 4 +
+         132 * 4;
 }
 
 // Carve RefineSmem from base (16-byte aligned).
@@ -131,7 +135,9 @@ __device__ __forceinline__ RefineSmem refine_carve(unsigned char *base, int64_t 
   m.srow = reinterpret_cast<uint32_t *>(m.sq + row_bytes);
   m.hkey = reinterpret_cast<uint64_t *>(m.srow + ST * TR);
   m.skey = m.hkey + 2 * k;
-  m.htag = reinterpret_cast<int *>(m.skey + 2 * TR);
+  m.logk = m.skey + 2 * TR;
+  m.logr = reinterpret_cast<uint32_t *>(m.logk + kLogBlock);
+  m.htag = reinterpret_cast<int *>(m.logr + kLogBlock);
   m.sctl = m.htag + 2 * k;
   return m;
 }
@@ -202,11 +208,72 @@ struct SpanLog {
   unsigned long long *pool_used;
   SpanEntry *pool;
   uint32_t pool_cap;
-  // out (warp 0): groups logged, the first and the last one, and whether the
-  // pool was full
-  uint32_t groups, off, last;
+  // out (warp 0): the first block written and the last, whether the pool was
+  // full, and the members waiting in shared memory
+  uint64_t first, last;
   bool full;
+  int waiting;
 };
+
+// Writes the members waiting in shared memory as a block of the span's log, by
+// warp 0.
+__device__ __forceinline__ void log_flush(const RefineSmem &m, SpanLog &lg) {
+  const int lane = threadIdx.x & 31, n = lg.waiting;
+  if (n == 0 || lg.full) return;
+  unsigned long long at = 0;
+  if (lane == 0) at = atomicAdd(lg.pool_used, (unsigned long long)n + 1ull);
+  at = __shfl_sync(kFull, at, 0);
+  lg.full = at + (unsigned)n + 1u > lg.pool_cap;
+  if (lg.full) return;
+  ulonglong2 *g = reinterpret_cast<ulonglong2 *>(lg.pool + at);
+  if (lane == 0) {
+    g[0] = make_ulonglong2(kEmpty, (unsigned long long)n);
+    if (lg.first != kEmpty) lg.pool[lg.last].key = at;
+  }
+  for (int e = lane; e < n; e += 32) g[1 + e] = make_ulonglong2(m.logk[e], (unsigned long long)m.logr[e]);
+  if (lg.first == kEmpty) lg.first = at;
+  lg.last = at;
+  lg.waiting = 0;
+  __syncwarp();
+}
+
+// Merges the ns keys of sk into the top-k, tagged with round `roundno`: merged
+// order by key; on equal keys (possible only when an index stores a row twice)
+// the members before the new ones, and those by slot, so ranks are unique.
+// Whole block; the keys are visible to it, and the result is on return.
+template <int TR>
+__device__ __forceinline__ void block_merge(const RefineSmem &m, SpanRun &r, int k, const uint64_t *sk_buf,
+                                            int ns, int roundno) {
+  const int tid = threadIdx.x;
+  const int nxt = r.cur ^ 1;
+  const uint64_t *H = m.hkey + r.cur * k;
+  for (int i = tid; i < ns; i += TR) {
+    const uint64_t sk = sk_buf[i];
+    int lo = 0, hi = r.hn;  // # of H at or below sk
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (H[mid] <= sk) lo = mid + 1; else hi = mid;
+    }
+    int rk = lo;
+    for (int j = 0; j < ns; ++j) rk += (sk_buf[j] < sk || (sk_buf[j] == sk && j < i)) ? 1 : 0;
+    if (rk < k) {
+      m.hkey[nxt * k + rk] = sk;
+      m.htag[nxt * k + rk] = roundno;
+    }
+  }
+  for (int j = tid; j < r.hn; j += TR) {
+    const uint64_t hk = H[j];
+    int rk = j;
+    for (int i = 0; i < ns; ++i) rk += sk_buf[i] < hk ? 1 : 0;
+    if (rk < k) {
+      m.hkey[nxt * k + rk] = hk;
+      m.htag[nxt * k + rk] = m.htag[r.cur * k + j];
+    }
+  }
+  __syncthreads();
+  r.cur = nxt;
+  r.hn = r.hn + ns < k ? r.hn + ns : k;
+}
 
 // Positions [p0, p1) of a query's stream of nl segments, p0 a whole number of
 // rounds and of tiles, p1 the stream's end or a whole number of rounds. The
@@ -268,8 +335,9 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
   int ci = 0;
   bool changed = false;  // the top-k in this round
   const uint32_t rmask_round = (uint32_t)a.R - 1u;  // R is a power of two
-  lg.groups = 0;
+  lg.first = kEmpty;
   lg.full = false;
+  lg.waiting = 0;
   // The committed threshold of the query, as the load of the previous tile
   // found it: a stale one only keeps more rows than it need, and waiting for
   // the load here would add an L2 latency to every tile.
@@ -299,36 +367,7 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
       const int ns = *cnt;
       const int roundno = r.rounds + 1;
       if (ns > 0) {
-        const int nxt = r.cur ^ 1;
-        const uint64_t *H = m.hkey + r.cur * k;
-        // merged order: by key; on equal keys (possible only when an index
-        // stores a row twice) H before S, and S by slot, so ranks are unique
-        for (int i = tid; i < ns; i += TR) {
-          const uint64_t sk = sk_buf[i];
-          int lo = 0, hi = r.hn;  // # of H at or below sk
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (H[mid] <= sk) lo = mid + 1; else hi = mid;
-          }
-          int rk = lo;
-          for (int j = 0; j < ns; ++j) rk += (sk_buf[j] < sk || (sk_buf[j] == sk && j < i)) ? 1 : 0;
-          if (rk < k) {
-            m.hkey[nxt * k + rk] = sk;
-            m.htag[nxt * k + rk] = roundno;
-          }
-        }
-        for (int j = tid; j < r.hn; j += TR) {
-          const uint64_t hk = H[j];
-          int rk = j;
-          for (int i = 0; i < ns; ++i) rk += sk_buf[i] < hk ? 1 : 0;
-          if (rk < k) {
-            m.hkey[nxt * k + rk] = hk;
-            m.htag[nxt * k + rk] = m.htag[r.cur * k + j];
-          }
-        }
-        __syncthreads();
-        r.cur = nxt;
-        r.hn = r.hn + ns < k ? r.hn + ns : k;
+        block_merge<TR>(m, r, k, sk_buf, ns, roundno);
         changed = true;
       }
       const uint32_t cend = p1 - cstart > (uint32_t)chunk ? cstart + chunk : p1;
@@ -340,30 +379,20 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
           round_done(a, r, roundno, newc, frontc);
         } else {
           r.rounds = roundno;
-          if (warp == 0 && newc > 0 && !lg.full) {  // log the members that entered
-            unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(lg.pool_used, (unsigned long long)newc + 1ull);
-            at = __shfl_sync(kFull, at, 0);
-            lg.full = at + (unsigned)newc + 1u > lg.pool_cap;
-            if (!lg.full) {
-              SpanEntry *g = lg.pool + at;
-              if (lane == 0) {
-                *reinterpret_cast<ulonglong2 *>(g) = make_ulonglong2(
-                    kEmpty, (unsigned long long)(roundno - 1) | ((unsigned long long)newc << 32));
-                if (lg.groups > 0) lg.pool[lg.last].key = at;
+          if (warp == 0 && newc > 0)  // log the members that entered
+            for (int i0 = 0; i0 < r.hn; i0 += 32) {
+              const bool nw = i0 + lane < r.hn && m.htag[r.cur * k + i0 + lane] == roundno;
+              const unsigned b = __ballot_sync(kFull, nw);
+              if (lg.waiting + __popc(b) > kLogBlock) log_flush(m, lg);
+              if (lg.full) break;
+              if (nw) {
+                const int e = lg.waiting + __popc(b & ((1u << lane) - 1u));
+                m.logk[e] = m.hkey[r.cur * k + i0 + lane];
+                m.logr[e] = (uint32_t)(roundno - 1);
               }
-              int e = 1;
-              for (int i0 = 0; i0 < r.hn; i0 += 32) {
-                const bool nw = i0 + lane < r.hn && m.htag[r.cur * k + i0 + lane] == roundno;
-                const unsigned b = __ballot_sync(kFull, nw);
-                if (nw) g[e + __popc(b & ((1u << lane) - 1u))].key = m.hkey[r.cur * k + i0 + lane];
-                e += __popc(b);
-              }
-              if (lg.groups == 0) lg.off = (uint32_t)at;
-              lg.last = (uint32_t)at;
-              ++lg.groups;
+              lg.waiting += __popc(b);
+              __syncwarp();
             }
-          }
         }
       }
     }
@@ -538,143 +567,289 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
   __syncthreads();
 }
 
-// Merges the keys of the lanes in `group` into the top-k, tagged with round
-// `roundno`, by one warp: the same merged order as refine_span's.
-__device__ __forceinline__ void warp_insert(const RefineSmem &m, SpanRun &r, int k, uint64_t key,
-                                            unsigned group, int roundno) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t *H = m.hkey + r.cur * k;
-  const bool in = ((group >> lane) & 1u) && (r.hn < k || key < H[k - 1]);
-  const unsigned sv = __ballot_sync(kFull, in);
-  if (!sv) return;
-  const int nxt = r.cur ^ 1;
-  int rk = 0;
-  if (in) {
-    int lo = 0, hi = r.hn;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (H[mid] <= key) lo = mid + 1; else hi = mid;
-    }
-    rk = lo;
-  }
-  for (unsigned b = sv; b; b &= b - 1) {
-    const int src = __ffs(b) - 1;
-    const uint64_t o = __shfl_sync(kFull, key, src);
-    rk += (o < key || (o == key && src < lane)) ? 1 : 0;
-  }
-  if (in && rk < k) {
-    m.hkey[nxt * k + rk] = key;
-    m.htag[nxt * k + rk] = roundno;
-  }
-  for (int j0 = 0; j0 < r.hn; j0 += 32) {
-    const int j = j0 + lane;
-    const uint64_t hk = j < r.hn ? H[j] : kEmpty;
-    int hr = j;
-    for (unsigned b = sv; b; b &= b - 1) {
-      const uint64_t o = __shfl_sync(kFull, key, __ffs(b) - 1);
-      hr += o < hk ? 1 : 0;
-    }
-    if (j < r.hn && hr < k) {
-      m.hkey[nxt * k + hr] = hk;
-      m.htag[nxt * k + hr] = m.htag[r.cur * k + j];
-    }
-  }
-  __syncwarp();
-  r.cur = nxt;
-  r.hn = min(k, r.hn + __popc(sv));
-}
+// The commit stages the first entries of the spans that can change the top-k in
+// the tiles' stages, which are free between spans.
+constexpr int kStagedEntries = 64;
 
-// Commits a logged span of nr rounds to the query's top-k, by one warp: its
-// first group of log entries starts at off of the pool, with its first kStaged
-// entries in shared memory.
-__device__ __forceinline__ void commit_span(const RefineParams &a, const RefineSmem &m, SpanRun &r,
-                                            const SpanEntry *pool, uint64_t off,
-                                            const uint4 *staged, int nr) {
-  const int lane = threadIdx.x & 31, k = a.k;
-  int done = 0;  // rounds of the span committed
-  uint4 v = staged[lane];
-  for (uint64_t at = off;;) {
-    const uint64_t key = ((uint64_t)v.y << 32) | v.x;
-    const uint64_t nextat = __shfl_sync(kFull, key, 0);
-    const int round = (int)__shfl_sync(kFull, v.z, 0), cnt = (int)__shfl_sync(kFull, v.w, 0);
-    rounds_unchanged(a, r, round - done);
-    if (r.stop) return;
-    const int roundno = r.rounds + 1;
-    warp_insert(m, r, k, key, __ballot_sync(kFull, lane >= 1 && lane <= cnt), roundno);
-    for (int e0 = 32; e0 <= cnt; e0 += 32) {
-      const int e = e0 + lane;
-      const uint64_t kk = e <= cnt ? __ldcg(&pool[at + e].key) : kEmpty;
-      warp_insert(m, r, k, kk, __ballot_sync(kFull, e <= cnt), roundno);
-    }
-    int newc, frontc;
-    count_new(m, r, k, a.nfront, roundno, newc, frontc);
-    round_done(a, r, roundno, newc, frontc);
-    if (r.stop) return;
-    done = round + 1;
-    if (nextat == kEmpty) break;
-    at = nextat;
-    // the next group's first entry, then its members
-    const uint4 h = __ldcg(reinterpret_cast<const uint4 *>(pool + at));
-    v = lane <= (int)h.w ? __ldcg(reinterpret_cast<const uint4 *>(pool + at + lane)) : h;
-  }
-  rounds_unchanged(a, r, nr - done);
-}
+struct CommitView {  // over the stages
+  uint64_t *min;     // [TR] smallest key of the batch's spans (kEmpty: nothing logged)
+  uint32_t *off;     // [TR] first block
+  uint32_t *slot;    // [TR] staged at, or 0xffffffff
+  uint32_t *want;    // [slots] the span of a slot
+  uint4 *entry;      // [slots][kStagedEntries]
+};
 
-// Commits the finished spans from `next` on, in order, to the query's top-k,
-// by one warp: until one is not finished, was not logged (returns true), or
-// the stop. Spans are looked at 32 at a time: those whose smallest key is
-// below the current k-th have their first group's entries staged in shared
-// memory together, so a batch costs two memory latencies and not one a span.
-__device__ __forceinline__ bool commit_ready(const RefineParams &a, const RefineSmem &m, SpanRun &r,
+// Commits the finished spans from `next` on, in stream order, to the query's
+// top-k: until one is not finished, was not logged (returns true), or the stop.
+// Whole block of TR threads. Spans are looked at TR at a time: those whose smallest key is
+// below the k-th have their first entries staged together, so a batch costs two
+// memory latencies and not one a span, and a round's members are merged by the
+// whole block. polls: how often to look again for one that is not finished.
+template <int TR, int SLOTS>
+__device__ __forceinline__ bool commit_block(const RefineParams &a, const RefineSmem &m, SpanRun &r,
                                              const SpanEntry *pool, uint32_t cap,
                                              const uint32_t *ready, const SpanHeader *hdr,
                                              uint32_t &next, uint32_t spans, uint32_t n,
-                                             uint32_t span_rows, uint4 *stage, int most) {
-  const int lane = threadIdx.x & 31, k = a.k;
+                                             uint32_t span_rows, int polls) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = a.k;
+  CommitView c;
+  c.min = reinterpret_cast<uint64_t *>(m.stage);
+  c.off = reinterpret_cast<uint32_t *>(c.min + TR);
+  c.slot = c.off + TR;
+  c.want = c.slot + TR;
+  c.entry = reinterpret_cast<uint4 *>(c.want + 64);
+  int *ctl = m.sctl + 1;  // [0] the first span not to commit, [1] wanted spans; then counters
+  const int rounds_span = (int)((span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+  const int rounds_last = (int)((n - (spans - 1u) * span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+  auto kth = [&]() { return r.hn == k ? m.hkey[r.cur * k + k - 1] : kEmpty; };
   while (next < spans) {
-    const uint32_t x = next + lane;
-    const uint32_t rdy = lane < most && x < spans ? ld_acquire(&ready[x]) : 0u;
+    const uint32_t x = next + tid;
+    const uint32_t rdy = x < spans ? ld_acquire(&ready[x]) : 0u;
+    if (tid == 0) {
+      ctl[0] = TR;
+      ctl[1] = 0;
+    }
     const bool logged = rdy > 1u && rdy != kSpanRedo;
-    uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);  // min key, first group
+    uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
+    if (logged) h = __ldcg(reinterpret_cast<const uint4 *>(hdr + x));
+    __syncthreads();
+    if (rdy == 0u || rdy == kSpanRedo) atomicMin(&ctl[0], tid);
+    c.min[tid] = ((uint64_t)h.y << 32) | h.x;
+    c.off[tid] = h.z;
+    c.slot[tid] = 0xffffffffu;
+    __syncthreads();
+    const int nb = ctl[0];  // finished spans of this batch
+    const bool redo = __syncthreads_or(tid == nb && rdy == kSpanRedo);
+    if (nb == 0 && polls > 0 && !redo) {
+      --polls;
+      continue;
+    }
+    {  // stage, the earliest first
+      const uint64_t top = kth();
+      for (int i0 = 0, at = 0; i0 < nb && at < SLOTS; i0 += 32) {
+        const unsigned b = __ballot_sync(kFull, i0 + lane < nb && c.min[min(i0 + lane, TR - 1)] < top);
+        if (warp == 0 && ((b >> lane) & 1u)) {
+          const int sl = at + __popc(b & ((1u << lane) - 1u));
+          if (sl < SLOTS) {
+            c.slot[i0 + lane] = sl;
+            c.want[sl] = i0 + lane;
+          }
+        }
+        at += __popc(b);
+        if (tid == 0) ctl[1] = min(at, SLOTS);
+      }
+      __syncthreads();
+      const int nw = ctl[1];
+      for (int e = tid; e < nw * kStagedEntries; e += TR) {
+        const uint32_t at = c.off[c.want[e / kStagedEntries]] + (uint32_t)(e % kStagedEntries);
+        if (at < cap) cp_async16((uint32_t)__cvta_generic_to_shared(c.entry + e), pool + at);
+      }
+      cp_async_commit();
+      cp_async_wait<0>();
+      if (tid == 0) ctl[0] = ctl[1] = ctl[2] = 0;  // survivor counters, as refine_span's
+      __syncthreads();
+    }
+    int at = 0, ci = 0;  // spans of the batch committed; merges (counters rotate)
+    while (at < nb && !r.stop) {
+      int j = nb;  // the next span that can change the top-k
+      const uint64_t top = kth();
+      for (int i0 = at & ~31; i0 < nb; i0 += 32) {
+        const int i = i0 + lane;
+        const unsigned b = __ballot_sync(kFull, i >= at && i < nb && c.min[min(i, TR - 1)] < top);
+        if (b) {
+          j = i0 + __ffs(b) - 1;
+          break;
+        }
+      }
+      const bool last = j == nb && next + nb == spans;  // the stream's last span may be short
+      rounds_unchanged(a, r, (j - at - (last ? 1 : 0)) * rounds_span + (last ? rounds_last : 0));
+      at = j;
+      if (r.stop || j == nb) break;
+      // span j: its members round by round
+      const uint32_t sl = c.slot[j];
+      int open = -1;  // the round being merged
+      auto close = [&]() {
+        int newc, frontc;
+        count_new(m, r, k, a.nfront, r.rounds + 1, newc, frontc);
+        round_done(a, r, r.rounds + 1, newc, frontc);
+      };
+      bool staged = sl != 0xffffffffu;
+      for (uint64_t blk = c.off[j]; blk != kEmpty && !r.stop;) {
+        const uint4 head = staged ? c.entry[sl * kStagedEntries] : __ldcg(reinterpret_cast<const uint4 *>(pool + blk));
+        const int cnt = (int)head.z;
+        for (int e0 = 0; e0 < cnt && !r.stop; e0 += TR) {
+          const int e = e0 + tid;
+          uint4 v = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0u);
+          if (e < cnt)
+            v = staged && e + 1 < kStagedEntries
+                    ? c.entry[sl * kStagedEntries + 1 + e]
+                    : __ldcg(reinterpret_cast<const uint4 *>(pool + blk + 1 + e));
+          const uint64_t key = ((uint64_t)v.y << 32) | v.x;
+          const int nch = min(TR, cnt - e0);
+          for (int i = 0; i < nch && !r.stop;) {
+            // the round of entry i, which opens if it is not open
+            int *cn = &ctl[ci % 3];
+            int *rd = reinterpret_cast<int *>(c.want);  // a word per turn
+            if (tid == i) rd[ci & 1] = (int)v.z;
+            if (tid == 0) ctl[(ci + 1) % 3] = 0;
+            __syncthreads();
+            const int round = rd[ci & 1];
+            if (round != open) {
+              if (open >= 0) close();
+              if (!r.stop) rounds_unchanged(a, r, round - open - 1);
+              if (r.stop) break;
+              open = round;
+            }
+            const bool in = tid >= i && tid < nch && (int)v.z == round;
+            uint64_t *sk = m.skey + (ci & 1) * TR;
+            if (in && key < kth()) sk[atomicAdd(cn, 1)] = key;
+            const int of = __syncthreads_count(in);
+            const int ns = *cn;
+            if (ns > 0) block_merge<TR>(m, r, k, sk, ns, r.rounds + 1);
+            i += of;
+            ++ci;
+          }
+        }
+        blk = ((uint64_t)head.y << 32) | head.x;
+        staged = false;
+      }
+      if (!r.stop) close();
+      if (!r.stop) rounds_unchanged(a, r, (next + j + 1 == spans ? rounds_last : rounds_span) - open - 1);
+      at = j + 1;
+    }
+    next += (uint32_t)at;
+    __syncthreads();  // the view is free
+    if (r.stop) return false;
+    if (redo) return true;
+    if (nb < TR && polls == 0) return false;  // the next one is not finished
+  }
+  return false;
+}
+
+// The same for k <= 32 by one warp, the top-k in its registers (a member a
+// lane): a member is merged by a vote and a shift. One query of 242 spans and
+// k = 10: 49 us a refinement with the top-k in shared memory, 53 by the block,
+// 41 so (37 queries 108, 110, 78).
+template <int SLOTS>
+__device__ __forceinline__ bool commit_warp(const RefineParams &a, const RefineSmem &m, SpanRun &r,
+                                            const SpanEntry *pool, uint32_t cap,
+                                            const uint32_t *ready, const SpanHeader *hdr,
+                                            uint32_t &next, uint32_t spans, uint32_t n,
+                                            uint32_t span_rows, int polls) {
+  constexpr int kEntries = 32;  // staged of a span: its block's first entry and 31 members
+  const int lane = threadIdx.x & 31, k = a.k;
+  uint4 *stage = reinterpret_cast<uint4 *>(m.stage);
+  uint64_t hk = lane < r.hn ? m.hkey[r.cur * k + lane] : kEmpty;  // kEmpty past the members
+  int ht = 0;                                                     // the round it entered
+  const int rounds_span = (int)((span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+  const int rounds_last = (int)((n - (spans - 1u) * span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
+  // kEmpty while there is room; by the whole warp (not behind a lane's condition)
+  auto kth = [&]() { return __shfl_sync(kFull, hk, k - 1); };
+  int open = -1;  // of the span being committed: the round being merged
+  auto close = [&]() {
+    const int roundno = r.rounds + 1;
+    const unsigned nw = __ballot_sync(kFull, lane < r.hn && ht == roundno);
+    round_done(a, r, roundno, __popc(nw), __popc(a.nfront < 32 ? nw & ((1u << a.nfront) - 1u) : nw));
+  };
+  // merges the members of the lanes in `left` (rounds in lane order)
+  auto take = [&](uint64_t key, int rd, unsigned left) {
+    while (left && !r.stop) {
+      const int round = __shfl_sync(kFull, rd, __ffs(left) - 1);
+      const unsigned group = __ballot_sync(kFull, rd == round) & left;
+      left &= ~group;
+      if (round != open) {
+        if (open >= 0) close();
+        if (!r.stop) rounds_unchanged(a, r, round - open - 1);
+        if (r.stop) return;
+        open = round;
+      }
+      const int roundno = r.rounds + 1;
+      const uint64_t top = kth();
+      unsigned g = __ballot_sync(kFull, key < top) & group;
+      for (; g; g &= g - 1) {
+        const uint64_t x = __shfl_sync(kFull, key, __ffs(g) - 1);
+        const int at = __popc(__ballot_sync(kFull, hk <= x && lane < r.hn));
+        const uint64_t uk = __shfl_up_sync(kFull, hk, 1);
+        const int ut = __shfl_up_sync(kFull, ht, 1);
+        if (lane >= at) {
+          hk = lane == at ? x : uk;
+          ht = lane == at ? roundno : ut;
+        }
+        r.hn = min(k, r.hn + 1);
+        if (lane >= k) hk = kEmpty;
+      }
+    }
+  };
+  bool redo = false;
+  while (next < spans && !r.stop) {
+    const uint32_t x = next + lane;
+    const uint32_t rdy = x < spans ? ld_acquire(&ready[x]) : 0u;
+    const bool logged = rdy > 1u && rdy != kSpanRedo;
+    uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);  // smallest key, first block
     if (logged) h = __ldcg(reinterpret_cast<const uint4 *>(hdr + x));
     const uint64_t mk = ((uint64_t)h.y << 32) | h.x;
     const unsigned idle = __ballot_sync(kFull, rdy == 0u || rdy == kSpanRedo);
     const int nb = idle ? __ffs(idle) - 1 : 32;  // finished spans of this batch
-    const bool redo = nb < 32 && __shfl_sync(kFull, rdy, nb) == kSpanRedo;
-    auto below = [&]() {  // spans that can change the top-k
-      const uint64_t kth = r.hn == k ? m.hkey[r.cur * k + k - 1] : kEmpty;
-      return __ballot_sync(kFull, lane < nb && logged && (r.hn < k || mk < kth));
-    };
-    const unsigned want = below();
-    for (unsigned b = want; b; b &= b - 1) {
-      const int j = __ffs(b) - 1;
-      const uint32_t at = __shfl_sync(kFull, h.z, j);
-      if (at + lane < cap)
-        cp_async16((uint32_t)__cvta_generic_to_shared(stage + j * kStaged + lane), pool + at + lane);
+    redo = nb < 32 && __shfl_sync(kFull, rdy, nb & 31) == kSpanRedo;
+    if (nb == 0 && polls > 0 && !redo) {
+      --polls;
+      continue;
+    }
+    const uint64_t top = kth();
+    const unsigned want = __ballot_sync(kFull, lane < nb && mk < top);  // can change the top-k
+    const int slot = __popc(want & ((1u << lane) - 1u));
+    int sl = 0;
+    for (unsigned b = want; b && sl < SLOTS; b &= b - 1, ++sl) {
+      const uint32_t at = __shfl_sync(kFull, h.z, __ffs(b) - 1) + (uint32_t)lane;
+      if (at < cap) cp_async16((uint32_t)__cvta_generic_to_shared(stage + sl * kEntries + lane), pool + at);
     }
     cp_async_commit();
     cp_async_wait<0>();
     __syncwarp();
-    const int rounds_span = (int)((span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
     int at = 0;  // spans of the batch committed
-    while (at < nb && !r.stop) {
-      const unsigned b = want & below() & (kFull << at);
+    while (at < nb) {
+      const uint64_t now = kth();
+      const unsigned b = want & __ballot_sync(kFull, mk < now) & (kFull << at);
       const int j = b ? __ffs(b) - 1 : nb;  // the next one that can change it
-      const bool last = next + nb == spans && j == nb;  // the stream's last span may be short
-      const int tail = (int)((n - (spans - 1u) * span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
-      if (j > at) rounds_unchanged(a, r, (j - at - (last ? 1 : 0)) * rounds_span + (last ? tail : 0));
+      const bool last = j == nb && next + nb == spans;  // the stream's last span may be short
+      rounds_unchanged(a, r, (j - at - (last ? 1 : 0)) * rounds_span + (last ? rounds_last : 0));
       at = j;
       if (r.stop || j == nb) break;
-      commit_span(a, m, r, pool, __shfl_sync(kFull, h.z, j), stage + j * kStaged,
-                  next + j + 1 == spans ? tail : rounds_span);
+      const int sj = __shfl_sync(kFull, slot, j);
+      bool staged = sj < SLOTS;
+      open = -1;
+      for (uint64_t blk = __shfl_sync(kFull, h.z, j); blk != kEmpty && !r.stop;) {
+        // lane 0: the block's first entry; the members after it
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (staged) v = stage[sj * kEntries + lane];
+        else if (blk + lane < cap) v = __ldcg(reinterpret_cast<const uint4 *>(pool + blk + lane));
+        const uint64_t key = ((uint64_t)v.y << 32) | v.x;
+        const uint64_t after = __shfl_sync(kFull, key, 0);
+        const int cnt = (int)__shfl_sync(kFull, v.z, 0);
+        take(key, (int)v.z, __ballot_sync(kFull, lane >= 1 && lane <= cnt));
+        for (int e0 = kEntries; e0 <= cnt && !r.stop; e0 += 32) {
+          const int e = e0 + lane;
+          if (e <= cnt) v = __ldcg(reinterpret_cast<const uint4 *>(pool + blk + e));
+          take(((uint64_t)v.y << 32) | v.x, (int)v.z, __ballot_sync(kFull, e <= cnt));
+        }
+        blk = after;
+        staged = false;
+      }
+      if (!r.stop) close();
+      if (!r.stop) rounds_unchanged(a, r, (next + j + 1 == spans ? rounds_last : rounds_span) - open - 1);
       at = j + 1;
+      if (r.stop) break;
     }
     next += (uint32_t)at;
-    if (r.stop) return false;
-    if (redo) return true;
-    if (nb < (most < 32 ? most : 32)) return false;  // the next one is not finished
+    __syncwarp();  // the stages are free
+    if (r.stop || redo || (nb < 32 && polls == 0)) break;
   }
-  return false;
+  if (lane < r.hn) {
+    m.hkey[r.cur * k + lane] = hk;
+    m.htag[r.cur * k + lane] = 0;
+  }
+  __syncwarp();
+  return redo && !r.stop;
 }
 
 }  // namespace nrq
