@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "nr_internal.cuh"
@@ -23,11 +24,32 @@
 
 namespace {
 
-constexpr int kThreads = 128;
+// Threads of a block: kThreads, and kFewThreads for the order-independent stage
+// of few queries, whose blocks have an SM to themselves and are bound by the
+// latency of their passes. The sequential stage is held to 168 registers, so
+// that a batch of 333 queries runs in one wave (229 registers and two blocks an
+// SM took 182 us a selection, three blocks 137).
+constexpr int kThreads = 128, kFewThreads = 512;
+static_assert(kFewThreads == nrq::kSelOvfThreads, "a block of few queries finishes deferred ones too");
+
+struct OverflowSmem {  // of select_overflow_block
+  uint64_t *keys;
+  uint32_t *hist;
+  int *warp_sums;
+  unsigned *ctl;  // 4, and the overflow kernel's item
+};
+__device__ __forceinline__ OverflowSmem overflow_carve(unsigned char *smem) {
+  OverflowSmem o;
+  o.keys = reinterpret_cast<uint64_t *>(smem);
+  o.hist = reinterpret_cast<uint32_t *>(smem + (size_t)nrq::select_smem_keys(nrq::kSelOvfKeys) * 8);
+  o.warp_sums = reinterpret_cast<int *>(o.hist + nrq::kSelOvfBuckets);
+  o.ctl = reinterpret_cast<unsigned *>(o.warp_sums + 32);
+  return o;
+}
 
 // MODE 0: the order-independent stage; MODE 1: the sequential stage
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, MODE == 0 ? 6 : 1)
+template <int MODE, int NT>
+__global__ void __launch_bounds__(NT, MODE == 1 ? 3 : NT == kThreads ? 6 : 1)
     select_kernel(nrq::SelectParams sp, const float *__restrict__ logits,
                   const uint32_t *__restrict__ codes, const int32_t *__restrict__ nprobe,
                   int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen, int64_t *stats,
@@ -42,7 +64,7 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 6 : 1)
   const int Lmax = sp.P + sp.C;
   unsigned char *scratch = smem;
   const size_t sbytes = MODE == 1 ? nrq::select_seq_bytes(sp.P, sp.C, sp.b_batch)
-                                   : nrq::select_scratch_bytes(sp.P, sp.K_max);
+                                   : nrq::select_scratch_bytes(sp.P, sp.K_max, NT);
   float *slog = reinterpret_cast<float *>(smem + sbytes);
   int *warp_sums = reinterpret_cast<int *>(slog + 32);
   unsigned *sred = reinterpret_cast<unsigned *>(warp_sums + 32);
@@ -52,7 +74,7 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 6 : 1)
   uint32_t total = 0;
   int scored = 0;
   unsigned char *qslab = slab ? slab + (size_t)q * slab_bytes : nullptr;
-  const int nl =
+  int nl =
       MODE == 1
           ? nrq::select_block_seq(sp, slog, codes + (size_t)q * sp.P, np, scratch, warp_sums, sred,
                                   seg + (size_t)q * Lmax, L ? L + (size_t)q * Lmax : nullptr, Lmax,
@@ -60,6 +82,15 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 6 : 1)
           : nrq::select_block(sp, slog, codes + (size_t)q * sp.P, np, scratch, qslab, warp_sums,
                               sred, seg + (size_t)q * Lmax, L ? L + (size_t)q * Lmax : nullptr,
                               Lmax, &total, &scored);
+  if (MODE == 0 && NT == kFewThreads && nl < 0) {
+    // a block this wide finishes the query itself (the selection's shared
+    // memory is free)
+    __syncthreads();
+    const OverflowSmem o = overflow_carve(smem);
+    nl = nrq::select_overflow_block(sp, qslab, scored, o.keys, o.hist, o.ctl, o.warp_sums,
+                                    seg + (size_t)q * Lmax, L ? L + (size_t)q * Lmax : nullptr, Lmax,
+                                    &total);
+  }
   if (tid == 0) {
     if (nl < 0) {  // deferred: the overflow kernel writes its list
       const unsigned i = atomicAdd(&ovf[0], 1u);
@@ -86,11 +117,8 @@ __global__ void __launch_bounds__(nrq::kSelOvfThreads, 2)
                            size_t slab_bytes, int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen,
                            int64_t *stats) {
   extern __shared__ __align__(16) unsigned char smem[];
-  uint64_t *skeys = reinterpret_cast<uint64_t *>(smem);
-  uint32_t *hist = reinterpret_cast<uint32_t *>(smem + (size_t)nrq::select_smem_keys(nrq::kSelOvfKeys) * 8);
-  int *warp_sums = reinterpret_cast<int *>(hist + nrq::kSelOvfBuckets);
-  unsigned *sctl = reinterpret_cast<unsigned *>(warp_sums + 32);
-  unsigned *item = sctl + 4;  // the query a block works on; sctl[0..3] are select_overflow_block's
+  const OverflowSmem o = overflow_carve(smem);
+  unsigned *item = o.ctl + 4;  // the query a block works on; ctl[0..3] are select_overflow_block's
   const int Lmax = sp.P + sp.C;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -102,8 +130,8 @@ __global__ void __launch_bounds__(nrq::kSelOvfThreads, 2)
     if (i == 0xffffffffu) break;
     const int q = (int)ovf[4 + 2 * (size_t)i], M = (int)ovf[4 + 2 * (size_t)i + 1];
     uint32_t total = 0;
-    const int nl = nrq::select_overflow_block(sp, slab + (size_t)q * slab_bytes, M, skeys, hist, sctl,
-                                              warp_sums, seg + (size_t)q * Lmax,
+    const int nl = nrq::select_overflow_block(sp, slab + (size_t)q * slab_bytes, M, o.keys, o.hist, o.ctl,
+                                              o.warp_sums, seg + (size_t)q * Lmax,
                                               L ? L + (size_t)q * Lmax : nullptr, Lmax, &total);
     if (threadIdx.x == 0) {
       nL[q] = nl;
@@ -161,41 +189,44 @@ size_t nr_select_slab_total(int64_t nq, int P, int K_max) {
   return (((size_t)nq * per + 255) & ~(size_t)255) + 16 + (size_t)nq * 8;
 }
 
-size_t nr_select_smem_bytes(const nr_index *ix, int P, int C) {
+static size_t select_smem(const nr_index *ix, int P, int C, int nt) {
   const nr_params &p = ix->params;
   const size_t s = p.cent_mode == 1 ? nrq::select_seq_bytes(P, C, p.b_batch)
-                                    : nrq::select_scratch_bytes(P, ix->K_max);
+                                    : nrq::select_scratch_bytes(P, ix->K_max, nt);
   return s + 32 * 4 + 32 * 4 + 16;
 }
+
+size_t nr_select_smem_bytes(const nr_index *ix, int P, int C) { return select_smem(ix, P, C, kThreads); }
 
 cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t *d_codes,
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
                              void *d_slab, nr_zero zero, cudaStream_t s) {
   if (nq <= 0) return cudaSuccess;
-  const size_t smem = nr_select_smem_bytes(ix, P, C);
   const nrq::SelectParams sp = nr_select_params(ix, P, C);  // before the launch configuration
   const size_t slab_bytes = nrq::select_slab_bytes(P, ix->K_max);
   unsigned char *slab = static_cast<unsigned char *>(d_slab);
+  // Wide blocks while each has an SM to itself (or, with much to do, half):
+  // select us narrow / wide: 1 query P 64 16.3 / 16.3, P 1024 44.0 / 24.5; 100
+  // queries P 256 38.8 / 22.5, P 1024 77.3 / 36.8; 200, P 1024 85.3 / 61.3; but
+  // 300, P 64 22.4 / 32.7 and 600, P 256 34.8 / 61.3.
+  const bool few = sp.mode == 0 && (nq <= ix->num_sms || (nq <= 2 * ix->num_sms && P >= 1024));
   unsigned *ovf = nullptr;  // the deferred-query list after the slabs
   cudaError_t e;
-  if (slab && slab_bytes && sp.mode == 0) {
+  if (slab && slab_bytes && sp.mode == 0 && !few) {
     ovf = reinterpret_cast<unsigned *>(slab + (((size_t)nq * slab_bytes + 255) & ~(size_t)255));
     e = cudaMemsetAsync(ovf, 0, 16, s);
     if (e != cudaSuccess) return e;
   }
-  if (sp.mode == 1) {
-    e = cudaFuncSetAttribute(select_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    select_kernel<1><<<(unsigned)nq, kThreads, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL,
-                                                          d_seg, d_slen, d_stats, slab, slab_bytes,
-                                                          nullptr, zero);
-  } else {
-    e = cudaFuncSetAttribute(select_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    select_kernel<0><<<(unsigned)nq, kThreads, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL,
-                                                          d_seg, d_slen, d_stats, slab, slab_bytes,
-                                                          ovf, zero);
+  const int nt = few ? kFewThreads : kThreads;
+  size_t smem = select_smem(ix, P, C, nt);
+  if (few && slab_bytes) smem = std::max(smem, nrq::select_overflow_smem_bytes());
+  auto kern = sp.mode == 1 ? select_kernel<1, kThreads> : few ? select_kernel<0, kFewThreads> : select_kernel<0, kThreads>;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)nq, nt, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL, d_seg, d_slen, d_stats,
+                                      slab, slab_bytes, ovf, zero);
+  if (sp.mode == 0) {
     ix->launches += 1;
     e = cudaGetLastError();
     if (e != cudaSuccess || !ovf) return e;

@@ -50,23 +50,22 @@ __host__ __device__ inline int select_sort_cap(int P, int K_max) {
   while (s < P * K_max) s <<= 1;
   return s;
 }
-// at least one key per thread of the 128-thread select block (the merge
-// sort's shortest padded length), at most kSelectSmemKeys
-constexpr int kSelectMinKeys = 128;
-__host__ __device__ inline int select_smem_cap(int P, int K_max) {
+// at least one key per thread of the block (nt threads: the merge sort's
+// shortest padded length), at most kSelectSmemKeys
+__host__ __device__ inline int select_smem_cap(int P, int K_max, int nt) {
   const int s = select_sort_cap(P, K_max);
-  return s < kSelectMinKeys ? kSelectMinKeys : (s < kSelectSmemKeys ? s : kSelectSmemKeys);
+  return s < nt ? nt : (s < kSelectSmemKeys ? s : kSelectSmemKeys);
 }
 // key capacity of the shared-memory scratch: S keys plus the merge sort's gaps
 __host__ __device__ inline int select_smem_keys(int S) { return S + S / 16; }
-__host__ __device__ inline size_t select_scratch_bytes(int P, int K_max) {
-  const int S = select_smem_cap(P, K_max);
+__host__ __device__ inline size_t select_scratch_bytes(int P, int K_max, int nt) {
+  const int S = select_smem_cap(P, K_max, nt);
   const int ib = S > 2 * P + 1 ? S : 2 * P + 1;
   return (size_t)select_smem_keys(S) * 8 + (size_t)ib * 4;
 }
 __host__ __device__ inline size_t select_slab_bytes(int P, int K_max) {
   const int full = select_sort_cap(P, K_max);
-  return full > select_smem_cap(P, K_max) ? (size_t)full * 12 : 0;
+  return full > kSelectSmemKeys ? (size_t)full * 12 : 0;
 }
 
 // Centroid distance d_c = sum_j (l_j - mu_cj)^2 as a sequential fmaf chain.
@@ -214,7 +213,7 @@ __device__ __forceinline__ int select_tail_smem(const SelectParams &sp, uint64_t
 // position) for i < nl, and L[i] (cluster index, -1 padded to Lmax) when L is
 // not null; *n_scored = the number of centroid distances evaluated (every
 // cluster of every probed bucket). slog: the query's b logits in shared memory; scratch:
-// select_scratch_bytes(P, K_max) bytes of shared memory; slab: this query's
+// select_scratch_bytes(P, K_max, nt) bytes of shared memory; slab: this query's
 // select_slab_bytes(P, K_max) bytes of global memory (null when that is 0);
 // warp_sums: 32 ints; sred: 2 unsigned. Returns nl (*total = stream length),
 // or -1 when the query is deferred to the overflow kernel. Whole block calls.
@@ -233,7 +232,7 @@ __device__ __forceinline__ int select_block(const SelectParams &sp, const float 
                                             nr_seg *seg, int32_t *L, int Lmax, uint32_t *total,
                                             int *n_scored) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int S_smem = select_smem_cap(sp.P, sp.K_max);
+  const int S_smem = select_smem_cap(sp.P, sp.K_max, nt);
   const int S_full = select_sort_cap(sp.P, sp.K_max);
   uint64_t *keys = reinterpret_cast<uint64_t *>(scratch);
   int *ibuf = reinterpret_cast<int *>(scratch + (size_t)select_smem_keys(S_smem) * 8);
