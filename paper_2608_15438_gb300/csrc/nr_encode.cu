@@ -907,6 +907,10 @@ __global__ void __launch_bounds__(kLyThreads, 1)
                                           *reinterpret_cast<const uint32_t *>(&h3));
             }
           }
+          // the reads above come before the tensor copy that refills the stage:
+          // its writes are the async proxy's, which the arrival alone does not
+          // order after them (rows of a slice then held a later slice's values)
+          fence_async_smem();
           mbar_arrive(smem_u32(&B.rawempty[rs]));
         } else {
 #pragma unroll
