@@ -613,7 +613,10 @@ constexpr int kLyKs = 64;        // K elements a slice
 constexpr int kLyStages = 3;
 // slices g and g + kLyPeriod use the same stage and the same producer group
 constexpr int kLyPeriod = kLyStages % 2 == 0 ? kLyStages : 2 * kLyStages;
-constexpr int kLyRawMax = 4;     // raw fp32 stages (first layer), at most
+// Raw fp32 stages (first layer): 2 or 4, so that one producer group reads all
+// slices of a stage. With an odd number a group could find the stage's other
+// slice still on its way and take the phase before it, of the same parity.
+constexpr int kLyRawMax = 4;
 constexpr uint32_t kLyRawStage = (uint32_t)kRows * kLyKs * 4u;  // 32 KB: two 16 KB boxes
 constexpr int kLyEpiWarps = 4, kLyProdWarps = 4;  // a producer group
 constexpr int kLyWarpEpi = 1, kLyWarpProd = kLyWarpEpi + kLyEpiWarps;
@@ -1153,13 +1156,13 @@ static cudaError_t launch_layer(nr_index *ix, const void *x, int K, int N, int l
                                 const float *bias, int64_t n, void *y, int64_t wait_ns,
                                 cudaStream_t s) {
   const int nt = ix->ly_nt[l], Np = (N + 15) / 16 * 16;
-  // fp32 first layer: raw stages for the tensor copies, as many as fit (<= 4)
+  // fp32 first layer: four raw stages for the tensor copies, or two
   int nraw = 0;
   CUtensorMap tm;
   memset(&tm, 0, sizeof(tm));
   if (XT == 1) {
     nraw = kLyRawMax;
-    while (nraw > 1 && ly_smem_bytes(nt, nraw) > (uint32_t)ix->smem_optin) --nraw;
+    while (nraw > 2 && ly_smem_bytes(nt, nraw) > (uint32_t)ix->smem_optin) nraw -= 2;
     if (ly_smem_bytes(nt, nraw) > (uint32_t)ix->smem_optin) return cudaErrorInvalidConfiguration;
     // x [n rows x K] fp32: boxes of 32 values x 128 rows, 128-byte swizzle
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)n};
