@@ -118,8 +118,27 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tc_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+// Waits for the warp's TMEM loads. Their registers hold the values only after
+// it, so those are operands: a use (or a register move at a branch's end, which
+// once read lanes 16-31 of a 16-column load too early) stays behind the wait.
+__device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                 "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                 "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]),
+                 "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),
+                 "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
 }
 
 // shared-memory matrix descriptor: start, leading (K) and stride (8-row group)
@@ -131,6 +150,18 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 // instruction descriptor, kind::f16: D fp32, A and B fp16, both K-major
 __host__ __device__ constexpr uint32_t mma_idesc(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
+               : "memory");
+}
+// bulk copy global -> this CTA's shared memory, completing on `bar` by bytes
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar)
+      : "memory");
 }
 
 // ------------------------------------------------------------ tensor-core kernel
@@ -151,6 +182,7 @@ struct TcBars {
   uint64_t a1full[2], a1empty[2];  // layer-1 accumulators: MMA -> epilogue -> MMA
   uint64_t hfull[2], hempty[2];    // hidden chunks in TMEM: epilogue -> MMA -> epilogue
   uint64_t a2full[2], a2empty[2];  // layer-2 accumulators
+  uint64_t wfull[2];               // the weights: W1's first chunk; the rest and W2
   uint64_t drain;                  // every MMA of the CTA complete
   uint32_t tmem_slot;
   int abort;                       // a wait expired: every role stops
@@ -401,18 +433,25 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       mbar_init(smem_u32(&B.a2full[i]), 1);
       mbar_init(smem_u32(&B.a2empty[i]), kEpiThreads);
     }
+    mbar_init(smem_u32(&B.wfull[0]), 1);
+    mbar_init(smem_u32(&B.wfull[1]), 1);
     mbar_init(smem_u32(&B.drain), 1);
     B.abort = 0;
     fence_mbar_init();
+    fence_async_smem();
+    // resident operands: W1 and W2 (already in operand order) by bulk copies,
+    // W1's first chunk on a barrier of its own so that layer 1 starts with it
+    // (a one-row launch: 10.3 us; with loads through registers, 14.1)
+    const uint32_t rest1 = (uint32_t)(nc - 1) * w1_bytes, all2 = (uint32_t)nc * w2_bytes;
+    const char *w1 = reinterpret_cast<const char *>(W1p);
+    mbar_arrive_tx(smem_u32(&B.wfull[0]), w1_bytes);
+    bulk_g2s(sbase + L.w1, w1, w1_bytes, smem_u32(&B.wfull[0]));
+    mbar_arrive_tx(smem_u32(&B.wfull[1]), rest1 + all2);
+    for (int c = 1; c < nc; ++c)
+      bulk_g2s(sbase + L.w1 + (uint32_t)c * w1_bytes, w1 + (size_t)c * w1_bytes, w1_bytes, smem_u32(&B.wfull[1]));
+    bulk_g2s(sbase + L.w2, W2p, all2, smem_u32(&B.wfull[1]));
   }
-  // resident operands: W1 and W2 (already in operand order) and the biases
-  {
-    const uint4 *w1 = reinterpret_cast<const uint4 *>(W1p), *w2 = reinterpret_cast<const uint4 *>(W2p);
-    uint4 *d1 = reinterpret_cast<uint4 *>(smem + L.w1), *d2 = reinterpret_cast<uint4 *>(smem + L.w2);
-    const int n1 = H * D / 8, n2v = n2 * H / 8;
-    for (int i = tid; i < n1; i += kTcThreads) d1[i] = __ldg(w1 + i);
-    for (int i = tid; i < n2v; i += kTcThreads) d2[i] = __ldg(w2 + i);
-  }
+  // the biases
   for (int i = tid; i < H; i += kTcThreads) sb1[i] = b1[i];
   if (tid < 32) sb2[tid] = tid < b ? b2[tid] : 0.0f;
   fence_async_smem();
@@ -430,6 +469,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       auto layer2 = [&](uint32_t gp, uint32_t ip, int cp) -> bool {
         const int hb = (int)(gp & 1);
         if (!wait_or_abort(smem_u32(&B.hfull[hb]), (gp >> 1) & 1u, abort, wait_ns)) return false;
+        if (gp == 0 && !wait_or_abort(smem_u32(&B.wfull[1]), 0, abort, wait_ns)) return false;
         if (cp == 0 && !wait_or_abort(smem_u32(&B.a2empty[ip & 1]), ((ip >> 1) & 1u) ^ 1u, abort, wait_ns))
           return false;
         tc_fence_after();
@@ -459,6 +499,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             break;
           }
           tc_fence_after();
+          // g = 0: the first chunk of W1; g = 1: the others (and W2, see layer2)
+          if (g < 2 && !wait_or_abort(smem_u32(&B.wfull[g]), 0, abort, wait_ns)) {
+            ok = false;
+            break;
+          }
           const uint32_t d1 = tmem + (uint32_t)a * kHC;
           for (int ks = 0; ks < D / 16; ++ks)
             tc_mma_f16(d1, smem_desc(sx + (uint32_t)xb * x_bytes + ks * 256, 128, kx * 128),
@@ -473,9 +518,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         }
       }
       if (ok && g > 0) layer2(g - 1, it - 1, nc - 1);
-      // every MMA of this thread completes before TMEM is freed
+      // every MMA of this thread completes before TMEM is freed, and the
+      // weights' copies land before the CTA ends, even if a role gave up
       tc_commit(smem_u32(&B.drain));
       mbar_wait_bounded(smem_u32(&B.drain), 0);
+      mbar_wait_bounded(smem_u32(&B.wfull[0]), 0);
+      mbar_wait_bounded(smem_u32(&B.wfull[1]), 0);
     }
     __syncwarp();
   } else if (warp < kWarpConv) {
@@ -493,7 +541,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       const bool reads = hh * 16 < n2;  // same for the whole warp
       if (reads) {
         tc_ld16(tmem + lane_base + kTmemAcc2 + (ip & 1u) * 32u + (uint32_t)hh * 16u, o);
-        tc_wait_ld();
+        tc_wait_ld(o);
       }
       tc_fence_before();
       mbar_arrive(smem_u32(&B.a2empty[ip & 1]));
@@ -537,7 +585,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         uint32_t v[64];
         tc_ld32(col, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
         tc_ld32(col + 32u, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        tc_wait_ld();
+        tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&v[0]));
+        tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&v[32]));
         uint32_t hp[32];
 #pragma unroll
         for (int j4 = 0; j4 < 16; ++j4) {
@@ -650,10 +699,6 @@ __host__ __device__ inline uint32_t ly_tmem_cols(int Nt) {
   return c;
 }
 
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
 // 2D tensor copy global -> this CTA's shared memory (box of the tensor map at
 // element coordinates (c0, c1)), completing on `bar` by bytes
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, uint32_t bar) {
@@ -662,22 +707,18 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm,
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(bar)
       : "memory");
 }
-// bulk copy global -> this CTA's shared memory, completing on `bar` by bytes
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
 // XT: the input's type (0 uint8 rows, 1 fp32 rows, 2 fp16 activations in
 // operand order); YF: 1 fp32 output rows (the logits, no activation), 0 fp16
-// activations in operand order with ReLU. x [n x K], y [n x N].
+// activations in operand order with ReLU. x [n x K], y [n x N]. Nw: the column
+// tile that W is stored in, a multiple of Nt: few rows run in narrower tiles
+// than it, one after the other in a stored tile (eight-row groups of its core
+// matrices), on more CTAs. box: rows of a tensor copy (XT 1). A tile's sums do
+// not depend on its width, nor on rows that are not there.
 template <int XT, int YF>
 __global__ void __launch_bounds__(kLyThreads, 1)
-    encode_layer_kernel(const void *__restrict__ x, int K, int N, int Nt, int Npad, float s,
+    encode_layer_kernel(const void *__restrict__ x, int K, int N, int Nt, int Nw, int Npad, float s,
                         const __half *__restrict__ Wp, const float *__restrict__ bias, int64_t n,
-                        void *__restrict__ y, int nraw, const __grid_constant__ CUtensorMap tmx,
+                        void *__restrict__ y, int nraw, int box, const __grid_constant__ CUtensorMap tmx,
                         int *err, int64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t stage_b = ly_stage_bytes(Nt);
@@ -739,7 +780,7 @@ __global__ void __launch_bounds__(kLyThreads, 1)
             break;
           }
           const uint32_t bar = smem_u32(&B.rawfull[rs]), dst = raw_s + rs * kLyRawStage;
-          mbar_arrive_tx(bar, kLyRawStage);
+          mbar_arrive_tx(bar, (uint32_t)box * kLyKs * 4u);
           tma_load_2d(dst, &tmx, ks * kLyKs, row0, bar);
           tma_load_2d(dst + kLyRawStage / 2, &tmx, ks * kLyKs + kLyKs / 2, row0, bar);
         }
@@ -806,13 +847,14 @@ __global__ void __launch_bounds__(kLyThreads, 1)
         uint32_t v[32];
         if (Nt - cc >= 32) {
           tc_ld32(tmem + lane_base + a * (uint32_t)Nt + (uint32_t)cc, v);
+          tc_wait_ld(v);
         } else {
           uint32_t w16[16];
           tc_ld16(tmem + lane_base + a * (uint32_t)Nt + (uint32_t)cc, w16);
+          tc_wait_ld(w16);
 #pragma unroll
           for (int j = 0; j < 16; ++j) v[j] = w16[j];
         }
-        tc_wait_ld();
         const int ncol = min(32, Nt - cc);
         if (row < n) {
           if (YF) {
@@ -859,7 +901,12 @@ __global__ void __launch_bounds__(kLyThreads, 1)
       const int ctile = (int)(item % nct);
       const int64_t row0 = rt * kRows;
       const int rows = n - row0 < kRows ? (int)(n - row0) : kRows;
-      const char *wt = reinterpret_cast<const char *>(Wp) + (size_t)ctile * nks * wbytes;
+      // slice ks of the column tile: at wt + ks wstep
+      const int wsub = Nw / Nt;
+      const size_t wstep = (size_t)Nw * kLyKs * 2;
+      const char *wt = reinterpret_cast<const char *>(Wp) + (size_t)(ctile / wsub) * nks * wstep +
+                       (size_t)(ctile % wsub) * wbytes;
+      const uint32_t xbytes = (uint32_t)((rows + 7) / 8) * (8u * kLyKs * 2u);  // XT 2: the rows there are
       for (int ks = 0; ks < nks; ++ks, ++g) {
         const uint32_t st = g % kLyStages, ph = ((g / kLyStages) & 1u) ^ 1u;
         unsigned char *sx = smem + st * stage_b;
@@ -870,10 +917,10 @@ __global__ void __launch_bounds__(kLyThreads, 1)
             break;
           }
           const uint32_t bar = smem_u32(&B.tfull[0][st]);
-          mbar_arrive_tx(bar, kLyXSlice + wbytes);
+          mbar_arrive_tx(bar, xbytes + wbytes);
           bulk_g2s(sbase + st * stage_b,
-                   static_cast<const char *>(x) + ((size_t)rt * nks + ks) * kLyXSlice, kLyXSlice, bar);
-          bulk_g2s(sbase + st * stage_b + kLyXSlice, wt + (size_t)ks * wbytes, wbytes, bar);
+                   static_cast<const char *>(x) + ((size_t)rt * nks + ks) * kLyXSlice, xbytes, bar);
+          bulk_g2s(sbase + st * stage_b + kLyXSlice, wt + (size_t)ks * wstep, wbytes, bar);
           continue;
         }
         // group grp takes the slices g with g % 2 == grp: two slices' loads
@@ -933,7 +980,7 @@ __global__ void __launch_bounds__(kLyThreads, 1)
         if (lead) {
           const uint32_t bar = smem_u32(&B.tfull[grp][st]);
           mbar_arrive_tx(bar, wbytes);
-          bulk_g2s(sbase + st * stage_b + kLyXSlice, wt + (size_t)ks * wbytes, wbytes, bar);
+          bulk_g2s(sbase + st * stage_b + kLyXSlice, wt + (size_t)ks * wstep, wbytes, bar);
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -1155,7 +1202,14 @@ template <int XT, int YF>
 static cudaError_t launch_layer(nr_index *ix, const void *x, int K, int N, int l, float sc,
                                 const float *bias, int64_t n, void *y, int64_t wait_ns,
                                 cudaStream_t s) {
-  const int nt = ix->ly_nt[l], Np = (N + 15) / 16 * 16;
+  const int nw = ix->ly_nt[l], Np = (N + 15) / 16 * 16;
+  // Narrower column tiles while they leave SMs idle: a CTA's slices follow one
+  // another at the latency of their copies. 4 rows of 1536 values: 42 us for
+  // five layers, 66 of full tiles (and whole row boxes). Past half the SMs
+  // the full tile stays: halving it again would read x twice as often.
+  int nt = nw;
+  while (nt % 32 == 0 && nt > 32 && (n + kRows - 1) / kRows * (Np / nt) * 2 <= ix->num_sms) nt /= 2;
+  const int rbox = n < kRows ? (int)((n + 7) / 8 * 8) : kRows;  // rows of a tensor copy
   // fp32 first layer: four raw stages for the tensor copies, or two
   int nraw = 0;
   CUtensorMap tm;
@@ -1164,10 +1218,10 @@ static cudaError_t launch_layer(nr_index *ix, const void *x, int K, int N, int l
     nraw = kLyRawMax;
     while (nraw > 2 && ly_smem_bytes(nt, nraw) > (uint32_t)ix->smem_optin) nraw -= 2;
     if (ly_smem_bytes(nt, nraw) > (uint32_t)ix->smem_optin) return cudaErrorInvalidConfiguration;
-    // x [n rows x K] fp32: boxes of 32 values x 128 rows, 128-byte swizzle
+    // x [n rows x K] fp32: boxes of 32 values x rbox rows, 128-byte swizzle
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)n};
     const cuuint64_t strides[1] = {(cuuint64_t)K * 4u};
-    const cuuint32_t box[2] = {(cuuint32_t)(kLyKs / 2), (cuuint32_t)kRows}, es[2] = {1u, 1u};
+    const cuuint32_t box[2] = {(cuuint32_t)(kLyKs / 2), (cuuint32_t)rbox}, es[2] = {1u, 1u};
     const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
     if (!encode) return cudaErrorNotSupported;
     if (encode(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(x), dims, strides, box, es,
@@ -1185,9 +1239,9 @@ static cudaError_t launch_layer(nr_index *ix, const void *x, int K, int N, int l
   if (e != cudaSuccess) return e;
   const int64_t items = (n + kRows - 1) / kRows * (Np / nt);
   const int64_t grid = items < ix->num_sms ? items : ix->num_sms;
-  kern<<<(unsigned)grid, kLyThreads, smem, s>>>(x, K, N, nt, Np, sc,
+  kern<<<(unsigned)grid, kLyThreads, smem, s>>>(x, K, N, nt, nw, Np, sc,
                                                 static_cast<const __half *>(ix->Wl) + ix->ly_off[l],
-                                                bias, n, y, nraw, tm, ix->d_err, wait_ns);
+                                                bias, n, y, nraw, rbox, tm, ix->d_err, wait_ns);
   ix->launches += 1;
   return cudaGetLastError();
 }
