@@ -5,18 +5,27 @@
 // one CTA per SM keeps W1 and W2 in shared memory and walks 128-row tiles (the
 // 128 TMEM lanes of its accumulators). Layer 1 runs in chunks of 128 hidden
 // units: one thread issues tcgen05.mma (kind::f16, fp16 operands, fp32
-// accumulation in TMEM) over the X tile and the chunk of W1; eight epilogue
-// warps read each accumulator back with tcgen05.ld, apply scale, bias and
-// ReLU, and write the chunk as fp16 pairs back into TMEM with tcgen05.st,
-// where it is the A operand of the layer-2 MMAs that accumulate
-// l [128 x N2] (N2 = b padded to 16 or 32) against W2. Two layer-1
-// accumulators, two hidden chunks and two layer-2 accumulators let the tensor
-// pipe work on the next chunk while the epilogue converts the previous one;
-// four converter warps turn the next X tile into fp16 meanwhile (two
-// buffers where shared memory allows; uint8 inputs are exact in fp16; the
-// input scale is applied to the fp32 accumulator). A tile's logits are
-// stored after the next tile's first chunk, when its layer-2 MMAs are done.
-// Every hand-off is an mbarrier (tcgen05.commit, or thread arrivals). Shared
+// accumulation in TMEM) over the X tile and the chunk of W1; two groups of
+// eight epilogue warps, which take alternate chunks, read each accumulator
+// back with tcgen05.ld, apply scale, bias and ReLU, and write the chunk as
+// fp16 pairs back into TMEM with tcgen05.st, where it is the A operand of the
+// layer-2 MMAs that accumulate l [128 x N2] (N2 = b padded to 16 or 32)
+// against W2. Two layer-1 accumulators, three hidden chunks and two layer-2
+// accumulators let the tensor pipe work on the next chunk while the groups
+// convert the two before it; four converter warps turn the next X tile into
+// fp16 meanwhile (two buffers where shared memory allows; uint8 inputs are
+// exact in fp16; the input scale is applied to the fp32 accumulator). A tile's
+// logits are stored during a later tile, when its layer-2 MMAs are done.
+// Every hand-off is an mbarrier (tcgen05.commit, or one arrival a warp).
+//
+// What bounds it (1,000,037 uint8 rows, D = 128, H = 512, b = 24): 182 us, 855
+// TFLOP/s. A chunk takes some 1,650 cycles: 896 of MMAs (512 in layer 1; 384
+// in layer 2, whose 128 x 32 x 16 step takes 48) and the hand-offs that are
+// not hidden behind them. At 254 us it was the issue of the MMAs: some 90
+// cycles each in a branch of one lane, where the descriptors went to uniform
+// registers one by one. The whole warp runs the loop now and one lane issues
+// eight at a time (201 us); two epilogue groups instead of one and layer 2 two
+// chunks behind layer 1 took it from there (one chunk behind: 192 us). Shared
 // memory operands sit in the canonical K-major no-swizzle layout
 // (nr_tc_kmajor_off), in which the host stores W1 and W2.
 //
@@ -101,6 +110,12 @@ __device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t adesc, uint
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// one lane of the warp, the same each time (all lanes call)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
@@ -167,20 +182,22 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
 // ------------------------------------------------------------ tensor-core kernel
 constexpr int kRows = 128;     // rows per tile = TMEM lanes of the accumulators
 constexpr int kHC = 128;       // hidden units per layer-1 chunk
-constexpr int kEpiWarps = 8;   // two per TMEM lane group, one column half of a chunk each
+// two epilogue groups, which take alternate chunks; in a group two warps per
+// TMEM lane group, one column half of a chunk each
+constexpr int kEpiWarps = 8;  // a group
 constexpr int kConvWarps = 4;
-constexpr int kWarpMma = 0, kWarpEpi = 1, kWarpConv = kWarpEpi + kEpiWarps;
-constexpr int kTcThreads = 32 * (kWarpConv + kConvWarps);  // 416
-constexpr int kEpiThreads = 32 * kEpiWarps, kConvThreads = 32 * kConvWarps;
-// TMEM columns: layer-1 accumulators at 0 and 128, layer-2 accumulators at 256
-// and 288, the hidden chunk as the fp16 A operand of layer 2 (two values a
-// column) at 320 and 384
-constexpr uint32_t kTmemCols = 512, kTmemAcc2 = 256, kTmemHid = 320;
+constexpr int kWarpMma = 0, kWarpEpi = 1, kWarpConv = kWarpEpi + 2 * kEpiWarps;
+constexpr int kTcThreads = 32 * (kWarpConv + kConvWarps);  // 672
+// TMEM columns: layer-1 accumulators at 0 and 128 (one per epilogue group),
+// hidden chunks as the fp16 A operand of layer 2 (two values a column) at 256,
+// 320 and 384, layer-2 accumulators at 448 and 480
+constexpr int kHid = 3;
+constexpr uint32_t kTmemCols = 512, kTmemHid = 256, kTmemAcc2 = 448;
 
 struct TcBars {
   uint64_t xfull[2], xempty[2];    // X tiles: converters -> MMA -> converters
   uint64_t a1full[2], a1empty[2];  // layer-1 accumulators: MMA -> epilogue -> MMA
-  uint64_t hfull[2], hempty[2];    // hidden chunks in TMEM: epilogue -> MMA -> epilogue
+  uint64_t hfull[kHid], hempty[kHid];  // hidden chunks in TMEM: epilogue -> MMA -> epilogue
   uint64_t a2full[2], a2empty[2];  // layer-2 accumulators
   uint64_t wfull[2];               // the weights: W1's first chunk; the rest and W2
   uint64_t drain;                  // every MMA of the CTA complete
@@ -205,9 +222,15 @@ __host__ __device__ inline TcLayout tc_layout(int D, int H, int n2, int nxb) {
   return L;
 }
 
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(bar)
-               : "memory");
+// One arrival for the whole warp, after all its lanes' work and fences
+// (instead of 32 updates of one barrier: 219 -> 201 us on the rows above,
+// 286 -> 282 us for 100,000 rows through the layer kernel)
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0)
+    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(bar)
+                 : "memory");
+  __syncwarp();
 }
 // layer-2 MMA with A read from TMEM (a_tmem: its first column), B from shared memory
 __device__ __forceinline__ void tc_mma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
@@ -227,16 +250,12 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
-      "%25,%26,%27,%28,%29,%30,%31,%32};\n" ::"r"(taddr),
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(taddr),
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
-      "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
-      "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
-      "r"(r[29]), "r"(r[30]), "r"(r[31])
+      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 __device__ __forceinline__ void tc_wait_st() {
@@ -297,8 +316,9 @@ __device__ __forceinline__ void u8x16_to_f16(const uint4 v, uint4 &lo, uint4 &hi
 
 // The converter warps' role in the tensor-core encoders: each X tile of 128
 // rows -> fp16 operand in the K-major core-matrix layout of buffer tile % nxb
-// (xempty: the buffer is free; xfull: it is written, kConvThreads arrivals).
+// (xempty: the buffer is free; xfull: it is written, an arrival a warp).
 // ct: the thread's index among the converter threads.
+constexpr int kF32Items = 6;  // a thread's fp32 pieces (32 bytes each) in flight
 template <int DT>
 __device__ __forceinline__ void tc_convert_tiles(const void *__restrict__ x, int D, int kx, int nxb,
                                                  int64_t nq, int64_t ntiles, uint32_t x_bytes,
@@ -350,12 +370,12 @@ __device__ __forceinline__ void tc_convert_tiles(const void *__restrict__ x, int
       }
     } else {
       const float *xs = static_cast<const float *>(x) + row0 * D;
-#pragma unroll
-      for (int j0 = 0; j0 < 16; j0 += 8) {
+#pragma unroll 1
+      for (int j0 = 0; j0 < 16; j0 += kF32Items) {
         if (j0 >= per || !ok) break;
-        float4 u[8], w[8];
+        float4 u[kF32Items], w[kF32Items];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < kF32Items; ++j) {
           int rr, pc;
           item(j0 + j, rr, pc);
           u[j] = w[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -368,7 +388,7 @@ __device__ __forceinline__ void tc_convert_tiles(const void *__restrict__ x, int
         if (j0 == 0) ok = warp_wait(smem_u32(&xempty[xb]), xpar, abort, wait_ns);
         if (!ok) break;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < kF32Items; ++j) {
           if (j0 + j >= per) break;
           int rr, pc;
           item(j0 + j, rr, pc);
@@ -382,21 +402,23 @@ __device__ __forceinline__ void tc_convert_tiles(const void *__restrict__ x, int
     }
     if (!ok) break;
     fence_async_smem();
-    mbar_arrive(smem_u32(&xfull[xb]));
+    warp_arrive(smem_u32(&xfull[xb]));
   }
 }
 
 // Persistent, warp-specialised: each CTA (one per SM) keeps W1 and W2 in
 // shared memory and takes 128-row tiles tile = blockIdx.x, + gridDim.x, ...:
 //   converter warps  X tile -> fp16 operand (nxb = 2 buffers, or 1 for wide shapes)
-//   MMA thread       layer 1 of chunk g (128 hidden units) into accumulator g % 2,
-//                    then layer 2 of chunk g - 1 with its A operand in TMEM
-//   epilogue warps   accumulator -> ReLU(s acc + b1) -> fp16 hidden chunk in TMEM
-//                    (buffer g % 2); after the next tile's first chunk, the
-//                    tile's layer-2 accumulator + b2 -> out (float4 stores if
-//                    vec_out: b % 4 == 0 and out 16-byte aligned)
-// so that the tensor pipe runs layer 1 of the next chunk while the epilogue
-// turns the previous one into the layer-2 operand.
+//   MMA warp         layer 1 of chunk g (128 hidden units) into accumulator g % 2,
+//                    then layer 2 of chunk g - 2 with its A operand in TMEM
+//   epilogue groups  chunks with g % 2 = the group: accumulator ->
+//                    ReLU(s acc + b1) -> fp16 hidden chunk in TMEM (buffer
+//                    g % 3); tiles of its parity, after its first chunk of a
+//                    later tile: layer-2 accumulator + b2 -> out (float4 stores
+//                    if vec_out: b % 4 == 0 and out 16-byte aligned)
+// so that the tensor pipe runs layer 1 of the next chunk while the groups turn
+// the two before it into layer-2 operands. 672 threads leave 80 registers each:
+// the epilogue takes a chunk's 64 columns a warp in two pieces of 32.
 template <int DT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     encode_tc_kernel(const void *__restrict__ x, int D, int H, int b, int n2, int nxb, int vec_out,
@@ -408,7 +430,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const TcLayout L = tc_layout(D, H, n2, nxb);
   TcBars &B = *reinterpret_cast<TcBars *>(smem + L.bars);
   volatile int *abort = &B.abort;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform to the compiler too
   const int kx = D / 8;      // 16-byte K chunks per row of X and W1
   const int nc = H / kHC;    // layer-1 chunks per tile
   const uint32_t x_bytes = (uint32_t)kRows * D * 2, w1_bytes = (uint32_t)kHC * D * 2;
@@ -424,14 +447,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&B.xfull[i]), kConvThreads);
+      mbar_init(smem_u32(&B.xfull[i]), kConvWarps);
       mbar_init(smem_u32(&B.xempty[i]), 1);
       mbar_init(smem_u32(&B.a1full[i]), 1);
-      mbar_init(smem_u32(&B.a1empty[i]), kEpiThreads);
-      mbar_init(smem_u32(&B.hfull[i]), kEpiThreads);
-      mbar_init(smem_u32(&B.hempty[i]), 1);
+      mbar_init(smem_u32(&B.a1empty[i]), kEpiWarps);
       mbar_init(smem_u32(&B.a2full[i]), 1);
-      mbar_init(smem_u32(&B.a2empty[i]), kEpiThreads);
+      mbar_init(smem_u32(&B.a2empty[i]), kEpiWarps);
+    }
+    for (int i = 0; i < kHid; ++i) {
+      mbar_init(smem_u32(&B.hfull[i]), kEpiWarps);
+      mbar_init(smem_u32(&B.hempty[i]), 1);
     }
     mbar_init(smem_u32(&B.wfull[0]), 1);
     mbar_init(smem_u32(&B.wfull[1]), 1);
@@ -461,75 +486,84 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = B.tmem_slot;
 
   if (warp == kWarpMma) {
-    if (lane == 0) {
-      const uint32_t idesc1 = mma_idesc(kRows, kHC), idesc2 = mma_idesc(kRows, n2);
-      const uint32_t sx = sbase + L.x, sw1 = sbase + L.w1, sw2 = sbase + L.w2;
-      // layer 2 of chunk number gp (chunk cp of tile number ip of this CTA):
-      // hidden chunk (TMEM) x W2 chunk into the tile's accumulator
-      auto layer2 = [&](uint32_t gp, uint32_t ip, int cp) -> bool {
-        const int hb = (int)(gp & 1);
-        if (!wait_or_abort(smem_u32(&B.hfull[hb]), (gp >> 1) & 1u, abort, wait_ns)) return false;
-        if (gp == 0 && !wait_or_abort(smem_u32(&B.wfull[1]), 0, abort, wait_ns)) return false;
-        if (cp == 0 && !wait_or_abort(smem_u32(&B.a2empty[ip & 1]), ((ip >> 1) & 1u) ^ 1u, abort, wait_ns))
-          return false;
-        tc_fence_after();
-        const uint32_t d2 = tmem + kTmemAcc2 + (ip & 1u) * 32u;
-        const uint32_t ah = tmem + kTmemHid + (uint32_t)hb * (kHC / 2);
-        for (int ks = 0; ks < kHC / 16; ++ks)
-          tc_mma_f16_ts(d2, ah + (uint32_t)ks * 8u,
-                        smem_desc(sw2 + (uint32_t)cp * w2_bytes + ks * 256, 128, 16 * 128), idesc2,
-                        (cp > 0 || ks > 0) ? 1u : 0u);
-        tc_commit(smem_u32(&B.hempty[hb]));
-        if (cp == nc - 1) tc_commit(smem_u32(&B.a2full[ip & 1]));
-        return true;
-      };
-      bool ok = true;
-      uint32_t g = 0, it = 0;  // chunks and tiles of this CTA so far
-      for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
-        const int xb = nxb == 2 ? (int)(it & 1) : 0;
-        const uint32_t xpar = (nxb == 2 ? it >> 1 : it) & 1u;
-        if (!wait_or_abort(smem_u32(&B.xfull[xb]), xpar, abort, wait_ns)) {
-          ok = false;
+    const bool issues = elect_one();  // the MMA thread: all MMAs and commits
+    const uint32_t idesc1 = mma_idesc(kRows, kHC), idesc2 = mma_idesc(kRows, n2);
+    const uint32_t sx = sbase + L.x, sw1 = sbase + L.w1, sw2 = sbase + L.w2;
+    // layer 1 of chunk number g1 (chunk c1 of tile number it1 of this CTA),
+    // then layer 2 of chunk number g2 (chunk c2 of tile number it2), two
+    // chunks behind it, and of the last ones after the last layer 1
+    uint32_t g1 = 0, it1 = 0, g2 = 0, it2 = 0, h2 = 0, hpar = 0;
+    int c1 = 0, c2 = 0;
+    int64_t tile = blockIdx.x;
+    while (tile < ntiles || g2 < g1) {
+      if (tile < ntiles) {
+        const int a = (int)(g1 & 1), xb = nxb == 2 ? (int)(it1 & 1) : 0;
+        if (!warp_wait(smem_u32(&B.a1empty[a]), ((g1 >> 1) & 1u) ^ 1u, abort, wait_ns)) break;
+        if (c1 == 0 && !warp_wait(smem_u32(&B.xfull[xb]), (nxb == 2 ? it1 >> 1 : it1) & 1u, abort, wait_ns))
           break;
-        }
-        for (int c = 0; c < nc; ++c, ++g) {
-          const int a = (int)(g & 1);
-          if (!wait_or_abort(smem_u32(&B.a1empty[a]), ((g >> 1) & 1u) ^ 1u, abort, wait_ns)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          // g = 0: the first chunk of W1; g = 1: the others (and W2, see layer2)
-          if (g < 2 && !wait_or_abort(smem_u32(&B.wfull[g]), 0, abort, wait_ns)) {
-            ok = false;
-            break;
-          }
-          const uint32_t d1 = tmem + (uint32_t)a * kHC;
-          for (int ks = 0; ks < D / 16; ++ks)
-            tc_mma_f16(d1, smem_desc(sx + (uint32_t)xb * x_bytes + ks * 256, 128, kx * 128),
-                       smem_desc(sw1 + (uint32_t)c * w1_bytes + ks * 256, 128, kx * 128), idesc1,
-                       ks > 0 ? 1u : 0u);
+        // g1 = 0: the first chunk of W1; g1 = 1: the others (and W2, see layer 2)
+        if (g1 < 2 && !warp_wait(smem_u32(&B.wfull[g1]), 0, abort, wait_ns)) break;
+        tc_fence_after();
+        const uint32_t d1 = tmem + (uint32_t)a * kHC;
+        const uint64_t ad = smem_desc(sx + (uint32_t)xb * x_bytes, 128, kx * 128);
+        const uint64_t bd = smem_desc(sw1 + (uint32_t)c1 * w1_bytes, 128, kx * 128);
+        if (issues) {
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            if (ks < D / 16)
+              tc_mma_f16(d1, ad + (uint64_t)(ks * 16), bd + (uint64_t)(ks * 16), idesc1, ks > 0 ? 1u : 0u);
           tc_commit(smem_u32(&B.a1full[a]));
-          if (c == nc - 1) tc_commit(smem_u32(&B.xempty[xb]));
-          if (g > 0 && !layer2(g - 1, c > 0 ? it : it - 1, c > 0 ? c - 1 : nc - 1)) {
-            ok = false;
-            break;
-          }
+          if (c1 == nc - 1) tc_commit(smem_u32(&B.xempty[xb]));
+        }
+        __syncwarp();
+        ++g1;
+        if (++c1 == nc) {
+          c1 = 0;
+          ++it1;
+          tile += gridDim.x;
         }
       }
-      if (ok && g > 0) layer2(g - 1, it - 1, nc - 1);
-      // every MMA of this thread completes before TMEM is freed, and the
-      // weights' copies land before the CTA ends, even if a role gave up
-      tc_commit(smem_u32(&B.drain));
-      mbar_wait_bounded(smem_u32(&B.drain), 0);
-      mbar_wait_bounded(smem_u32(&B.wfull[0]), 0);
-      mbar_wait_bounded(smem_u32(&B.wfull[1]), 0);
+      if (g2 + 3 <= g1 || tile >= ntiles) {
+        if (!warp_wait(smem_u32(&B.hfull[h2]), hpar, abort, wait_ns)) break;
+        if (c2 == 0 && !warp_wait(smem_u32(&B.a2empty[it2 & 1]), ((it2 >> 1) & 1u) ^ 1u, abort, wait_ns))
+          break;
+        if (g2 == 0 && !warp_wait(smem_u32(&B.wfull[1]), 0, abort, wait_ns)) break;
+        tc_fence_after();
+        const uint32_t d2 = tmem + kTmemAcc2 + (it2 & 1u) * 32u;
+        const uint32_t ah = tmem + kTmemHid + h2 * (kHC / 2);
+        const uint64_t bd = smem_desc(sw2 + (uint32_t)c2 * w2_bytes, 128, 16 * 128);
+        if (issues) {
+#pragma unroll
+          for (int ks = 0; ks < kHC / 16; ++ks)
+            tc_mma_f16_ts(d2, ah + (uint32_t)ks * 8u, bd + (uint64_t)(ks * 16), idesc2,
+                          (c2 > 0 || ks > 0) ? 1u : 0u);
+          tc_commit(smem_u32(&B.hempty[h2]));
+          if (c2 == nc - 1) tc_commit(smem_u32(&B.a2full[it2 & 1]));
+        }
+        __syncwarp();
+        ++g2;
+        if (++h2 == kHid) {
+          h2 = 0;
+          hpar ^= 1u;
+        }
+        if (++c2 == nc) {
+          c2 = 0;
+          ++it2;
+        }
+      }
     }
+    // every MMA of this thread completes before TMEM is freed, and the
+    // weights' copies land before the CTA ends, even if a role gave up
+    if (issues) tc_commit(smem_u32(&B.drain));
     __syncwarp();
+    mbar_wait_bounded(smem_u32(&B.drain), 0);
+    mbar_wait_bounded(smem_u32(&B.wfull[0]), 0);
+    mbar_wait_bounded(smem_u32(&B.wfull[1]), 0);
   } else if (warp < kWarpConv) {
-    const int lg = warp & 3;                 // TMEM lane group this warp may access
-    const int hh = (warp - kWarpEpi) >> 2;   // column half of each chunk
-    const int r = lg * 32 + lane;            // tile row = TMEM lane
+    const int lg = warp & 3;       // TMEM lane group this warp may access
+    const int hh = ((warp - kWarpEpi) >> 2) & 1;  // column half of each chunk
+    const uint32_t grp = (uint32_t)(warp - kWarpEpi) / kEpiWarps;  // chunks and tiles of this parity
+    const int r = lg * 32 + lane;  // tile row = TMEM lane
     const uint32_t lane_base = (uint32_t)(lg * 32) << 16;
     const __half2 zero2 = __float2half2_rn(0.0f);
     // logits of tile number ip (global tile t): layer-2 accumulator + b2 -> out,
@@ -544,7 +578,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         tc_wait_ld(o);
       }
       tc_fence_before();
-      mbar_arrive(smem_u32(&B.a2empty[ip & 1]));
+      warp_arrive(smem_u32(&B.a2empty[ip & 1]));
       const int64_t row = t * kRows + r;
       const int ncol = b - hh * 16 < 16 ? b - hh * 16 : 16;
       if (reads && row < nq) {
@@ -567,30 +601,31 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
       return true;
     };
-    uint32_t g = 0, it = 0;
-    int64_t last_tile = 0;
+    // this group's chunks: number g (accumulator grp, hidden buffer h) is chunk
+    // c of tile number it; and the next tile whose logits it writes
+    uint32_t it = 0, h = grp, hpar = 1u, apar = 0, ip = grp;
+    int c = (int)grp;
     bool ok = true;
-    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
-      for (int c = 0; c < nc; ++c, ++g) {
-        const int a = (int)(g & 1);
-        if (!warp_wait(smem_u32(&B.a1full[a]), (g >> 1) & 1u, abort, wait_ns)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        // h = ReLU(s acc + b1) as fp16 pairs, 32 accumulator columns at a time
-        const uint32_t col = tmem + lane_base + (uint32_t)a * kHC + (uint32_t)hh * 64u;
-        const float *bb = sb1 + c * kHC + hh * 64;
-        // both 32-column loads in flight before one wait
-        uint32_t v[64];
-        tc_ld32(col, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tc_ld32(col + 32u, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&v[0]));
-        tc_wait_ld(*reinterpret_cast<uint32_t(*)[32]>(&v[32]));
-        uint32_t hp[32];
+    for (;;) {
+      while (c >= nc) {
+        c -= nc;
+        ++it;
+      }
+      if (blockIdx.x + (int64_t)it * gridDim.x >= ntiles) break;
+      if (!warp_wait(smem_u32(&B.a1full[grp]), apar, abort, wait_ns)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      // h = ReLU(s acc + b1) as fp16 pairs, 32 accumulator columns at a time
+      const uint32_t col = tmem + lane_base + grp * kHC + (uint32_t)hh * 64u;
+      const uint32_t hid = tmem + lane_base + kTmemHid + h * (kHC / 2) + (uint32_t)hh * 32u;
+      const float *bb = sb1 + c * kHC + hh * 64;
+      uint32_t v[32], hp[16];
+      auto relu = [&](const float *bp) {
 #pragma unroll
-        for (int j4 = 0; j4 < 16; ++j4) {
-          const float4 bq = reinterpret_cast<const float4 *>(bb)[j4];
+        for (int j4 = 0; j4 < 8; ++j4) {
+          const float4 bq = reinterpret_cast<const float4 *>(bp)[j4];
           const float h0 = __fmaf_rn(s, __uint_as_float(v[4 * j4]), bq.x);
           const float h1 = __fmaf_rn(s, __uint_as_float(v[4 * j4 + 1]), bq.y);
           const float h2 = __fmaf_rn(s, __uint_as_float(v[4 * j4 + 2]), bq.z);
@@ -600,28 +635,45 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           hp[2 * j4] = *reinterpret_cast<const uint32_t *>(&p0);
           hp[2 * j4 + 1] = *reinterpret_cast<const uint32_t *>(&p1);
         }
-        tc_fence_before();
-        mbar_arrive(smem_u32(&B.a1empty[a]));
-        // the layer-2 MMAs of chunk g - 2 have read this hidden buffer
-        if (!warp_wait(smem_u32(&B.hempty[a]), ((g >> 1) & 1u) ^ 1u, abort, wait_ns)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        tc_st32(tmem + lane_base + kTmemHid + (uint32_t)a * (kHC / 2) + (uint32_t)hh * 32u, hp);
-        tc_wait_st();
-        tc_fence_before();
-        mbar_arrive(smem_u32(&B.hfull[a]));
-        // the previous tile's logits, once this tile's first chunk is on its way
-        if (c == 0 && it > 0 && !logits(it - 1, last_tile)) {
-          ok = false;
-          break;
-        }
+      };
+      tc_ld32(col, v);
+      tc_wait_ld(v);
+      relu(bb);
+      tc_ld32(col + 32u, v);
+      // the layer-2 MMAs of the chunk three before have read this hidden buffer
+      if (!warp_wait(smem_u32(&B.hempty[h]), hpar, abort, wait_ns)) {
+        tc_wait_ld(v);
+        ok = false;
+        break;
       }
-      last_tile = tile;
-      if (!ok) break;
+      tc_fence_after();
+      tc_st16(hid, hp);
+      tc_wait_ld(v);
+      tc_fence_before();
+      warp_arrive(smem_u32(&B.a1empty[grp]));
+      relu(bb + 32);
+      tc_st16(hid + 16u, hp);
+      tc_wait_st();
+      tc_fence_before();
+      warp_arrive(smem_u32(&B.hfull[h]));
+      // an earlier tile's logits, once this chunk is on its way
+      if (ip < it) {
+        if (!logits(ip, blockIdx.x + (int64_t)ip * gridDim.x)) {
+          ok = false;
+          break;
+        }
+        ip += 2;
+      }
+      apar ^= 1u;
+      c += 2;
+      h += 2;
+      if (h >= kHid) {
+        h -= kHid;
+        hpar ^= 1u;
+      }
     }
-    if (ok && it > 0) ok = logits(it - 1, last_tile);
+    for (; ok && blockIdx.x + (int64_t)ip * gridDim.x < ntiles; ip += 2)
+      ok = logits(ip, blockIdx.x + (int64_t)ip * gridDim.x);
   } else {
     tc_convert_tiles<DT>(x, D, kx, nxb, nq, ntiles, x_bytes, smem + L.x, B.xfull, B.xempty, abort,
                          wait_ns, tid - kWarpConv * 32);
@@ -671,7 +723,7 @@ constexpr int kLyEpiWarps = 4, kLyProdWarps = 4;  // a producer group
 constexpr int kLyWarpEpi = 1, kLyWarpProd = kLyWarpEpi + kLyEpiWarps;
 constexpr int kLyWarpTma = kLyWarpProd + 2 * kLyProdWarps;
 constexpr int kLyThreads = 32 * (kLyWarpTma + 1);  // 448
-constexpr int kLyProdThreads = 32 * kLyProdWarps, kLyEpiThreads = 32 * kLyEpiWarps;
+constexpr int kLyProdThreads = 32 * kLyProdWarps;
 constexpr uint32_t kLyXSlice = (uint32_t)kRows * kLyKs * 2u;    // 16 KB of fp16
 
 struct LyBars {
@@ -742,18 +794,18 @@ __global__ void __launch_bounds__(kLyThreads, 1)
   }
   if (tid == 0) {
     for (int i = 0; i < kLyStages; ++i) {
-      mbar_init(smem_u32(&B.xfull[i]), kLyProdThreads);
+      mbar_init(smem_u32(&B.xfull[i]), kLyProdWarps);
       mbar_init(smem_u32(&B.tfull[0][i]), 1);
       mbar_init(smem_u32(&B.tfull[1][i]), 1);
       mbar_init(smem_u32(&B.empty[i]), 1);
     }
     for (int i = 0; i < kLyRawMax; ++i) {
       mbar_init(smem_u32(&B.rawfull[i]), 1);
-      mbar_init(smem_u32(&B.rawempty[i]), kLyProdThreads);
+      mbar_init(smem_u32(&B.rawempty[i]), kLyProdWarps);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&B.accfull[i]), 1);
-      mbar_init(smem_u32(&B.accempty[i]), kLyEpiThreads);
+      mbar_init(smem_u32(&B.accempty[i]), kLyEpiWarps);
     }
     mbar_init(smem_u32(&B.drain), 1);
     B.abort = 0;
@@ -888,7 +940,7 @@ __global__ void __launch_bounds__(kLyThreads, 1)
         }
       }
       tc_fence_before();
-      mbar_arrive(smem_u32(&B.accempty[a]));
+      warp_arrive(smem_u32(&B.accempty[a]));
     }
   } else if (warp < kLyWarpTma) {  // producers: x and W slices into the stage ring
     const int grp = (warp - kLyWarpProd) / kLyProdWarps;  // XT 0 / 1: two groups
@@ -961,7 +1013,7 @@ __global__ void __launch_bounds__(kLyThreads, 1)
           // its writes are the async proxy's, which the arrival alone does not
           // order after them (rows of a slice then held a later slice's values)
           fence_async_smem();
-          mbar_arrive(smem_u32(&B.rawempty[rs]));
+          warp_arrive(smem_u32(&B.rawempty[rs]));
         } else {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {  // 16 uint8 values (piece q) -> chunks 2q, 2q + 1
@@ -992,7 +1044,7 @@ __global__ void __launch_bounds__(kLyThreads, 1)
           }
         }
         fence_async_smem();
-        mbar_arrive(smem_u32(&B.xfull[st]));
+        warp_arrive(smem_u32(&B.xfull[st]));
       }
     }
     // the bulk copies it issued land before the CTA ends, even if a role
