@@ -473,7 +473,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     bulk_g2s(sbase + L.w1, w1, w1_bytes, smem_u32(&B.wfull[0]));
     mbar_arrive_tx(smem_u32(&B.wfull[1]), rest1 + all2);
     for (int c = 1; c < nc; ++c)
-      bulk_g2s(sbase + L.w1 + (uint32_t)c * w1_bytes, w1 + (size_t)c * w1_bytes, w1_bytes, smem_u32(&B.wfull[1]));
+      bulk_g2s(sbase + L.w1 + (uint32_t)c * w1_bytes, w1 + (size_t)c * w1_bytes, w1_bytes,
+               smem_u32(&B.wfull[1]));
     bulk_g2s(sbase + L.w2, W2p, all2, smem_u32(&B.wfull[1]));
   }
   // the biases

@@ -5,9 +5,9 @@
 // spans of a query in stream order.
 //
 // Bound by HBM at large batches, less what queries share in L2, and by latency
-// at small ones: one block a query left a single query to one SM (one uint8 query
-// of 31,000 candidates 523 us, four fp32 queries of 154 MB each 7.8 ms; cut
-// into spans 60 us and 0.12 ms).
+// at small ones: one block a query left a single query to one SM (one uint8
+// query of 61,900 candidates 523 us, four fp32 queries of 154 MB each 7.8 ms;
+// cut into spans 41 us and 0.16 ms, with the commits).
 //
 // Launch shapes measured on GB300: the scan is limited by the bytes in flight
 // per SM, so tiles are small (128 uint8 rows, 32-64 fp32 rows). uint8, D = 128:
@@ -206,8 +206,9 @@ struct RefineArgs {
   uint32_t pool_cap;
 };
 
-// The item of ticket t: its query i and its span, by a whole warp. Tickets go group by group: the first spans of the group's
-// queries, then the other spans query by query.
+// The item of ticket t: its query i and its span, by a whole warp. Tickets go
+// group by group: the first spans of the group's queries, then the other spans
+// query by query.
 template <class F>
 __device__ __forceinline__ void item_of(const RefineArgs &a, F pre, uint32_t t, int &i, uint32_t &span) {
   const int nq = (int)a.nq;
@@ -326,7 +327,8 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
       lg.pool_used = &a.plan->pool_used;
       lg.pool = a.pool;
       lg.pool_cap = a.pool_cap;
-      nrq::refine_span<DT, TR, CPR, KCC, ST>(a.rf, m, p0, p1, a.nL[q], a.seg + (size_t)q * a.Lmax, held, r, lg);
+      nrq::refine_span<DT, TR, CPR, KCC, ST>(a.rf, m, p0, p1, a.nL[q], a.seg + (size_t)q * a.Lmax, held, r,
+                                             lg);
       const uint32_t base = (uint32_t)ctl[kCtlItem], spans = (uint32_t)ctl[kCtlSpans];
       uint32_t next = sp + 1;  // the next span to commit, when held
       bool redo = false;
@@ -525,7 +527,7 @@ nrq::RefineParams refine_params(const nr_index *ix, int k) {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Scratch of a refine launch: [plan][order of whole streams], and where
+// Scratch of a refine launch: [order of whole streams][plan], and where
 // streams may be cut into items spans: [item prefix][plan, query states, ready
 // flags (zeroed together)][span headers][committed top-k][log entries]
 struct RefineScratch {

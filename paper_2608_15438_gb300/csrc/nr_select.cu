@@ -1,6 +1,6 @@
 // K3 select: bucket lookup through the CSR directory (Sec. 3.3) and the
-// centroid stage of Sec. 3.4.2 / Algorithm 2, one 128-thread CTA per query
-// (nrq::select_block):
+// centroid stage of Sec. 3.4.2 / Algorithm 2, one CTA per query of 128 threads,
+// or 512 where there are few queries (nrq::select_block):
 //   1. probe i -> cluster range [bkt_off[u_i], bkt_off[u_i + 1]) (range-checked);
 //   2. every cluster c of every probed bucket gets its centroid distance
 //      d_c = sum_j (l_j - mu_cj)^2 as a sequential fp32 fmaf chain over j;

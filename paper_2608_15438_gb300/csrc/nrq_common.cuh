@@ -1,6 +1,6 @@
 // Shared definitions of the per-query building blocks of the query path
 // (nrq_route.cuh: route_warp, nrq_select.cuh: select_block,
-// nrq_refine.cuh: refine_block).
+// nrq_refine.cuh: refine_span).
 #pragma once
 
 #include <cuda_runtime.h>
