@@ -23,16 +23,17 @@ __global__ void route_kernel(nrq::RouteParams rp, const float *__restrict__ logi
   if (lane == 0) nprobe[q] = n;
 }
 
-// One 128-thread block per query: the threshold enumeration (route_block).
-__global__ void __launch_bounds__(nrq::kRouteThreads) route_block_kernel(
+// One block of NT threads per query: the threshold enumeration (route_block).
+template <int NT>
+__global__ void __launch_bounds__(NT) route_block_kernel(
     nrq::RouteParams rp, const float *__restrict__ logits, int64_t nq, uint32_t *__restrict__ codes,
     int32_t *__restrict__ nprobe) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t q = blockIdx.x;
   if (q >= nq) return;
   uint32_t *out = codes + (size_t)q * rp.P;
-  const int n = nrq::route_block(rp, logits + q * rp.b, smem, out);
-  for (int t = n + (int)threadIdx.x; t < rp.P; t += nrq::kRouteThreads) out[t] = 0xffffffffu;
+  const int n = nrq::route_block<NT>(rp, logits + q * rp.b, smem, out);
+  for (int t = n + (int)threadIdx.x; t < rp.P; t += NT) out[t] = 0xffffffffu;
   if (threadIdx.x == 0) nprobe[q] = n;
 }
 
@@ -61,11 +62,15 @@ cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int
   const nrq::RouteParams rpb = nr_route_params(ix, P);  // before the launch configuration
   if (ix->params.r_max <= 0) {  // threshold enumeration
     const size_t smem = nrq::route_block_bytes(P, rpb.nonempty, rpb.Q);
-    cudaError_t e = cudaFuncSetAttribute(route_block_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // Few queries leave SMs to themselves: wider blocks take the walk's and the
+    // ranking's strides together (one query at P = 1024 18.5 -> 14.5 us, at P =
+    // 64 no change; past one block an SM the narrow ones overlap better).
+    const bool few = nq <= ix->num_sms;
+    const auto kern = few ? route_block_kernel<nrq::kRouteFewThreads> : route_block_kernel<nrq::kRouteThreads>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    route_block_kernel<<<(unsigned)nq, nrq::kRouteThreads, smem, s>>>(rpb, d_logits, nq, d_codes,
-                                                                       d_nprobe);
+    kern<<<(unsigned)nq, few ? nrq::kRouteFewThreads : nrq::kRouteThreads, smem, s>>>(rpb, d_logits, nq,
+                                                                                     d_codes, d_nprobe);
     ix->launches += 1;
     return cudaGetLastError();
   }

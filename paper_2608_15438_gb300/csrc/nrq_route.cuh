@@ -222,6 +222,7 @@ __device__ __forceinline__ int route_warp(const RouteParams &rp, const float *__
 // filter, a subtree beyond its capacity of 2N keys, or a bucket above
 // kRouteBucketMax keys take route_warp too (warp 0 of the block).
 constexpr int kRouteThreads = 128;
+constexpr int kRouteFewThreads = 512;      // a block's threads where there are few queries
 constexpr int kRouteBins = 480;
 constexpr int kRouteSeedRanks = 7;          // the walk starts from all subsets of ranks 0..6
 constexpr int kRouteDp = kRouteBins + 32;  // sums of rounded-up steps overshoot by < 1 per rank
@@ -252,7 +253,7 @@ struct RouteSmem {
   float *ssd;       // deviation of rank r
   int *bitidx;      // bit index of rank r
   int *ctl;         // [0] tail, [1] chosen bin, [2] u0, [3] route_warp's count, [4] largest
-                    // cost bits, [5] largest bucket, [6] base code occupied, [8..11] warp totals
+                    // cost bits, [5] largest bucket, [6] base code occupied, [8..23] warp totals
 };
 
 __host__ __device__ inline size_t route_region_bytes(int N, int Q) {
@@ -265,7 +266,7 @@ __host__ __device__ inline size_t route_region_bytes(int N, int Q) {
 __host__ __device__ inline size_t route_block_bytes(int P, int nonempty, int Q) {
   const int N = route_enum_target(P, nonempty, Q);
   return route_region_bytes(N, Q) + (size_t)route_cap(N) * 4 * (nonempty ? 2 : 1) +
-         (size_t)2 * kRouteDp * 4 + (size_t)3 * 256 * 4 + 32 * 4 + 32 * 4 + 16 * 4;
+         (size_t)2 * kRouteDp * 4 + (size_t)3 * 256 * 4 + 32 * 4 + 32 * 4 + 24 * 4;
 }
 
 __device__ __forceinline__ RouteSmem route_carve(unsigned char *base, int N, int Q, int nonempty) {
@@ -287,7 +288,10 @@ __device__ __forceinline__ bool route_occupied(const RouteParams &rp, uint32_t c
 }
 
 // Writes codes[0..n) (any address space) and returns n, uniform in the block.
-// Called by the whole 128-thread block; smem: route_block_bytes(P, nonempty, Q) bytes.
+// Called by a whole block of NT threads, kRouteThreads or kRouteFewThreads (the
+// walk's order differs, the subtree and the ranks of its keys do not); smem:
+// route_block_bytes(P, nonempty, Q) bytes.
+template <int NT>
 __device__ __forceinline__ int route_block(const RouteParams &rp, const float *__restrict__ logit,
                                            unsigned char *smem, uint32_t *codes) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -326,7 +330,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
   __syncthreads();
   const uint32_t u0 = (uint32_t)m.ctl[2];
   // flip[t][v] = the bits of the ranks 8t + i, i in v (ApplyFlips by bytes)
-  for (int e = tid; e < 3 * 256; e += kRouteThreads) {
+  for (int e = tid; e < 3 * 256; e += NT) {
     const int t = e >> 8, v = e & 255;
     uint32_t f = 0;
     for (int i = 0; i < 8; ++i)
@@ -350,7 +354,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
       // kRouteDp) the 0.001 covers, so s_r D >= delta_r exactly
       const float step = __fdiv_rn(trange, (float)kRouteBins);
       uint32_t *d0 = m.dp, *d1 = m.dp + kRouteDp;
-      for (int c = tid; c < kRouteDp; c += kRouteThreads) d0[c] = 0u;
+      for (int c = tid; c < kRouteDp; c += NT) d0[c] = 0u;
       // the counts over the first ranks in one step: each subset of ranks
       // 0 .. r0 - 1 (those that fit a bin, at most kRouteSeedRanks) adds one
       // to the bin of its sum of steps, as the passes below would
@@ -380,7 +384,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
         const float qv = __fdiv_rn(m.ssd[r], step);
         if (!(qv < (float)(kRouteDp - 2))) break;  // this rank and all later ones fit no bin
         const int sr = (int)__fadd_rn(qv, 0.001f) + 1;
-        for (int c = tid; c < kRouteDp; c += kRouteThreads) d1[c] = d0[c] + (c >= sr ? d0[c - sr] : 0u);
+        for (int c = tid; c < kRouteDp; c += NT) d1[c] = d0[c] + (c >= sr ? d0[c - sr] : 0u);
         __syncthreads();
         uint32_t *t = d0;
         d0 = d1;
@@ -453,7 +457,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
     tail = m.ctl[0];
     __syncthreads();  // every thread has read the tail before the first appends
     while (head < tail && tail <= cap) {
-      const int nb = min(tail - head, kRouteThreads);
+      const int nb = min(tail - head, NT);
       uint64_t k1 = kEmpty, k2 = kEmpty;
       float p1 = 0.0f, p2 = 0.0f;
       if (tid < nb) {
@@ -511,22 +515,22 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
   if (!use_heap && tail > 0) {
     // bucket histogram over [0, largest cost]; costs are non-negative, so
     // their bits order as their values
-    for (int i = tid; i < kRouteBuckets; i += kRouteThreads) hist[i] = 0u;
+    for (int i = tid; i < kRouteBuckets; i += NT) hist[i] = 0u;
     uint32_t cmax = 0u;
-    for (int i = tid; i < tail; i += kRouteThreads) cmax = max(cmax, (uint32_t)(m.keys[i] >> 32));
+    for (int i = tid; i < tail; i += NT) cmax = max(cmax, (uint32_t)(m.keys[i] >> 32));
     cmax = __reduce_max_sync(kFull, cmax);
     if (lane == 0) atomicMax(reinterpret_cast<unsigned *>(&m.ctl[4]), cmax);
     __syncthreads();
     const float top = __uint_as_float((uint32_t)m.ctl[4]);
     if (top > 0.0f && top < __int_as_float(0x7f800000))
       scale = __fdiv_rn((float)kRouteBuckets, top);
-    for (int i = tid; i < tail; i += kRouteThreads) {
+    for (int i = tid; i < tail; i += NT) {
       const float cost = __uint_as_float((uint32_t)(m.keys[i] >> 32));
       atomicAdd(&hist[min(kRouteBuckets - 1, (int)__fmul_rn(cost, scale))], 1u);
     }
     __syncthreads();
     uint32_t bmax = 0u;
-    for (int i = tid; i < kRouteBuckets; i += kRouteThreads) bmax = max(bmax, hist[i]);
+    for (int i = tid; i < kRouteBuckets; i += NT) bmax = max(bmax, hist[i]);
     bmax = __reduce_max_sync(kFull, bmax);
     if (lane == 0) atomicMax(reinterpret_cast<unsigned *>(&m.ctl[5]), bmax);
     __syncthreads();
@@ -535,10 +539,10 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
   int nlist = 0;  // codes listed (uniform)
   if (!use_heap) {
     if (tail > 0) {
-      // bucket ranges: an exclusive scan of the histogram (kRouteBuckets /
-      // 128 buckets a thread), then a scatter in which each key takes the
+      // bucket ranges: an exclusive scan of the histogram (kRouteBuckets / NT
+      // buckets a thread), then a scatter in which each key takes the
       // next slot of its bucket, leaving hist[z] = the end of bucket z
-      constexpr int per = kRouteBuckets / kRouteThreads;
+      constexpr int per = kRouteBuckets / NT;
       uint32_t loc[per], sum = 0;
 #pragma unroll
       for (int e = 0; e < per; ++e) {
@@ -550,7 +554,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
         const uint32_t v = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += v;
       }
-      uint32_t *wsum = reinterpret_cast<uint32_t *>(m.ctl + 8);  // 4 warp totals
+      uint32_t *wsum = reinterpret_cast<uint32_t *>(m.ctl + 8);  // warp totals
       if (lane == 31) wsum[warp] = incl;
       __syncthreads();
       uint32_t run = incl - sum;
@@ -561,7 +565,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
         run += loc[e];
       }
       __syncthreads();
-      for (int i = tid; i < tail; i += kRouteThreads) {
+      for (int i = tid; i < tail; i += NT) {
         const float cost = __uint_as_float((uint32_t)(m.keys[i] >> 32));
         const int z = min(kRouteBuckets - 1, (int)__fmul_rn(cost, scale));
         order[atomicAdd(&hist[z], 1u)] = i;
@@ -571,7 +575,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
     // rank of each key = its bucket's start + the smaller keys of its bucket;
     // its code is u0 XOR the flips of its rank mask
     const int nexam = rp.nonempty ? min(tail, rp.Q - 1) : min(tail, P - 1);
-    for (int i = tid; i < tail; i += kRouteThreads) {
+    for (int i = tid; i < tail; i += NT) {
       const uint64_t key = m.keys[i];
       const float cost = __uint_as_float((uint32_t)(key >> 32));
       const int z = min(kRouteBuckets - 1, (int)__fmul_rn(cost, scale));
@@ -594,7 +598,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
     // order, after the base code when it is non-empty
     __syncthreads();
     const int base_ne = m.ctl[6];
-    const int per = (nexam + kRouteThreads - 1) / kRouteThreads;
+    const int per = (nexam + NT - 1) / NT;
     const int r0 = min(nexam, tid * per), r1 = min(nexam, r0 + per);
     int cnt = 0;
     for (int r = r0; r < r1; ++r) cnt += (int)(m.rc[r] >> 31);
@@ -608,7 +612,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     int before = incl - cnt, total = 0;
-    for (int w = 0; w < 4; ++w) {
+    for (int w = 0; w < NT / 32; ++w) {
       before += w < warp ? wsum[w] : 0;
       total += wsum[w];
     }
