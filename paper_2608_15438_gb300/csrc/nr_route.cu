@@ -23,18 +23,46 @@ __global__ void route_kernel(nrq::RouteParams rp, const float *__restrict__ logi
   if (lane == 0) nprobe[q] = n;
 }
 
-// One block of NT threads per query: the threshold enumeration (route_block).
-template <int NT>
+// One block of NT threads per query: the threshold enumeration (route_block) of
+// N flip sets and, where a non-empty budget needs more, of N2 (0: the heap).
+// RETRY: the block has the shared memory for N2 and goes on itself; else the
+// query is left to route_more_kernel (nprobe -1).
+template <int NT, bool RETRY>
 __global__ void __launch_bounds__(NT) route_block_kernel(
     nrq::RouteParams rp, const float *__restrict__ logits, int64_t nq, uint32_t *__restrict__ codes,
-    int32_t *__restrict__ nprobe) {
+    int32_t *__restrict__ nprobe, int N, int N2) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t q = blockIdx.x;
   if (q >= nq) return;
   uint32_t *out = codes + (size_t)q * rp.P;
-  const int n = nrq::route_block<NT>(rp, logits + q * rp.b, smem, out);
-  for (int t = n + (int)threadIdx.x; t < rp.P; t += NT) out[t] = 0xffffffffu;
+  int n;
+  if constexpr (RETRY) {
+    for (bool more = true;; more = false) {
+      n = nrq::route_block<NT>(rp, logits + q * rp.b, smem, out, more ? N : N2, more);
+      if (n >= 0) break;
+      __syncthreads();
+    }
+  } else {
+    n = nrq::route_block<NT>(rp, logits + q * rp.b, smem, out, N, N2 > 0);
+  }
   if (threadIdx.x == 0) nprobe[q] = n;
+  if (n < 0) return;
+  for (int t = n + (int)threadIdx.x; t < rp.P; t += NT) out[t] = 0xffffffffu;
+}
+
+// The queries that route_block_kernel left, one block an SM.
+__global__ void __launch_bounds__(nrq::kRouteFewThreads) route_more_kernel(
+    nrq::RouteParams rp, const float *__restrict__ logits, int64_t nq, uint32_t *__restrict__ codes,
+    int32_t *__restrict__ nprobe, int N) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  for (int64_t q = blockIdx.x; q < nq; q += gridDim.x) {
+    if (nprobe[q] >= 0) continue;  // uniform: only this block writes it
+    uint32_t *out = codes + (size_t)q * rp.P;
+    const int n = nrq::route_block<nrq::kRouteFewThreads>(rp, logits + q * rp.b, smem, out, N, false);
+    for (int t = n + (int)threadIdx.x; t < rp.P; t += nrq::kRouteFewThreads) out[t] = 0xffffffffu;
+    __syncthreads();  // every thread has read nprobe[q] and the block's results
+    if (threadIdx.x == 0) nprobe[q] = n;
+  }
 }
 
 }  // namespace
@@ -61,16 +89,30 @@ cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int
   if (nq <= 0) return cudaSuccess;
   const nrq::RouteParams rpb = nr_route_params(ix, P);  // before the launch configuration
   if (ix->params.r_max <= 0) {  // threshold enumeration
-    const size_t smem = nrq::route_block_bytes(P, rpb.nonempty, rpb.Q);
     // Few queries leave SMs to themselves: wider blocks take the walk's and the
     // ranking's strides together (one query at P = 1024 18.5 -> 14.5 us, at P =
     // 64 no change; past one block an SM the narrow ones overlap better).
     const bool few = nq <= ix->num_sms;
-    const auto kern = few ? route_block_kernel<nrq::kRouteFewThreads> : route_block_kernel<nrq::kRouteThreads>;
+    // Non-empty budgets: 2 P flip sets first, which three blocks an SM hold at P
+    // = 1024; where less than half of the buckets are occupied, all 4 P that may
+    // be examined, by the same block or, with many queries, a second kernel (the
+    // heap, one flip set after another: 3,230 us for 100 queries at P = 1024).
+    const int N = nrq::route_enum_target(P, rpb.nonempty, rpb.Q);
+    const int N2 = nrq::route_enum_more(P, rpb.nonempty, rpb.Q);
+    const size_t smem2 = N2 > 0 ? nrq::route_block_bytes(N2, rpb.nonempty, rpb.Q) : 0;
+    const size_t smem = few && N2 > 0 ? smem2 : nrq::route_block_bytes(N, rpb.nonempty, rpb.Q);
+    constexpr int kFew = nrq::kRouteFewThreads, kMany = nrq::kRouteThreads;
+    const auto kern = !few ? route_block_kernel<kMany, false>
+                           : N2 > 0 ? route_block_kernel<kFew, true> : route_block_kernel<kFew, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nq, few ? nrq::kRouteFewThreads : nrq::kRouteThreads, smem, s>>>(rpb, d_logits, nq,
-                                                                                     d_codes, d_nprobe);
+    kern<<<(unsigned)nq, few ? kFew : kMany, smem, s>>>(rpb, d_logits, nq, d_codes, d_nprobe, N, N2);
+    ix->launches += 1;
+    if (few || N2 == 0) return cudaGetLastError();
+    e = cudaFuncSetAttribute(route_more_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+    if (e != cudaSuccess) return e;
+    route_more_kernel<<<(unsigned)ix->num_sms, nrq::kRouteFewThreads, smem2, s>>>(rpb, d_logits, nq, d_codes,
+                                                                                 d_nprobe, N2);
     ix->launches += 1;
     return cudaGetLastError();
   }

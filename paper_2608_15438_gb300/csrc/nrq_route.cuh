@@ -217,8 +217,8 @@ __device__ __forceinline__ int route_warp(const RouteParams &rp, const float *__
 // min(N, Q) in key order is looked up (all lookups in flight at once), and a
 // scan over them in rank order lists the first P non-empty codes. When that
 // prefix holds fewer than P non-empty codes while more flip sets may be
-// examined (fewer than Q examined, and sets above T remain), the block takes
-// route_warp instead. Keys, ties and codes are those of route_warp; the R_max
+// examined (fewer than Q examined, and sets above T remain), an enumeration of
+// all Q decides it where it fits (Q <= kRouteMoreMax), else route_warp. Keys, ties and codes are those of route_warp; the R_max
 // filter, a subtree beyond its capacity of 2N keys, or a bucket above
 // kRouteBucketMax keys take route_warp too (warp 0 of the block).
 constexpr int kRouteThreads = 128;
@@ -237,6 +237,12 @@ __host__ __device__ inline int route_enum_target(int P, int nonempty, int Q) {
   if (!nonempty) return P;
   int n = 2 * P < Q ? 2 * P : Q;
   return n < kRouteNonemptyMax ? n : kRouteNonemptyMax;
+}
+// Flip sets of a second, larger enumeration for the non-empty budget: all Q that
+// may be examined, where a block's shared memory holds them (else none).
+constexpr int kRouteMoreMax = 6144;
+__host__ __device__ inline int route_enum_more(int P, int nonempty, int Q) {
+  return nonempty && Q <= kRouteMoreMax && Q > route_enum_target(P, nonempty, Q) ? Q : 0;
 }
 // Subtree capacity for an enumeration of N: 2N keys, a whole number of block strides.
 __host__ __device__ inline int route_cap(int N) {
@@ -262,9 +268,8 @@ __host__ __device__ inline size_t route_region_bytes(int N, int Q) {
   return ((keys > heap ? keys : heap) + 15) & ~(size_t)15;
 }
 
-// Shared memory of route_block for probe budget P (Q: route_warp's limit).
-__host__ __device__ inline size_t route_block_bytes(int P, int nonempty, int Q) {
-  const int N = route_enum_target(P, nonempty, Q);
+// Shared memory of route_block for an enumeration of N (Q: route_warp's limit).
+__host__ __device__ inline size_t route_block_bytes(int N, int nonempty, int Q) {
   return route_region_bytes(N, Q) + (size_t)route_cap(N) * 4 * (nonempty ? 2 : 1) +
          (size_t)2 * kRouteDp * 4 + (size_t)3 * 256 * 4 + 32 * 4 + 32 * 4 + 24 * 4;
 }
@@ -289,14 +294,15 @@ __device__ __forceinline__ bool route_occupied(const RouteParams &rp, uint32_t c
 
 // Writes codes[0..n) (any address space) and returns n, uniform in the block.
 // Called by a whole block of NT threads, kRouteThreads or kRouteFewThreads (the
-// walk's order differs, the subtree and the ranks of its keys do not); smem:
-// route_block_bytes(P, nonempty, Q) bytes.
+// walk's order differs, the subtree and the ranks of its keys do not). N: flip
+// sets to enumerate; more: with a non-empty budget that they do not decide,
+// return -1 instead of going on with the heap. smem: route_block_bytes(N,
+// nonempty, Q) bytes.
 template <int NT>
 __device__ __forceinline__ int route_block(const RouteParams &rp, const float *__restrict__ logit,
-                                           unsigned char *smem, uint32_t *codes) {
+                                           unsigned char *smem, uint32_t *codes, int N, bool more) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = rp.b, bsel = rp.bsel, P = rp.P;
-  const int N = route_enum_target(P, rp.nonempty, rp.Q);
   const int cap = route_cap(N);
   const RouteSmem m = route_carve(smem, N, rp.Q, rp.nonempty);
   if (warp == 0) {  // deviations, base code and ranks (Eq. 10, Sec. 3.2.3)
@@ -617,7 +623,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
       total += wsum[w];
     }
     // fewer than P non-empty codes, fewer than Q flip sets examined and sets
-    // above the enumerated cost left: the heap continues where this stopped
+    // above the enumerated cost left: a larger enumeration or the heap decides
     const bool complete = tail >= rp.Q - 1 || !(T < rp.smax);
     if (base_ne + total >= P || complete) {
       if (tid == 0 && base_ne) codes[0] = u0;
@@ -626,6 +632,7 @@ __device__ __forceinline__ int route_block(const RouteParams &rp, const float *_
         if (m.rc[r] >> 31) codes[pos++] = m.rc[r] & 0x7fffffffu;
       return min(P, base_ne + total);
     }
+    if (more) return -1;
     use_heap = true;  // uniform
   }
   __syncthreads();
