@@ -90,13 +90,15 @@ cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int
   const nrq::RouteParams rpb = nr_route_params(ix, P);  // before the launch configuration
   if (ix->params.r_max <= 0) {  // threshold enumeration
     // Few queries leave SMs to themselves: wider blocks take the walk's and the
-    // ranking's strides together (one query at P = 1024 18.5 -> 14.5 us, at P =
-    // 64 no change; past one block an SM the narrow ones overlap better).
+    // ranking's strides together (the stage of one query at P = 1024 22 -> 18 us,
+    // four 1536-value ones 20 -> 16; at P = 64 14 both; past one block an SM the
+    // narrow ones overlap).
     const bool few = nq <= ix->num_sms;
     // Non-empty budgets: 2 P flip sets first, which three blocks an SM hold at P
     // = 1024; where less than half of the buckets are occupied, all 4 P that may
-    // be examined, by the same block or, with many queries, a second kernel (the
-    // heap, one flip set after another: 3,230 us for 100 queries at P = 1024).
+    // be examined, by the same block or, with many queries, a second kernel (100
+    // queries at P = 1024, 1e7 rows: 61 us, 3,220 by the heap, one flip set after
+    // another; 3,000 queries 808 and 13,280).
     const int N = nrq::route_enum_target(P, rpb.nonempty, rpb.Q);
     const int N2 = nrq::route_enum_more(P, rpb.nonempty, rpb.Q);
     const size_t smem2 = N2 > 0 ? nrq::route_block_bytes(N2, rpb.nonempty, rpb.Q) : 0;
