@@ -875,7 +875,8 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
       if (e != cudaSuccess) break;
     }
     ev = tstart(1, sa);
-    e = nr_launch_route(ix, lg, n, P, (uint32_t *)(cw + l.codes), (int32_t *)(cw + l.nprobe), sa);
+    e = nr_launch_route(ix, lg, n, P, (uint32_t *)(cw + l.codes), (int32_t *)(cw + l.nprobe), sa,
+                        !d_logits_in);
     tend(ev, sa);
     if (e != cudaSuccess) break;
     ev = tstart(2, sa);
@@ -883,7 +884,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
                          (int32_t *)(cw + l.L), (int32_t *)(cw + l.nL), (nr_seg *)(cw + l.seg),
                          (uint32_t *)(cw + l.slen), stats + q0 * NR_QSTATS,
                          nr_select_slab_bytes(P, ix->K_max) ? cw + l.slab : nullptr,
-                         nr_refine_zero(n, k, cw + l.refine, l.total - l.refine), sa);
+                         nr_refine_zero(n, k, cw + l.refine, l.total - l.refine), sa, true);
     tend(ev, sa);
     if (e != cudaSuccess) break;
     if (pipe) {
@@ -895,7 +896,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     e = nr_launch_refine(ix, qp, n, k, P + C, (nr_seg *)(cw + l.seg), (int32_t *)(cw + l.nL),
                          (uint32_t *)(cw + l.slen), (uint32_t *)(cw + l.codes), P, d_ids + q0 * k,
                          d_d + q0 * k, stats + q0 * NR_QSTATS,
-                         cw + l.refine, l.total - l.refine, sb);
+                         cw + l.refine, l.total - l.refine, sb, !pipe);
     tend(ev, sb);
     if (pipe && e == cudaSuccess) e = cudaEventRecord(ps.ref[slot], sb);
   }

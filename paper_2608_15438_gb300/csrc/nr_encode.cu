@@ -427,6 +427,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                      const __half *__restrict__ W2p, const float *__restrict__ b2, int64_t nq,
                      float *__restrict__ out, int *err, int64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
+  nr_let_next();
   const TcLayout L = tc_layout(D, H, n2, nxb);
   TcBars &B = *reinterpret_cast<TcBars *>(smem + L.bars);
   volatile int *abort = &B.abort;
@@ -774,6 +775,8 @@ __global__ void __launch_bounds__(kLyThreads, 1)
                         void *__restrict__ y, int nraw, int box, const __grid_constant__ CUtensorMap tmx,
                         int *err, int64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char smem[];
+  nr_let_next();
+  nr_after_previous();
   const uint32_t stage_b = ly_stage_bytes(Nt);
   LyBars &B = *reinterpret_cast<LyBars *>(smem + kLyStages * stage_b);
   // raw stages (XT 1): nraw x 32 KB from the first 1024-byte boundary after the bars
@@ -1292,11 +1295,11 @@ static cudaError_t launch_layer(nr_index *ix, const void *x, int K, int N, int l
   if (e != cudaSuccess) return e;
   const int64_t items = (n + kRows - 1) / kRows * (Np / nt);
   const int64_t grid = items < ix->num_sms ? items : ix->num_sms;
-  kern<<<(unsigned)grid, kLyThreads, smem, s>>>(x, K, N, nt, nw, Np, sc,
-                                                static_cast<const __half *>(ix->Wl) + ix->ly_off[l],
-                                                bias, n, y, nraw, rbox, tm, ix->d_err, wait_ns);
+  e = nr_launch_kernel(kern, (unsigned)grid, kLyThreads, smem, s, l > 0 && n <= 8 * kRows, x, K, N, nt, nw, Np, sc,
+                       static_cast<const __half *>(ix->Wl) + ix->ly_off[l], bias, n, y, nraw, rbox, tm,
+                       ix->d_err, wait_ns);
   ix->launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 // An encoder with hidden layers after the first, layer by layer on tensor

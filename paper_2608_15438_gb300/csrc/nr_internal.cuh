@@ -138,6 +138,34 @@ size_t nr_mid_floats(const nr_index *ix);
 
 // kernel launchers (each returns cudaGetLastError() after the launch)
 bool nr_encode_uses_tensor_cores(const nr_index *ix);
+// A chain of small launches: each kernel lets the next one's blocks come onto
+// the SMs beside its own (nr_let_next) and waits itself, before it touches
+// memory, until the launch before it has completed (nr_after_previous; both do
+// nothing in launches that are not early). Hides the start of a launch: one
+// query 61 -> 59 us, at P = 1024 90.5 -> 86, four 1536-value queries 246 -> 238.
+// Larger batches launch as before: their blocks leave no room beside them.
+__device__ __forceinline__ void nr_let_next() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+__device__ __forceinline__ void nr_after_previous() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+// early: the launch before on the stream is a kernel of the same call
+template <class... Param, class... Arg>
+cudaError_t nr_launch_kernel(void (*kern)(Param...), unsigned grid, unsigned block, size_t smem,
+                             cudaStream_t s, bool early, const Arg &...arg) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kern, static_cast<Param>(arg)...);
+}
 // device scratch an encode of n rows needs (the activations of an encoder
 // with several hidden layers on tensor cores), 0 when none
 size_t nr_encode_scratch_bytes(const nr_index *ix, int64_t n);
@@ -146,7 +174,7 @@ size_t nr_encode_scratch_bytes(const nr_index *ix, int64_t n);
 cudaError_t nr_launch_encode(nr_index *ix, const void *d_x, int64_t nq, float *d_logits,
                              cudaStream_t s, void *scratch = nullptr);
 cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int P,
-                            uint32_t *d_codes, int32_t *d_nprobe, cudaStream_t s);
+                            uint32_t *d_codes, int32_t *d_nprobe, cudaStream_t s, bool early = false);
 // dynamic shared memory of the select kernel for budgets (P, C) under the
 // index's current parameters
 size_t nr_select_smem_bytes(const nr_index *ix, int P, int C);
@@ -164,7 +192,7 @@ struct nr_zero {
 cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t *d_codes,
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
-                             void *d_slab, nr_zero zero, cudaStream_t s);
+                             void *d_slab, nr_zero zero, cudaStream_t s, bool early = false);
 // the flags of a refine launch's scratch that have to be zero: the select
 // launch before it clears them
 nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes);
@@ -177,4 +205,5 @@ size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least);
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
                              const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
-                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s);
+                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s,
+                             bool early = false);

@@ -235,6 +235,7 @@ enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlRun, kCtlHn, kCtlRounds
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
+  nr_after_previous();
   const int tid = threadIdx.x, lane = tid & 31;
   const int k = a.rf.k;
   const nrq::RefineSmem m = nrq::refine_carve<TR, KCC, ST>(smem, a.row_bytes, k);
@@ -467,7 +468,7 @@ bool whole_streams(int64_t nq, int64_t grid, int t_low, bool long_rows) {
 }
 
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
-cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s) {
+cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s, bool early) {
   const size_t smem = nrq::refine_smem_bytes<TR, KCC, ST>(a.row_bytes, a.rf.k);
   auto kern = refine_kernel<DT, TR, CPR, KCC, ST, MINB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -498,9 +499,9 @@ cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t 
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  kern<<<(unsigned)grid, TR, smem, s>>>(a);
+  e = nr_launch_kernel(kern, (unsigned)grid, TR, smem, s, early && a.own_plan, a);
   ix->launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 nrq::RefineParams refine_params(const nr_index *ix, int k) {
@@ -574,7 +575,8 @@ nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes) {
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
                              const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
-                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s) {
+                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s,
+                             bool early) {
   if (nq <= 0) return cudaSuccess;
   char *w = static_cast<char *>(d_scratch);
   const int64_t items = span_items(nq), entries = span_entries(nq, k);
@@ -614,16 +616,16 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   pa.pre = reinterpret_cast<uint32_t *>(w + l.pre);
   pa.perm = reinterpret_cast<int32_t *>(w + l.perm);
   if (ix->dtype == 0) {
-    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s);  // uint8, D = 128
-    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s);
-    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s);
+    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s, early);  // uint8, D = 128
+    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s, early);
+    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s, early);
   }
   if (ix->row_bytes > 1024) {  // fp32, D above 256: rows staged in pieces
-    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s);
-    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s);
-    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s);  // row_bytes % 64 == 0 (load check)
+    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s, early);
+    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s, early);
+    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s, early);  // row_bytes % 64 == 0 (load check)
   }
-  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s);  // fp32, D = 96
-  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s);
-  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s);
+  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s, early);  // fp32, D = 96
+  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s, early);
+  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s, early);
 }

@@ -32,6 +32,8 @@ __global__ void __launch_bounds__(NT) route_block_kernel(
     nrq::RouteParams rp, const float *__restrict__ logits, int64_t nq, uint32_t *__restrict__ codes,
     int32_t *__restrict__ nprobe, int N, int N2) {
   extern __shared__ __align__(16) unsigned char smem[];
+  nr_let_next();
+  nr_after_previous();
   const int64_t q = blockIdx.x;
   if (q >= nq) return;
   uint32_t *out = codes + (size_t)q * rp.P;
@@ -85,7 +87,7 @@ nrq::RouteParams nr_route_params(const nr_index *ix, int P) {
 size_t nr_route_heap_bytes(int Q) { return nrq::route_heap_bytes(Q); }
 
 cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int P,
-                            uint32_t *d_codes, int32_t *d_nprobe, cudaStream_t s) {
+                            uint32_t *d_codes, int32_t *d_nprobe, cudaStream_t s, bool early) {
   if (nq <= 0) return cudaSuccess;
   const nrq::RouteParams rpb = nr_route_params(ix, P);  // before the launch configuration
   if (ix->params.r_max <= 0) {  // threshold enumeration
@@ -108,9 +110,10 @@ cudaError_t nr_launch_route(nr_index *ix, const float *d_logits, int64_t nq, int
                            : N2 > 0 ? route_block_kernel<kFew, true> : route_block_kernel<kFew, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nq, few ? kFew : kMany, smem, s>>>(rpb, d_logits, nq, d_codes, d_nprobe, N, N2);
+    e = nr_launch_kernel(kern, (unsigned)nq, few ? kFew : kMany, smem, s, early && few, rpb, d_logits, nq, d_codes,
+                         d_nprobe, N, N2);
     ix->launches += 1;
-    if (few || N2 == 0) return cudaGetLastError();
+    if (few || N2 == 0 || e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(route_more_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
     if (e != cudaSuccess) return e;
     route_more_kernel<<<(unsigned)ix->num_sms, nrq::kRouteFewThreads, smem2, s>>>(rpb, d_logits, nq, d_codes,

@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(NT, MODE == 1 ? 3 : NT == kThreads ? 6 : 1)
                   int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen, int64_t *stats,
                   unsigned char *slab, size_t slab_bytes, unsigned *ovf, nr_zero zero) {
   extern __shared__ __align__(16) unsigned char smem[];
+  nr_let_next();
+  nr_after_previous();
   const int q = blockIdx.x, tid = threadIdx.x;
   // the block's share of the refinement's flags (in place of a memset between
   // the kernels)
@@ -201,7 +203,7 @@ size_t nr_select_smem_bytes(const nr_index *ix, int P, int C) { return select_sm
 cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t *d_codes,
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
-                             void *d_slab, nr_zero zero, cudaStream_t s) {
+                             void *d_slab, nr_zero zero, cudaStream_t s, bool early) {
   if (nq <= 0) return cudaSuccess;
   const nrq::SelectParams sp = nr_select_params(ix, P, C);  // before the launch configuration
   const size_t slab_bytes = nrq::select_slab_bytes(P, ix->K_max);
@@ -224,11 +226,10 @@ cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t
   auto kern = sp.mode == 1 ? select_kernel<1, kThreads> : few ? select_kernel<0, kFewThreads> : select_kernel<0, kThreads>;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)nq, nt, smem, s>>>(sp, d_logits, d_codes, d_nprobe, d_L, d_nL, d_seg, d_slen, d_stats,
-                                      slab, slab_bytes, ovf, zero);
+  e = nr_launch_kernel(kern, (unsigned)nq, nt, smem, s, early && few, sp, d_logits, d_codes, d_nprobe, d_L, d_nL,
+                       d_seg, d_slen, d_stats, slab, slab_bytes, ovf, zero);
   if (sp.mode == 0) {
     ix->launches += 1;
-    e = cudaGetLastError();
     if (e != cudaSuccess || !ovf) return e;
     // the deferred queries (none at most budgets: its blocks exit at once)
     const size_t osm = nrq::select_overflow_smem_bytes();

@@ -101,17 +101,17 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   // refinement's flags, which its launcher clears on the stream
   cudaError_t e = nr_launch_encode(ix, d_queries, nq, logits, s, w + o_enc);
   if (e == cudaSuccess)
-    e = nr_launch_route(ix, logits, nq, P, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), s);
+    e = nr_launch_route(ix, logits, nq, P, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), s, true);
   if (e == cudaSuccess)
     e = nr_launch_select(ix, logits, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), nq, P, C,
                          (int32_t *)(w + o_L), (int32_t *)(w + o_nL), (nr_seg *)(w + o_seg),
                          (uint32_t *)(w + o_slen), stats, slab_q ? w + o_slab : nullptr,
-                         nr_refine_zero(nq, k, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine), s);
+                         nr_refine_zero(nq, k, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine), s, true);
   if (e == cudaSuccess)
     e = nr_launch_refine(ix, d_queries, nq, k, (int)Lmax, (nr_seg *)(w + o_seg),
                          (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), (uint32_t *)(w + o_codes), P,
                          d_out_ids, d_out_dists,
-                         stats, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine, s);
+                         stats, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine, s, true);
   // statistics of this call are read from the array by nr_last_stats / nr_query_stats
   ix->d_stats = stats;
   ix->last_nq = nq;
