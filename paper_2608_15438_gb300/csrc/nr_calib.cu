@@ -72,6 +72,7 @@ struct LocateArgs {
   const uint32_t *small, *large;  // the filters, or null
   uint32_t mask;                  // of the large one
   int32_t *out;
+  bool vec_out;                   // out is 16-byte aligned: a request is one store
 };
 
 // the requests of stored row p, whose id is `id`: its cluster and bucket
@@ -97,9 +98,17 @@ __device__ __forceinline__ void locate_row(const LocateArgs &a, int64_t p, uint3
     else w = mid - 1;
   }
   const uint32_t f = a.bkt_off[u], e = a.bkt_off[u + 1];
-  for (int64_t t = lo; t < a.n && a.skeys[t] == id; ++t)
-    *reinterpret_cast<int4 *>(a.out + (size_t)a.sidx[t] * 4) =
-        make_int4((int)c, (int)u, (int)f, (int)(e - f));
+  for (int64_t t = lo; t < a.n && a.skeys[t] == id; ++t) {
+    int32_t *o = a.out + (size_t)a.sidx[t] * 4;
+    if (a.vec_out) {
+      *reinterpret_cast<int4 *>(o) = make_int4((int)c, (int)u, (int)f, (int)(e - f));
+    } else {
+      o[0] = (int32_t)c;
+      o[1] = (int32_t)u;
+      o[2] = (int32_t)f;
+      o[3] = (int32_t)(e - f);
+    }
+  }
 }
 
 // every stored row: if its id is requested, record its cluster and bucket for
@@ -312,7 +321,8 @@ nr_status nr_index_locate(nr_index *ix, const int64_t *d_ids, int64_t n, int32_t
     e = cub::DeviceRadixSort::SortPairs(mem + 4 * vb + fb, tb, keys, skeys, idx, sidx, n, 0, 32, s);
   if (e == cudaSuccess) {
     const LocateArgs a = {ix->ids, ix->N, ix->cl_off, ix->n_cl, ix->bkt_off, ix->b,
-                          skeys,   sidx,  n,          small,    large,       fbits - 1, d_out};
+                          skeys,   sidx,  n,          small,    large,       fbits - 1, d_out,
+                          (reinterpret_cast<uintptr_t>(d_out) & 15) == 0};
     locate_kernel<<<grid_for(ix->N, sms), 256, 0, s>>>(a);
     e = cudaGetLastError();
   }

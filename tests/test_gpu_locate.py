@@ -33,3 +33,22 @@ def test_locate_matches_the_stored_order(tmp_path, n):
     exp = np.stack([c, u, first, last - first], 1)
     exp[~ok] = (-1, -1, -1, 0)
     assert np.array_equal(got, exp)
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_locate_into_a_buffer_at_any_int32(tmp_path, offset):
+    """d_out need be no more aligned than int32; nothing beside it is written."""
+    torch = need_cuda()
+    from paper_2608_15438_gb300 import neuroute as nr
+
+    path, _, _ = build_small(tmp_path, "tiny", n=30_000, bits=10, name="loc")
+    ix = nr.Index(path, 0)
+    ids = torch.randint(-10, 30_010, (5_000,), device="cuda")
+    exp = ix.locate(ids)
+    buf = torch.full((5_000 * 4 + 4,), 7, dtype=torch.int32, device="cuda")
+    assert buf.data_ptr() % 16 == 0
+    out = buf[offset:offset + 5_000 * 4]
+    assert nr.lib().nr_index_locate(ix.h, ids.data_ptr(), 5_000, out.data_ptr(), None) == 0
+    ix.close()
+    assert torch.equal(out.view(-1, 4), exp)
+    assert buf[:offset].eq(7).all() and buf[offset + 5_000 * 4:].eq(7).all()
