@@ -768,9 +768,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm,
 // than it, one after the other in a stored tile (eight-row groups of its core
 // matrices), on more CTAs. box: rows of a tensor copy (XT 1). A tile's sums do
 // not depend on its width, nor on rows that are not there.
+// (x is not __restrict__: an early launch begins while the layer before writes it.)
 template <int XT, int YF>
 __global__ void __launch_bounds__(kLyThreads, 1)
-    encode_layer_kernel(const void *__restrict__ x, int K, int N, int Nt, int Nw, int Npad, float s,
+    encode_layer_kernel(const void *x, int K, int N, int Nt, int Nw, int Npad, float s,
                         const __half *__restrict__ Wp, const float *__restrict__ bias, int64_t n,
                         void *__restrict__ y, int nraw, int box, const __grid_constant__ CUtensorMap tmx,
                         int *err, int64_t wait_ns) {

@@ -27,10 +27,12 @@ __global__ void route_kernel(nrq::RouteParams rp, const float *__restrict__ logi
 // N flip sets and, where a non-empty budget needs more, of N2 (0: the heap).
 // RETRY: the block has the shared memory for N2 and goes on itself; else the
 // query is left to route_more_kernel (nprobe -1).
+// logits are not __restrict__: an early launch begins while the encoder still
+// writes them, and loads of such data may not take the read-only path.
 template <int NT, bool RETRY>
-__global__ void __launch_bounds__(NT) route_block_kernel(
-    nrq::RouteParams rp, const float *__restrict__ logits, int64_t nq, uint32_t *__restrict__ codes,
-    int32_t *__restrict__ nprobe, int N, int N2) {
+__global__ void __launch_bounds__(NT) route_block_kernel(nrq::RouteParams rp, const float *logits,
+                                                         int64_t nq, uint32_t *codes,
+                                                         int32_t *nprobe, int N, int N2) {
   extern __shared__ __align__(16) unsigned char smem[];
   nr_let_next();
   nr_after_previous();

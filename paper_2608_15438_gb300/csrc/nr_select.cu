@@ -48,11 +48,13 @@ __device__ __forceinline__ OverflowSmem overflow_carve(unsigned char *smem) {
 }
 
 // MODE 0: the order-independent stage; MODE 1: the sequential stage
+// logits, codes and nprobe are not __restrict__: an early launch begins while
+// the kernels that write them still run, and loads of data that is written in a
+// kernel's lifetime may not take the read-only path.
 template <int MODE, int NT>
 __global__ void __launch_bounds__(NT, MODE == 1 ? 3 : NT == kThreads ? 6 : 1)
-    select_kernel(nrq::SelectParams sp, const float *__restrict__ logits,
-                  const uint32_t *__restrict__ codes, const int32_t *__restrict__ nprobe,
-                  int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen, int64_t *stats,
+    select_kernel(nrq::SelectParams sp, const float *logits, const uint32_t *codes,
+                  const int32_t *nprobe, int32_t *L, int32_t *nL, nr_seg *seg, uint32_t *slen, int64_t *stats,
                   unsigned char *slab, size_t slab_bytes, unsigned *ovf, nr_zero zero) {
   extern __shared__ __align__(16) unsigned char smem[];
   nr_let_next();

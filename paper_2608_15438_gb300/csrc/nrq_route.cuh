@@ -45,7 +45,7 @@ __host__ __device__ inline size_t route_heap_bytes(int Q) { return (size_t)(Q + 
 // Writes codes[0..n) (any address space) and returns n, uniform in the warp.
 // Must be called by a whole warp. heap: route_heap_bytes(P) bytes of shared
 // memory (8-byte aligned).
-__device__ __forceinline__ int route_warp(const RouteParams &rp, const float *__restrict__ logit,
+__device__ __forceinline__ int route_warp(const RouteParams &rp, const float *logit,
                                           unsigned char *heap, uint32_t *codes) {
   const int lane = threadIdx.x & 31;
   const int b = rp.b;
@@ -299,7 +299,7 @@ __device__ __forceinline__ bool route_occupied(const RouteParams &rp, uint32_t c
 // return -1 instead of going on with the heap. smem: route_block_bytes(N,
 // nonempty, Q) bytes.
 template <int NT>
-__device__ __forceinline__ int route_block(const RouteParams &rp, const float *__restrict__ logit,
+__device__ __forceinline__ int route_block(const RouteParams &rp, const float *logit,
                                            unsigned char *smem, uint32_t *codes, int N, bool more) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = rp.b, bsel = rp.bsel, P = rp.P;
