@@ -788,6 +788,9 @@ __device__ __forceinline__ bool commit_warp(const RefineParams &a, const RefineS
     uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);  // smallest key, first block
     if (logged) h = __ldcg(reinterpret_cast<const uint4 *>(hdr + x));
     const uint64_t mk = ((uint64_t)h.y << 32) | h.x;
+    // each lane has acquired its own span's flag; the lanes copy one another's
+    // logs below, and votes and shuffles order no memory
+    __syncwarp();
     const unsigned idle = __ballot_sync(kFull, rdy == 0u || rdy == kSpanRedo);
     const int nb = idle ? __ffs(idle) - 1 : 32;  // finished spans of this batch
     redo = nb < 32 && __shfl_sync(kFull, rdy, nb & 31) == kSpanRedo;

@@ -61,3 +61,29 @@ def test_captured_and_replayed(case, entry):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(i, ids[a:a + 40]) and torch.equal(d, dist[a:a + 40])
+
+
+@pytest.mark.parametrize("n", [1, 7, 40, 128, 153, 300])
+def test_cut_streams_back_to_back(case, n):
+    """Without an early stop these batches' streams are cut into spans, whose
+    logs one block commits for another (the batch of 600 keeps them whole)."""
+    torch, ix, q, _, _ = case
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    got = []
+    for x in ix:
+        x.set_params(t_low=0)
+    try:
+        ids, dist = (v.clone() for v in ix[0].search(q, 10, 256, 1024))
+        torch.cuda.synchronize()
+        for r in range(20):
+            for j in range(2):
+                a = (37 * r + 11 * j) % (600 - n)
+                with torch.cuda.stream(streams[j]):
+                    i, d = ix[j].search(q[a:a + n], 10, 256, 1024)
+                    got.append((a, i, d))
+        torch.cuda.synchronize()
+    finally:
+        for x in ix:
+            x.set_params()
+    for a, i, d in got:
+        assert torch.equal(i, ids[a:a + n]) and torch.equal(d, dist[a:a + n])
