@@ -321,7 +321,11 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
     // a bit for each row of the warp that begins a segment after the first's
     const bool starts = wpos > first && wpos <= last;
     const unsigned bits = __reduce_or_sync(kFull, starts ? 1u << (wpos - first) : 0u);
-    if (__popc(__ballot_sync(kFull, starts)) == __popc(bits)) {
+    // the bits name the segments if no two begin at one row, neither in the
+    // window nor just past one that ends among these rows (31 of one row and one
+    // without rows as its last: the row at `last` is the segment's after it)
+    const bool whole = __shfl_sync(kFull, wpos, 31) > last || wseg + 32 >= nl || segs[wseg + 32].pos > last;
+    if (whole && __popc(__ballot_sync(kFull, starts)) == __popc(bits)) {
       const int i = head - 1 + __popc(bits & (0xffffffffu >> (31 - lane)));
       const uint32_t row = __shfl_sync(kFull, wdelta, i) + p;
       return p < p1 ? row : 0u;
