@@ -312,10 +312,12 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
     const uint32_t first = p0 + t * TR + warp * 32u, p = first + lane;
     if (first >= p1) return 0u;
     const uint32_t last = min(first + 31u, p1 - 1u);
-    int head;  // segments of the window that begin at or before the first row
+    int head;       // segments of the window that begin at or before the first row
+    uint32_t tail;  // where its last one begins
     for (;;) {
       head = __popc(__ballot_sync(kFull, wpos <= first));
-      if (__shfl_sync(kFull, wpos, 31) > last || head <= 1) break;
+      tail = __shfl_sync(kFull, wpos, 31);
+      if (tail > last || head <= 1) break;
       window(wseg + head - 1);
     }
     // a bit for each row of the warp that begins a segment after the first's
@@ -324,7 +326,7 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
     // the bits name the segments if no two begin at one row, neither in the
     // window nor just past one that ends among these rows (31 of one row and one
     // without rows as its last: the row at `last` is the segment's after it)
-    const bool whole = __shfl_sync(kFull, wpos, 31) > last || wseg + 32 >= nl || segs[wseg + 32].pos > last;
+    const bool whole = tail > last || wseg + 32 >= nl || segs[wseg + 32].pos > last;
     if (whole && __popc(__ballot_sync(kFull, starts)) == __popc(bits)) {
       const int i = head - 1 + __popc(bits & (0xffffffffu >> (31 - lane)));
       const uint32_t row = __shfl_sync(kFull, wdelta, i) + p;
@@ -561,7 +563,10 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
       into = st;
       st = st + 1 == ST ? 0 : st + 1;
       if (KCC > 0) {
-        if (kk + 1 < nk) continue;  // the row is not complete yet
+        if (kk + 1 < nk) {  // the row is not complete yet
+          __syncwarp();     // the piece is read before the next copies reuse its stage
+          continue;
+        }
         acc = 0.0f;
       }
       merge(t, dkey, m.srow[(t % ST) * TR + tid], ext);
