@@ -1,8 +1,9 @@
 // K4 refine (Sec. 3.4, Algorithm 2's T_low rule; uint8 distances kept as
-// integers, Sec. 4.1.1): a plan kernel cuts the queries' candidate streams
-// into spans, and persistent CTAs pull spans from an atomic counter, run
-// nrq::refine_span on the segments K3 wrote to global memory and commit the
-// spans of a query in stream order.
+// integers, Sec. 4.1.1), by persistent CTAs that pull work from an atomic
+// counter and run nrq::refine_span on the segments K3 wrote to global memory.
+// Many queries: a CTA refines a query's whole candidate stream (refine_kernel).
+// Few: a plan cuts the streams into spans, which CTAs refine side by side and
+// commit in stream order (refine_spans_kernel).
 //
 // Bound by HBM at large batches, less what queries share in L2, and by latency
 // at small ones: one block a query left a single query to one SM (one uint8
@@ -11,12 +12,12 @@
 //
 // Launch shapes measured on GB300: the scan is limited by the bytes in flight
 // per SM, so tiles are small (128 uint8 rows, 32-64 fp32 rows). uint8, D = 128:
-// 3 stages and 4 CTAs an SM hold 8 tiles in flight, 2 stages and 6 CTAs 6 (with
-// nearby codes side by side 7,780 and 8,318 us a batch of 10,000; 4 stages and
-// 3 CTAs 8,754, 6 and 2 11,815). fp32, D = 96: 2 stages of 64
-// rows and 4 CTAs of two warps (4,473 us a batch of 10,000; 32 rows and 9 CTAs
-// 4,805, 3 stages and 6 CTAs 4,905: fewer queries side by side share more,
-// but a row's chain is serial and needs the warps).
+// 3 stages and 4 CTAs an SM hold 8 tiles in flight, 2 stages and 6 CTAs 6 but
+// more warps (see bound_by_stream; 4 stages and 3 CTAs, 6 and 2 were slower
+// than both). fp32, D = 96: 2 stages of 64 rows and 4 CTAs of two warps (4,473
+// us a batch of 10,000; 32 rows and 9 CTAs 4,805, 3 stages and 6 CTAs 4,905:
+// fewer queries side by side share more, but a row's chain is serial and needs
+// the warps).
 // Tiles held in registers (eight lanes a 128-byte row, no shared memory) had
 // fewer bytes in flight: 14.8 ms for 9.1.
 #include <cuda_runtime.h>
@@ -96,11 +97,10 @@ __device__ __forceinline__ uint32_t spans_of(uint32_t n, uint32_t span) {
 // go at the end, longest first (1024 buckets scaled to the longest stream), so
 // that the persistent CTAs finish together; the others go by the top bits of
 // their base code, since queries of nearby codes have many clusters in common
-// and those that run at the same time read them from L2. Against longest first
-// throughout: 10,000 queries of the 3e7-row uint8 index 9,016 -> 7,792 us, of
-// the 1e7-row fp32 one 5,130 -> 4,796 (tiles of 32 rows). Order inside a bucket is arbitrary; no
-// order affects any result. Streams cut into spans keep the batch's order:
-// their items are short.
+// and those that run at the same time read them from L2 (last = nq: longest
+// first throughout; see nearby_first for both). Order inside a bucket is
+// arbitrary; no order affects any result. Streams cut into spans keep the
+// batch's order: their items are short.
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(PlanArgs a) {
   __shared__ uint64_t wsum[32];
   __shared__ unsigned int hist[kOrderBins], hcode[kOrderBins];
@@ -194,10 +194,10 @@ struct RefineArgs {
   float *out_d;
   int64_t *stats;
   nrq::RefinePlan *plan;
-  const uint32_t *pre;       // null: whole streams, in the order of perm
+  const uint32_t *pre;       // [nq + 1] first item of a query (not with own_plan)
   bool own_plan;             // every block works the plan out itself (at most kOwnPlan queries)
   SpanRule rule;
-  const int32_t *perm;
+  const int32_t *perm;       // order of whole streams; they use nothing below
   nrq::RefineQState *state;  // [nq]
   uint32_t *ready;           // [items] 0: not finished, 1: nothing logged, 2: logged, or kSpanRedo
   nrq::SpanHeader *hdr;      // [items]
@@ -232,15 +232,73 @@ constexpr int kPolls = 64;
 // sctl words of the kernel (1..3 are refine_span's)
 enum { kCtlQuery = 4, kCtlItem, kCtlSpan, kCtlSpans, kCtlRun, kCtlHn, kCtlRounds, kCtlLow, kCtlNext };
 
+// The answer of query q (a stream of n rows) from the top-k in r, sorted by
+// (distance, id), padded. Whole block of TR threads.
+template <int DT, int TR>
+__device__ __forceinline__ void write_answer(const RefineArgs &a, const nrq::RefineSmem &m,
+                                             const nrq::SpanRun &r, int64_t q, uint32_t n) {
+  const int tid = threadIdx.x, k = a.rf.k;
+  const uint64_t *H = m.hkey + r.cur * k;
+  for (int i = tid; i < k; i += TR) {
+    int64_t id = -1;
+    float d = __int_as_float(0x7f800000);
+    if (i < r.hn) {
+      const uint64_t kk = H[i];
+      id = (int64_t)(uint32_t)kk;
+      const uint32_t db = (uint32_t)(kk >> 32);
+      d = DT == 0 ? (float)db : __uint_as_float(db);
+    }
+    a.out_ids[q * k + i] = id;
+    a.out_d[q * k + i] = d;
+  }
+  if (tid == 0 && a.stats) {
+    const uint64_t rows = (uint64_t)r.rounds * (uint64_t)a.rf.R;
+    a.stats[q * NR_QSTATS] = (int64_t)(rows < n ? rows : n);  // rows of completed rounds
+    a.stats[q * NR_QSTATS + 1] = r.rounds;
+  }
+}
+
+// Whole streams, a block each, in the order of perm. A kernel of its own: what
+// spans need (the log, the commit, the plan) costs registers and 2 KB of shared
+// memory, a block an SM less at some row sizes, and instructions in every tile.
+// In one kernel with the spans, and here: 10,000 uint8 queries, P 64, k 100
+// 5,479 and 3,475 us, k 10 1,370 and 1,113; 2,000 of fp32 rows, D = 64, 1,988
+// and 1,642, D = 272 6,020 and 4,886 (each with the order and shape it takes).
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int tid = threadIdx.x;
+  const nrq::RefineSmem m = nrq::refine_carve<DT, TR, CPR, KCC, ST, false>(smem, a.row_bytes, a.rf.k);
+  volatile int *ctl = m.sctl;
+  for (bool first = true;; first = false) {
+    if (tid == 0) {
+      const uint32_t t = first ? blockIdx.x : gridDim.x + atomicAdd(&a.plan->ticket, 1u);
+      ctl[kCtlQuery] = t < (uint32_t)a.nq ? a.perm[t] : -1;
+    }
+    __syncthreads();
+    const int64_t q = ctl[kCtlQuery];
+    if (q < 0) return;
+    for (int c = tid; c * 16 < a.row_bytes; c += TR)
+      reinterpret_cast<uint4 *>(m.sq)[c] = reinterpret_cast<const uint4 *>(a.q + q * a.row_bytes)[c];
+    const uint32_t n = a.slen[q];
+    nrq::SpanRun r = {0, 0, 0, 0, false};
+    nrq::SpanLog lg;  // not used: nothing is logged
+    nrq::refine_span<DT, TR, CPR, KCC, ST>(a.rf, m, 0u, n, a.nL[q], a.seg + (size_t)q * a.Lmax, true, r, lg);
+    write_answer<DT, TR>(a, m, r, q, n);
+    __syncthreads();  // m and ctl are free for the next query
+  }
+}
+
+// Streams cut into spans.
+template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
+__global__ void __launch_bounds__(TR, MINB) refine_spans_kernel(RefineArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   nr_after_previous();
   const int tid = threadIdx.x, lane = tid & 31;
   const int k = a.rf.k;
-  const nrq::RefineSmem m = nrq::refine_carve<TR, KCC, ST>(smem, a.row_bytes, k);
+  const nrq::RefineSmem m = nrq::refine_carve<DT, TR, CPR, KCC, ST, true>(smem, a.row_bytes, k);
   volatile int *ctl = m.sctl;
-  uint32_t *spre = reinterpret_cast<uint32_t *>(m.sctl + 16);  // [kOwnPlan + 1], then the span's rows
+  uint32_t *spre = m.plan;  // [kOwnPlan + 1], then the span's rows
   if (a.own_plan && tid < 32) {
     constexpr int per = kOwnPlan / 32;
     uint32_t n[per], rounds = 0, items = 0;
@@ -291,10 +349,6 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
           t = __shfl_sync(nrq::kFull, t, 0);
         }
         if (t >= nitems) break;
-        if (!a.pre) {
-          q = a.perm[t];
-          break;
-        }
         int i;
         item_of(a, pre, t, i, sp);
         if (sp > 0 && __ldcg(&a.state[i].done)) continue;
@@ -321,7 +375,7 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
     bool held = sp == 0;  // this block owns the query's top-k
     nrq::SpanRun r = {0, 0, 0, 0, false};
     for (;;) {
-      const uint32_t p0 = sp * span_rows;  // span 0 when streams are whole
+      const uint32_t p0 = sp * span_rows;
       const uint32_t p1 = n - p0 > span_rows ? p0 + span_rows : n;
       nrq::SpanLog lg;
       lg.nthr = &st->nthr;
@@ -395,33 +449,15 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
                                                  a.hdr + base, next, spans, n, span_rows, polls);
           }
         }
-        const uint64_t *H = m.hkey + r.cur * k;
-        if (r.stop || next == spans) {  // the answer, sorted by (distance, id), padded
-          for (int i = tid; i < k; i += TR) {
-            int64_t id = -1;
-            float d = __int_as_float(0x7f800000);
-            if (i < r.hn) {
-              const uint64_t kk = H[i];
-              id = (int64_t)(uint32_t)kk;
-              const uint32_t db = (uint32_t)(kk >> 32);
-              d = DT == 0 ? (float)db : __uint_as_float(db);
-            }
-            a.out_ids[q * k + i] = id;
-            a.out_d[q * k + i] = d;
-          }
-          if (tid == 0) {
-            const uint64_t rows = (uint64_t)r.rounds * (uint64_t)a.rf.R;
-            if (a.stats) {
-              a.stats[q * NR_QSTATS] = (int64_t)(rows < n ? rows : n);  // rows of completed rounds
-              a.stats[q * NR_QSTATS + 1] = r.rounds;
-            }
-            if (spans > 1) atomicExch(&st->done, 1);
-          }
+        if (r.stop || next == spans) {
+          write_answer<DT, TR>(a, m, r, q, n);
+          if (tid == 0 && spans > 1) atomicExch(&st->done, 1);
           redo = false;
           break;  // the lock stays taken: there is nothing more to commit
         }
         if (redo) break;
         // hand the top-k back
+        const uint64_t *H = m.hkey + r.cur * k;
         for (int i = tid; i < r.hn; i += TR) a.heap[q * k + i] = H[i];
         if (tid == 0) {
           st->hn = r.hn;
@@ -449,6 +485,25 @@ __global__ void __launch_bounds__(TR, MINB) refine_kernel(RefineArgs a) {
   }
 }
 
+// Resident blocks of `kern` (blocks of TR threads with smem bytes), or 0 and
+// the error.
+template <class K>
+int64_t resident(const nr_index *ix, K kern, int TR, size_t smem, cudaError_t *e) {
+  int per_sm = 0;
+  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (*e == cudaSuccess) *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TR, smem);
+  if (*e == cudaSuccess && per_sm < 1) *e = cudaErrorInvalidConfiguration;
+  if (*e != cudaSuccess) return 0;
+  if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
+  return (int64_t)per_sm * ix->num_sms;
+}
+
+cudaError_t launch_plan(nr_index *ix, const PlanArgs &pa, cudaStream_t s) {
+  plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
+  ix->launches += 1;
+  return cudaGetLastError();
+}
+
 // Whether a batch keeps its streams whole (a block a query) when grid blocks
 // are resident. Few queries leave most blocks idle; many keep them busy, and
 // cutting their streams only adds work per span (about 7 us each: the item,
@@ -467,38 +522,62 @@ bool whole_streams(int64_t nq, int64_t grid, int t_low, bool long_rows) {
   return nq * 16 >= grid * sixteenths;
 }
 
+// Of whole streams: whether nearby queries go side by side (see plan_kernel).
+// Only where the rows read bound the tile (the generic ones are bound by their
+// instructions: 2,000 fp32 queries, D = 64, 1,640 us longest first, 1,907 by
+// code), and with queries enough to share (long rows, D = 288: 2,000 queries
+// 4,565 and 4,868 us, 8,000 16,978 and 14,980; f32-10m, P = 512: 3,000 2,435 and
+// 2,454, 10,000 7,858 and 7,134).
+bool nearby_first(const RefineArgs &a, bool bound_by_rows) { return bound_by_rows && a.nq >= 4096; }
+
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
-cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s, bool early) {
-  const size_t smem = nrq::refine_smem_bytes<TR, KCC, ST>(a.row_bytes, a.rf.k);
+cudaError_t launch_whole(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s) {
+  const size_t smem = nrq::refine_smem_bytes<DT, TR, CPR, KCC, ST, false>(a.row_bytes, a.rf.k);
   auto kern = refine_kernel<DT, TR, CPR, KCC, ST, MINB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e;
+  const int64_t grid = std::min(resident(ix, kern, TR, smem, &e), a.nq);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TR, smem);
+  pa.rule.items_cap = (unsigned int)a.nq;
+  pa.last = nearby_first(a, CPR > 0 || KCC > 0) ? grid : a.nq;
+  if ((e = launch_plan(ix, pa, s)) != cudaSuccess) return e;
+  kern<<<(unsigned)grid, TR, smem, s>>>(a);
+  ix->launches += 1;
+  return cudaGetLastError();
+}
+
+// Of uint8 rows of 128 bytes, whole streams: whether the stream's bytes bound a
+// block (three stages, four blocks an SM: more rows in flight) or its merges
+// (two stages, six blocks). Long streams and a small top-k the one, short ones,
+// a larger top-k and many queries that share rows the other. us, three stages
+// and two: u8-30m P = C = 1024, t_low 80, 10,000 queries: k 10 10,019 / 10,528,
+// k 100 13,720 / 12,885; u8-10m P = C = 256, no early stop, k 10: 900 queries
+// 607 / 702, 3,000 1,478 / 1,567, 10,000 4,507 / 4,061; k 100, 10,000 6,541 /
+// 5,431; P 64, C 128, t_low 4: 2,000 330 / 312, 10,000 1,290 / 1,113.
+bool bound_by_stream(const RefineArgs &a, int C) {
+  return a.rf.k <= 32 && (C >= 1024 || (C >= 256 && a.nq < 4096 && (a.rf.t_low == 0 || a.rf.t_low >= 8)));
+}
+
+template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
+cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s, bool early, bool room) {
+  const size_t smem = nrq::refine_smem_bytes<DT, TR, CPR, KCC, ST, true>(a.row_bytes, a.rf.k);
+  auto kern = refine_spans_kernel<DT, TR, CPR, KCC, ST, MINB>;
+  cudaError_t e;
+  const int64_t grid = resident(ix, kern, TR, smem, &e);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
-  int64_t grid = (int64_t)per_sm * ix->num_sms;
+  if (!room || whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) {
+    if constexpr (CPR == 8)
+      if (!bound_by_stream(a, a.Lmax - pa.P)) return launch_whole<DT, TR, CPR, KCC, 2, 6>(ix, a, pa, s);
+    return launch_whole<DT, TR, CPR, KCC, ST, MINB>(ix, a, pa, s);
+  }
   pa.rule.align = a.rf.R < TR ? TR / a.rf.R : 1;
   // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
   // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
   // 1,075)
   pa.rule.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
-  if (whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) pa.rule.items_cap = (unsigned int)a.nq;
   a.group = (int)grid;
   a.rule = pa.rule;
-  a.own_plan = pa.rule.items_cap > a.nq && a.nq <= kOwnPlan;
-  if (pa.rule.items_cap <= a.nq) {  // whole streams
-    a.pre = nullptr;
-    grid = std::min(grid, a.nq);
-    pa.last = std::min(grid, a.nq);
-  }
-  if (!a.own_plan) {
-    plan_kernel<<<1, kPlanThreads, 0, s>>>(pa);
-    ix->launches += 1;
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  a.own_plan = a.nq <= kOwnPlan;
+  if (!a.own_plan && (e = launch_plan(ix, pa, s)) != cudaSuccess) return e;
   e = nr_launch_kernel(kern, (unsigned)grid, TR, smem, s, early && a.own_plan, a);
   ix->launches += 1;
   return e;
@@ -581,8 +660,8 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   char *w = static_cast<char *>(d_scratch);
   const int64_t items = span_items(nq), entries = span_entries(nq, k);
   RefineScratch l = refine_scratch(nq, k, items, entries);
-  const bool whole = l.total > scratch_bytes;  // no room to cut streams
-  if (whole) l = refine_scratch(nq, k, nq, 0);
+  const bool room = l.total <= scratch_bytes;  // to cut streams
+  if (!room) l = refine_scratch(nq, k, nq, 0);
   RefineArgs a;
   a.rf = refine_params(ix, k);
   a.q = static_cast<const uint8_t *>(d_q);
@@ -603,7 +682,7 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   a.hdr = reinterpret_cast<nrq::SpanHeader *>(w + l.hdr);
   a.heap = reinterpret_cast<uint64_t *>(w + l.heap);
   a.pool = reinterpret_cast<nrq::SpanEntry *>(w + l.pool);
-  a.pool_cap = whole ? 0u : (uint32_t)entries;
+  a.pool_cap = room ? (uint32_t)entries : 0u;
   PlanArgs pa;
   pa.slen = d_slen;
   pa.codes = d_codes;
@@ -611,21 +690,21 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   pa.b = ix->b;
   pa.last = nq;
   pa.nq = nq;
-  pa.rule = {a.rf.R, 1, std::max(1, 8192 / a.rf.R), 1u, (unsigned int)(whole ? nq : items)};
+  pa.rule = {a.rf.R, 1, std::max(1, 8192 / a.rf.R), 1u, (unsigned int)(room ? items : nq)};
   pa.plan = a.plan;
   pa.pre = reinterpret_cast<uint32_t *>(w + l.pre);
   pa.perm = reinterpret_cast<int32_t *>(w + l.perm);
   if (ix->dtype == 0) {
-    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s, early);  // uint8, D = 128
-    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s, early);
-    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s, early);
+    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s, early, room);  // uint8, D = 128
+    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s, early, room);
+    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s, early, room);
   }
   if (ix->row_bytes > 1024) {  // fp32, D above 256: rows staged in pieces
-    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s, early);
-    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s, early);
-    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s, early);  // row_bytes % 64 == 0 (load check)
+    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s, early, room);
+    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s, early, room);
+    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s, early, room);  // row_bytes % 64 == 0 (load check)
   }
-  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s, early);  // fp32, D = 96
-  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s, early);
-  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s, early);
+  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s, early, room);  // fp32, D = 96
+  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s, early, room);
+  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s, early, room);
 }

@@ -68,7 +68,7 @@ struct RefineParams {
 struct RefinePlan {
   unsigned int ticket;            // items handed out beyond each block's first
   unsigned int nitems;            // spans of all queries
-  uint32_t span_rows;             // rows of a span (S R; 0xffffffff: whole streams)
+  uint32_t span_rows;             // rows of a span (S R)
   unsigned int pad;
   unsigned long long pool_used;   // log entries reserved
 };
@@ -97,9 +97,6 @@ constexpr uint32_t kSpanRedo = 0xffffffffu;  // ready value: not logged (the poo
 template <int DT, int CPR>
 constexpr bool kRow128 = DT == 0 && CPR == 8;
 
-// Log entries of a span that the commit stages in shared memory: its first
-// group's first 32.
-constexpr int kStaged = 32;
 // Bytes of the stages: ST tiles.
 template <int TR, int KCC, int ST>
 __host__ __device__ constexpr size_t refine_stage_bytes(int64_t row_bytes) {
@@ -110,36 +107,38 @@ __host__ __device__ constexpr size_t refine_stage_bytes(int64_t row_bytes) {
 struct RefineSmem {
   unsigned char *stage;  // refine_stage_bytes (16-byte aligned)
   unsigned char *sq;     // the query row (row_bytes)
-  uint32_t *srow;        // ST x TR: rows of the open tiles
+  uint32_t *srow;        // ST x TR: rows of the open tiles (kRow128: held in registers)
   uint64_t *hkey;        // 2 x k
   uint64_t *skey;        // 2 x TR
+  int *htag;             // 2 x k
+  int *sctl;             // 16 ints: [1..3] survivor counters, [4..15] the kernel's
+  // only where streams are cut (CUT):
   uint64_t *logk;        // kLogBlock: members logged and not yet written, and
   uint32_t *logr;        // their rounds
-  int *htag;             // 2 x k
-  int *sctl;             // 16 ints: [1..3] survivor counters, [4..15] the kernel's; then its plan (132 ints)
+  uint32_t *plan;        // 132: the kernel's
 };
 
-template <int TR, int KCC, int ST>
-__host__ __device__ inline size_t refine_smem_bytes(int64_t row_bytes, int k) {
-  return refine_stage_bytes<TR, KCC, ST>(row_bytes) + (size_t)row_bytes + (size_t)ST * TR * 4 +
-         (size_t)2 * k * 8 + (size_t)2 * TR * 8 + (size_t)kLogBlock * 12 + (size_t)2 * k * 4 + 16 * 4 +
-         132 * 4;
-}
-
 // Carve RefineSmem from base (16-byte aligned).
-template <int TR, int KCC, int ST>
+template <int DT, int TR, int CPR, int KCC, int ST, bool CUT>
 __device__ __forceinline__ RefineSmem refine_carve(unsigned char *base, int64_t row_bytes, int k) {
   RefineSmem m;
   m.stage = base;
   m.sq = base + refine_stage_bytes<TR, KCC, ST>(row_bytes);
   m.srow = reinterpret_cast<uint32_t *>(m.sq + row_bytes);
-  m.hkey = reinterpret_cast<uint64_t *>(m.srow + ST * TR);
+  m.hkey = reinterpret_cast<uint64_t *>(m.srow + (kRow128<DT, CPR> ? 0 : ST * TR));
   m.skey = m.hkey + 2 * k;
   m.logk = m.skey + 2 * TR;
-  m.logr = reinterpret_cast<uint32_t *>(m.logk + kLogBlock);
-  m.htag = reinterpret_cast<int *>(m.logr + kLogBlock);
+  m.htag = reinterpret_cast<int *>(m.logk + (CUT ? kLogBlock : 0));
   m.sctl = m.htag + 2 * k;
+  m.logr = reinterpret_cast<uint32_t *>(m.sctl + 16);
+  m.plan = m.logr + kLogBlock;
   return m;
+}
+template <int DT, int TR, int CPR, int KCC, int ST, bool CUT>
+__host__ __device__ inline size_t refine_smem_bytes(int64_t row_bytes, int k) {
+  return refine_stage_bytes<TR, KCC, ST>(row_bytes) + (size_t)row_bytes +
+         (kRow128<DT, CPR> ? 0 : (size_t)ST * TR * 4) + (size_t)2 * k * 8 + (size_t)2 * TR * 8 +
+         (size_t)2 * k * 4 + 16 * 4 + (CUT ? (size_t)kLogBlock * 12 + 132 * 4 : 0);
 }
 
 // Top-k state of a block (uniform in the block): which buffer, members,
@@ -326,12 +325,14 @@ __device__ __forceinline__ void refine_span(const RefineParams &a, const RefineS
     // the bits name the segments if no two begin at one row, neither in the
     // window nor just past one that ends among these rows (31 of one row and one
     // without rows as its last: the row at `last` is the segment's after it)
-    const bool whole = tail > last || wseg + 32 >= nl || segs[wseg + 32].pos > last;
-    if (whole && __popc(__ballot_sync(kFull, starts)) == __popc(bits)) {
+    const bool one_each = __popc(__ballot_sync(kFull, starts)) == __popc(bits);
+    auto by_bits = [&]() {
       const int i = head - 1 + __popc(bits & (0xffffffffu >> (31 - lane)));
       const uint32_t row = __shfl_sync(kFull, wdelta, i) + p;
       return p < p1 ? row : 0u;
-    }
+    };
+    if (one_each && tail > last) return by_bits();
+    if (one_each && (wseg + 32 >= nl || segs[wseg + 32].pos > last)) return by_bits();
     // segments without rows share their place with the next: the last one counts
     int i = wseg;
     while (i + 1 < nl && segs[i + 1].pos <= min(p, last)) ++i;

@@ -21,4 +21,4 @@ def test_handed_on_buffers_are_not_restrict():
             seen.add(name)
             const = re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", params)
             assert not HANDED_ON & set(const), (name, const)
-    assert seen == {"route_block_kernel", "select_kernel", "refine_kernel", "encode_layer_kernel"}
+    assert seen == {"route_block_kernel", "select_kernel", "refine_spans_kernel", "encode_layer_kernel"}
