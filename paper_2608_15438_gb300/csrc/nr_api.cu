@@ -39,8 +39,8 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 struct Layout {
   size_t logits, codes, nprobe, L, nL, seg, slen, slab, enc, refine, total;
 };
-// Without k there is no refinement (its scratch is bounded, whatever qc).
-Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C, int k = 0) {
+// refine: the refinement's scratch (0 without one)
+Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C, size_t refine = 0) {
   Layout l;
   size_t o = 0;
   const size_t Lmax = (size_t)P + (size_t)C;
@@ -53,7 +53,7 @@ Layout chunk_layout(const nr_index *ix, int64_t qc, int P, int C, int k = 0) {
   l.slen = o;   o = align256(o + (size_t)qc * 4);
   l.slab = o;   o = align256(o + nr_select_slab_total(qc, P, ix->K_max));
   l.enc = o;    o = align256(o + nr_encode_scratch_bytes(ix, qc));
-  l.refine = o; o = align256(o + (k > 0 ? nr_refine_scratch_bytes(qc, k, false) : 0));
+  l.refine = o; o = align256(o + refine);
   l.total = o;
   return l;
 }
@@ -814,16 +814,34 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
   const int64_t pc = ix->params.pipe_chunk;
   const bool pipe = pc > 0 && nq > pc;
   const int slots = pipe ? kPipeSlots : 1;
-  Layout one = chunk_layout(ix, 1, P, C);
+  nr_refine_room room;
+  cudaError_t e = nr_refine_room_of(ix, k, &room);
+  if (e != cudaSuccess) return cuda_status(e);
+  Layout one = chunk_layout(ix, 1, P, C, nr_refine_scratch_bytes(1, k, false));
   int64_t qc = (int64_t)(kChunkBudget / slots / (one.total > 0 ? one.total : 1));
   if (qc < 1) qc = 1;
   if (pipe && qc > pc) qc = pc;
   if (qc > nq) qc = nq;
-  Layout l = chunk_layout(ix, qc, P, C, k);
-  const size_t slot_bytes = align256(l.total);
+  // Beside the budget, room to cut as many of the queries as are ever cut (bounded:
+  // some 1,000 at 0.1 MB for k = 100), whether this batch is or not: a later,
+  // smaller one then fits the workspace, in a stream capture too.
+  const size_t whole_bytes = nr_refine_scratch_bytes(qc, k, false);
+  size_t cut_bytes = nr_refine_scratch_bytes(std::min(qc, room.most), k, true);
+  Layout l = chunk_layout(ix, qc, P, C, std::max(whole_bytes, cut_bytes));
+  size_t slot_bytes = align256(l.total);
   // workspace: [per-query stats][chunk buffers]
   const size_t stats_off = 0;
   const size_t chunk_off = align256(stats_off + (size_t)nq * NR_QSTATS * 8);
+  if (chunk_off + slot_bytes * (size_t)slots > ix->ws_cap) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) {
+      // it cannot grow now: streams stay whole (captured after calls of a smaller k)
+      cut_bytes = 0;
+      l = chunk_layout(ix, qc, P, C, whole_bytes);
+      slot_bytes = align256(l.total);
+    }
+  }
   if ((st = ensure_ws(ix, chunk_off + slot_bytes * (size_t)slots)) != NR_OK) return st;
   if (pipe && (st = ensure_pipe(ix)) != NR_OK) return st;
   char *w = (char *)ix->ws;
@@ -851,7 +869,6 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     cudaEventRecord(ex->timers[slot].b, st);
     ++tslot;
   };
-  cudaError_t e = cudaSuccess;
   if (pipe) {  // both library streams start after the caller's earlier work
     e = cudaEventRecord(ps.fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(sa, ps.fork, 0);
@@ -863,6 +880,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     const int64_t n = (nq - q0) < qc ? (nq - q0) : qc;
     const int slot = (int)(i % slots);
     char *cw = w + chunk_off + slot_bytes * (size_t)slot;
+    const bool cut = cut_bytes > 0 && nr_refine_cuts(ix, n, room);
     // buffer `slot` is free again once the refinement that last read it ended
     if (pipe && i >= slots && (e = cudaStreamWaitEvent(sa, ps.ref[slot], 0)) != cudaSuccess) break;
     const void *qp = (const char *)d_q + q0 * RB;
@@ -884,7 +902,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
                          (int32_t *)(cw + l.L), (int32_t *)(cw + l.nL), (nr_seg *)(cw + l.seg),
                          (uint32_t *)(cw + l.slen), stats + q0 * NR_QSTATS,
                          nr_select_slab_bytes(P, ix->K_max) ? cw + l.slab : nullptr,
-                         nr_refine_zero(n, k, cw + l.refine, l.total - l.refine), sa, true);
+                         nr_refine_zero(n, k, cut, cw + l.refine), sa, true);
     tend(ev, sa);
     if (e != cudaSuccess) break;
     if (pipe) {
@@ -895,8 +913,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     ev = tstart(3, sb);
     e = nr_launch_refine(ix, qp, n, k, P + C, (nr_seg *)(cw + l.seg), (int32_t *)(cw + l.nL),
                          (uint32_t *)(cw + l.slen), (uint32_t *)(cw + l.codes), P, d_ids + q0 * k,
-                         d_d + q0 * k, stats + q0 * NR_QSTATS,
-                         cw + l.refine, l.total - l.refine, sb, !pipe);
+                         d_d + q0 * k, stats + q0 * NR_QSTATS, cut, room.blocks, cw + l.refine, sb, !pipe);
     tend(ev, sb);
     if (pipe && e == cudaSuccess) e = cudaEventRecord(ps.ref[slot], sb);
   }

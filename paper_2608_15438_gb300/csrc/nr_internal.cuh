@@ -193,17 +193,26 @@ cudaError_t nr_launch_select(nr_index *ix, const float *d_logits, const uint32_t
                              const int32_t *d_nprobe, int64_t nq, int P, int C, int32_t *d_L,
                              int32_t *d_nL, nr_seg *d_seg, uint32_t *d_slen, int64_t *d_stats,
                              void *d_slab, nr_zero zero, cudaStream_t s, bool early = false);
-// the flags of a refine launch's scratch that have to be zero: the select
-// launch before it clears them
-nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes);
-// scratch of a refine launch over nq queries: room to refine one query's
-// stream by several blocks at once, or (least) only whole streams a block
-size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least);
-// d_codes: the probe codes [nq x P], the base code first. scratch: at least the
-// least bytes, nr_refine_zero of it cleared; whole streams a block below the
-// others
+// Whether the refinement of a batch cuts its queries' streams into spans, which
+// several blocks refine at once, or keeps them whole, a block each. A caller
+// decides it before it lays out its scratch: cutting takes buffers for spans and
+// logs (0.1 MB a query at k = 100; few queries are cut), whole streams
+// take 4 bytes a query.
+struct nr_refine_room {
+  int64_t blocks;  // of the spans' kernel, resident at once
+  int64_t most;    // no larger batch is cut, whatever the parameters
+};
+cudaError_t nr_refine_room_of(const nr_index *ix, int k, nr_refine_room *room);
+bool nr_refine_cuts(const nr_index *ix, int64_t nq, const nr_refine_room &room);
+// scratch of a refine launch over nq queries
+size_t nr_refine_scratch_bytes(int64_t nq, int k, bool cut);
+// the flags in it that have to be zero (none of whole streams): the select launch
+// before the refinement clears them
+nr_zero nr_refine_zero(int64_t nq, int k, bool cut, void *scratch);
+// d_codes: the probe codes [nq x P], the base code first. scratch:
+// nr_refine_scratch_bytes of it, nr_refine_zero of it cleared
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
                              const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
-                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s,
-                             bool early = false);
+                             int64_t *d_stats, bool cut, int64_t blocks, void *d_scratch,
+                             cudaStream_t s, bool early = false);

@@ -486,16 +486,21 @@ __global__ void __launch_bounds__(TR, MINB) refine_spans_kernel(RefineArgs a) {
 }
 
 // Resident blocks of `kern` (blocks of TR threads with smem bytes), or 0 and
-// the error.
+// the error. The kernel may take all the shared memory there is from here on:
+// the same for every caller, so that no other thread's call lowers it before
+// this one's launch.
 template <class K>
 int64_t resident(const nr_index *ix, K kern, int TR, size_t smem, cudaError_t *e) {
   int per_sm = 0;
-  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ix->smem_optin);
   if (*e == cudaSuccess) *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TR, smem);
   if (*e == cudaSuccess && per_sm < 1) *e = cudaErrorInvalidConfiguration;
-  if (*e != cudaSuccess) return 0;
-  if (ix->params.refine_ctas > 0 && per_sm > ix->params.refine_ctas) per_sm = ix->params.refine_ctas;
-  return (int64_t)per_sm * ix->num_sms;
+  return *e == cudaSuccess ? (int64_t)per_sm * ix->num_sms : 0;
+}
+// Those of them that the parameters allow.
+int64_t allowed(const nr_index *ix, int64_t blocks) {
+  const int64_t most = (int64_t)ix->params.refine_ctas * ix->num_sms;
+  return most > 0 && blocks > most ? most : blocks;
 }
 
 cudaError_t launch_plan(nr_index *ix, const PlanArgs &pa, cudaStream_t s) {
@@ -535,9 +540,8 @@ cudaError_t launch_whole(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s
   const size_t smem = nrq::refine_smem_bytes<DT, TR, CPR, KCC, ST, false>(a.row_bytes, a.rf.k);
   auto kern = refine_kernel<DT, TR, CPR, KCC, ST, MINB>;
   cudaError_t e;
-  const int64_t grid = std::min(resident(ix, kern, TR, smem, &e), a.nq);
+  const int64_t grid = std::min(allowed(ix, resident(ix, kern, TR, smem, &e)), a.nq);
   if (e != cudaSuccess) return e;
-  pa.rule.items_cap = (unsigned int)a.nq;
   pa.last = nearby_first(a, CPR > 0 || KCC > 0) ? grid : a.nq;
   if ((e = launch_plan(ix, pa, s)) != cudaSuccess) return e;
   kern<<<(unsigned)grid, TR, smem, s>>>(a);
@@ -558,17 +562,10 @@ bool bound_by_stream(const RefineArgs &a, int C) {
 }
 
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
-cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t s, bool early, bool room) {
+cudaError_t launch_spans(nr_index *ix, RefineArgs a, PlanArgs pa, int64_t grid, cudaStream_t s, bool early) {
   const size_t smem = nrq::refine_smem_bytes<DT, TR, CPR, KCC, ST, true>(a.row_bytes, a.rf.k);
-  auto kern = refine_spans_kernel<DT, TR, CPR, KCC, ST, MINB>;
+  auto kern = refine_spans_kernel<DT, TR, CPR, KCC, ST, MINB>;  // (resident has set its attribute)
   cudaError_t e;
-  const int64_t grid = resident(ix, kern, TR, smem, &e);
-  if (e != cudaSuccess) return e;
-  if (!room || whole_streams(a.nq, grid, a.rf.t_low, KCC > 0)) {
-    if constexpr (CPR == 8)
-      if (!bound_by_stream(a, a.Lmax - pa.P)) return launch_whole<DT, TR, CPR, KCC, 2, 6>(ix, a, pa, s);
-    return launch_whole<DT, TR, CPR, KCC, ST, MINB>(ix, a, pa, s);
-  }
   pa.rule.align = a.rf.R < TR ? TR / a.rf.R : 1;
   // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
   // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
@@ -581,6 +578,30 @@ cudaError_t launch_refine(nr_index *ix, RefineArgs a, PlanArgs pa, cudaStream_t 
   e = nr_launch_kernel(kern, (unsigned)grid, TR, smem, s, early && a.own_plan, a);
   ix->launches += 1;
   return e;
+}
+
+// A row size's tile: rows of a tile, chunks of a row (0: any), chunks of a piece
+// (0: whole rows), stages, blocks an SM at least.
+template <int DT_, int TR_, int CPR_, int KCC_, int ST_, int MINB_>
+struct Shape {
+  static constexpr int DT = DT_, TR = TR_, CPR = CPR_, KCC = KCC_, ST = ST_, MINB = MINB_;
+};
+template <class F>
+cudaError_t by_shape(const nr_index *ix, F f) {
+  const int64_t rb = ix->row_bytes;
+  if (ix->dtype == 0) {
+    if (rb == 128) return f(Shape<0, 128, 8, 0, 3, 4>());  // uint8, D = 128
+    if (rb <= 512) return f(Shape<0, 128, 0, 0, 2, 4>());
+    return f(Shape<0, 64, 0, 0, 2, 4>());
+  }
+  if (rb > 1024) {  // fp32, D above 256: rows staged in pieces
+    if (rb % 256 == 0) return f(Shape<1, 128, 0, 16, 2, 3>());
+    if (rb % 128 == 0) return f(Shape<1, 128, 0, 8, 2, 3>());
+    return f(Shape<1, 128, 0, 4, 2, 3>());  // rb % 64 == 0 (load check)
+  }
+  if (rb == 384) return f(Shape<1, 64, 24, 0, 2, 4>());  // fp32, D = 96
+  if (rb <= 512) return f(Shape<1, 64, 0, 0, 2, 4>());
+  return f(Shape<1, 32, 0, 0, 2, 4>());
 }
 
 nrq::RefineParams refine_params(const nr_index *ix, int k) {
@@ -607,17 +628,15 @@ nrq::RefineParams refine_params(const nr_index *ix, int k) {
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Scratch of a refine launch: [order of whole streams][plan], and where
-// streams may be cut into items spans: [item prefix][plan, query states, ready
-// flags (zeroed together)][span headers][committed top-k][log entries]
+// Scratch of a refine launch. Whole streams: [their order][plan]. Cut ones:
+// [item prefix][plan, query states, ready flags (zeroed together)][span
+// headers][committed top-k][log entries]
 struct RefineScratch {
   size_t plan, perm, pre, state, ready, zero_end, hdr, heap, pool, total;
 };
 RefineScratch refine_scratch(int64_t nq, int k, int64_t items, int64_t entries) {
   RefineScratch l = {};
   size_t o = 0;
-  l.perm = o; o = up256(o + (size_t)nq * 4);
-  l.plan = o; o = up256(o + sizeof(nrq::RefinePlan));
   if (items > nq) {
     l.pre = o;   o = up256(o + ((size_t)nq + 1) * 4);
     l.plan = o;  o = up256(o + sizeof(nrq::RefinePlan));
@@ -627,6 +646,9 @@ RefineScratch refine_scratch(int64_t nq, int k, int64_t items, int64_t entries) 
     l.hdr = o;   o = up256(o + (size_t)items * sizeof(nrq::SpanHeader));
     l.heap = o;  o = up256(o + (size_t)nq * k * 8);
     l.pool = o;  o = up256(o + (size_t)entries * sizeof(nrq::SpanEntry));
+  } else {
+    l.perm = o; o = up256(o + (size_t)nq * 4);
+    l.plan = o; o = up256(o + sizeof(nrq::RefinePlan));
   }
   l.total = o;
   return l;
@@ -638,30 +660,43 @@ int64_t span_entries(int64_t nq, int k) {
   return std::min<int64_t>(16 << 20, (int64_t)k * std::max<int64_t>(4096, nq * 32));
 }
 
-}  // namespace
-
-size_t nr_refine_scratch_bytes(int64_t nq, int k, bool least) {
-  return least ? refine_scratch(nq, k, nq, 0).total
-               : refine_scratch(nq, k, span_items(nq), span_entries(nq, k)).total;
+RefineScratch refine_scratch(int64_t nq, int k, bool cut) {
+  return cut ? refine_scratch(nq, k, span_items(nq), span_entries(nq, k)) : refine_scratch(nq, k, nq, 0);
 }
 
-nr_zero nr_refine_zero(int64_t nq, int k, void *scratch, size_t scratch_bytes) {
-  const RefineScratch l = refine_scratch(nq, k, span_items(nq), span_entries(nq, k));
-  if (nq <= 0 || l.total > scratch_bytes) return {nullptr, 0};  // whole streams
+}  // namespace
+
+cudaError_t nr_refine_room_of(const nr_index *ix, int k, nr_refine_room *room) {
+  return by_shape(ix, [&](auto sh) {
+    using S = decltype(sh);
+    cudaError_t e;
+    const int64_t blocks = resident(ix, refine_spans_kernel<S::DT, S::TR, S::CPR, S::KCC, S::ST, S::MINB>, S::TR,
+                       nrq::refine_smem_bytes<S::DT, S::TR, S::CPR, S::KCC, S::ST, true>(ix->row_bytes, k), &e);
+    *room = {allowed(ix, blocks), blocks};  // whole_streams: less than a query a block
+    return e;
+  });
+}
+
+bool nr_refine_cuts(const nr_index *ix, int64_t nq, const nr_refine_room &room) {
+  return !whole_streams(nq, room.blocks, ix->params.t_low, ix->dtype == 1 && ix->row_bytes > 1024);
+}
+
+size_t nr_refine_scratch_bytes(int64_t nq, int k, bool cut) { return refine_scratch(nq, k, cut).total; }
+
+nr_zero nr_refine_zero(int64_t nq, int k, bool cut, void *scratch) {
+  if (!cut) return {nullptr, 0};
+  const RefineScratch l = refine_scratch(nq, k, cut);
   return {static_cast<char *>(scratch) + l.plan, (l.zero_end - l.plan) / 16};
 }
 
 cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, int Lmax,
                              const nr_seg *d_seg, const int32_t *d_nL, const uint32_t *d_slen,
                              const uint32_t *d_codes, int P, int64_t *d_ids, float *d_dists,
-                             int64_t *d_stats, void *d_scratch, size_t scratch_bytes, cudaStream_t s,
+                             int64_t *d_stats, bool cut, int64_t blocks, void *d_scratch, cudaStream_t s,
                              bool early) {
   if (nq <= 0) return cudaSuccess;
   char *w = static_cast<char *>(d_scratch);
-  const int64_t items = span_items(nq), entries = span_entries(nq, k);
-  RefineScratch l = refine_scratch(nq, k, items, entries);
-  const bool room = l.total <= scratch_bytes;  // to cut streams
-  if (!room) l = refine_scratch(nq, k, nq, 0);
+  const RefineScratch l = refine_scratch(nq, k, cut);
   RefineArgs a;
   a.rf = refine_params(ix, k);
   a.q = static_cast<const uint8_t *>(d_q);
@@ -682,7 +717,7 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   a.hdr = reinterpret_cast<nrq::SpanHeader *>(w + l.hdr);
   a.heap = reinterpret_cast<uint64_t *>(w + l.heap);
   a.pool = reinterpret_cast<nrq::SpanEntry *>(w + l.pool);
-  a.pool_cap = room ? (uint32_t)entries : 0u;
+  a.pool_cap = cut ? (uint32_t)span_entries(nq, k) : 0u;
   PlanArgs pa;
   pa.slen = d_slen;
   pa.codes = d_codes;
@@ -690,21 +725,15 @@ cudaError_t nr_launch_refine(nr_index *ix, const void *d_q, int64_t nq, int k, i
   pa.b = ix->b;
   pa.last = nq;
   pa.nq = nq;
-  pa.rule = {a.rf.R, 1, std::max(1, 8192 / a.rf.R), 1u, (unsigned int)(room ? items : nq)};
+  pa.rule = {a.rf.R, 1, std::max(1, 8192 / a.rf.R), 1u, (unsigned int)(cut ? span_items(nq) : nq)};
   pa.plan = a.plan;
   pa.pre = reinterpret_cast<uint32_t *>(w + l.pre);
   pa.perm = reinterpret_cast<int32_t *>(w + l.perm);
-  if (ix->dtype == 0) {
-    if (a.rf.cpr == 8) return launch_refine<0, 128, 8, 0, 3, 4>(ix, a, pa, s, early, room);  // uint8, D = 128
-    if (ix->row_bytes <= 512) return launch_refine<0, 128, 0, 0, 2, 4>(ix, a, pa, s, early, room);
-    return launch_refine<0, 64, 0, 0, 2, 4>(ix, a, pa, s, early, room);
-  }
-  if (ix->row_bytes > 1024) {  // fp32, D above 256: rows staged in pieces
-    if (ix->row_bytes % 256 == 0) return launch_refine<1, 128, 0, 16, 2, 3>(ix, a, pa, s, early, room);
-    if (ix->row_bytes % 128 == 0) return launch_refine<1, 128, 0, 8, 2, 3>(ix, a, pa, s, early, room);
-    return launch_refine<1, 128, 0, 4, 2, 3>(ix, a, pa, s, early, room);  // row_bytes % 64 == 0 (load check)
-  }
-  if (a.rf.cpr == 24) return launch_refine<1, 64, 24, 0, 2, 4>(ix, a, pa, s, early, room);  // fp32, D = 96
-  if (ix->row_bytes <= 512) return launch_refine<1, 64, 0, 0, 2, 4>(ix, a, pa, s, early, room);
-  return launch_refine<1, 32, 0, 0, 2, 4>(ix, a, pa, s, early, room);
+  return by_shape(ix, [&](auto sh) {
+    using S = decltype(sh);
+    if (cut) return launch_spans<S::DT, S::TR, S::CPR, S::KCC, S::ST, S::MINB>(ix, a, pa, blocks, s, early);
+    if constexpr (S::CPR == 8)
+      if (!bound_by_stream(a, Lmax - P)) return launch_whole<S::DT, S::TR, S::CPR, S::KCC, 2, 6>(ix, a, pa, s);
+    return launch_whole<S::DT, S::TR, S::CPR, S::KCC, S::ST, S::MINB>(ix, a, pa, s);
+  });
 }

@@ -85,8 +85,8 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   const size_t slab_q = nr_select_slab_bytes(P, ix->K_max);
   const size_t o_slab = o;   o = up256(o + nr_select_slab_total((int64_t)q, P, ix->K_max));
   const size_t o_enc = o;    o = up256(o + nr_encode_scratch_bytes(ix, (int64_t)q));
-  // the rest serves the refinement, which takes what it can use of it
-  const size_t o_refine = o; o += nr_refine_scratch_bytes(nq, k, true);
+  // the rest serves the refinement, which cuts streams where there is room for it
+  const size_t o_refine = o; o += nr_refine_scratch_bytes(nq, k, false);
   if (o > NR_STATIC_SCRATCH_BYTES) return NR_ERR_INVALID_ARG;  // request too large for the array
   DeviceGuard g(ix->device);
   if (!g.ok) return NR_ERR_CUDA;
@@ -97,21 +97,25 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   cudaStream_t s = (cudaStream_t)stream;
   float *logits = (float *)(w + o_logits);
   int64_t *stats = (int64_t *)(w + o_stats);
+  nr_refine_room room;
+  cudaError_t e = nr_refine_room_of(ix, k, &room);
+  if (e != cudaSuccess) return cuda_status(e);
+  const bool cut = nr_refine_cuts(ix, nq, room) &&
+                   nr_refine_scratch_bytes(nq, k, true) <= NR_STATIC_SCRATCH_BYTES - o_refine;
   // every buffer below is fully written before it is read, except the
-  // refinement's flags, which its launcher clears on the stream
-  cudaError_t e = nr_launch_encode(ix, d_queries, nq, logits, s, w + o_enc);
+  // refinement's flags, which the selection clears
+  e = nr_launch_encode(ix, d_queries, nq, logits, s, w + o_enc);
   if (e == cudaSuccess)
     e = nr_launch_route(ix, logits, nq, P, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), s, true);
   if (e == cudaSuccess)
     e = nr_launch_select(ix, logits, (uint32_t *)(w + o_codes), (int32_t *)(w + o_nprobe), nq, P, C,
                          (int32_t *)(w + o_L), (int32_t *)(w + o_nL), (nr_seg *)(w + o_seg),
                          (uint32_t *)(w + o_slen), stats, slab_q ? w + o_slab : nullptr,
-                         nr_refine_zero(nq, k, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine), s, true);
+                         nr_refine_zero(nq, k, cut, w + o_refine), s, true);
   if (e == cudaSuccess)
     e = nr_launch_refine(ix, d_queries, nq, k, (int)Lmax, (nr_seg *)(w + o_seg),
                          (int32_t *)(w + o_nL), (uint32_t *)(w + o_slen), (uint32_t *)(w + o_codes), P,
-                         d_out_ids, d_out_dists,
-                         stats, w + o_refine, NR_STATIC_SCRATCH_BYTES - o_refine, s, true);
+                         d_out_ids, d_out_dists, stats, cut, room.blocks, w + o_refine, s, true);
   // statistics of this call are read from the array by nr_last_stats / nr_query_stats
   ix->d_stats = stats;
   ix->last_nq = nq;
