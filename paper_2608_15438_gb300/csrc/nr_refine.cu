@@ -486,13 +486,13 @@ __global__ void __launch_bounds__(TR, MINB) refine_spans_kernel(RefineArgs a) {
 }
 
 // Resident blocks of `kern` (blocks of TR threads with smem bytes), or 0 and
-// the error. The kernel may take all the shared memory there is from here on:
-// the same for every caller, so that no other thread's call lowers it before
-// this one's launch.
+// the error. (The attribute is what the launch takes and no more: with all there
+// is, less is left for L1, and 1,300 fp32 queries, D = 272, took 3,294 us for
+// 3,135.)
 template <class K>
 int64_t resident(const nr_index *ix, K kern, int TR, size_t smem, cudaError_t *e) {
   int per_sm = 0;
-  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ix->smem_optin);
+  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (*e == cudaSuccess) *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TR, smem);
   if (*e == cudaSuccess && per_sm < 1) *e = cudaErrorInvalidConfiguration;
   return *e == cudaSuccess ? (int64_t)per_sm * ix->num_sms : 0;
@@ -564,8 +564,10 @@ bool bound_by_stream(const RefineArgs &a, int C) {
 template <int DT, int TR, int CPR, int KCC, int ST, int MINB>
 cudaError_t launch_spans(nr_index *ix, RefineArgs a, PlanArgs pa, int64_t grid, cudaStream_t s, bool early) {
   const size_t smem = nrq::refine_smem_bytes<DT, TR, CPR, KCC, ST, true>(a.row_bytes, a.rf.k);
-  auto kern = refine_spans_kernel<DT, TR, CPR, KCC, ST, MINB>;  // (resident has set its attribute)
-  cudaError_t e;
+  auto kern = refine_spans_kernel<DT, TR, CPR, KCC, ST, MINB>;
+  // (another thread's call may have set another size since `resident`)
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   pa.rule.align = a.rf.R < TR ? TR / a.rf.R : 1;
   // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
   // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
