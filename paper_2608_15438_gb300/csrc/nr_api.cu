@@ -880,7 +880,7 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
     const int64_t n = (nq - q0) < qc ? (nq - q0) : qc;
     const int slot = (int)(i % slots);
     char *cw = w + chunk_off + slot_bytes * (size_t)slot;
-    const bool cut = cut_bytes > 0 && nr_refine_cuts(ix, n, room);
+    const bool cut = cut_bytes > 0 && nr_refine_cuts(ix, n, k, C, room);
     // buffer `slot` is free again once the refinement that last read it ended
     if (pipe && i >= slots && (e = cudaStreamWaitEvent(sa, ps.ref[slot], 0)) != cudaSuccess) break;
     const void *qp = (const char *)d_q + q0 * RB;

@@ -203,7 +203,7 @@ struct nr_refine_room {
   int64_t most;    // no larger batch is cut, whatever the parameters
 };
 cudaError_t nr_refine_room_of(const nr_index *ix, int k, nr_refine_room *room);
-bool nr_refine_cuts(const nr_index *ix, int64_t nq, const nr_refine_room &room);
+bool nr_refine_cuts(const nr_index *ix, int64_t nq, int k, int C, const nr_refine_room &room);
 // scratch of a refine launch over nq queries
 size_t nr_refine_scratch_bytes(int64_t nq, int k, bool cut);
 // the flags in it that have to be zero (none of whole streams): the select launch

@@ -509,22 +509,28 @@ cudaError_t launch_plan(nr_index *ix, const PlanArgs &pa, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Whether a batch keeps its streams whole (a block a query) when grid blocks
+// Whether a batch keeps its streams whole (a block a query) when `blocks` blocks
 // are resident. Few queries leave most blocks idle; many keep them busy, and
-// cutting their streams only adds work per span (about 7 us each: the item,
-// the segment search, the first tile's latency, the commit) and rows read
-// beyond an early stop. Measured (search us, cut / whole): u8-10m P 256, no
-// early stop, 608 blocks: 100 queries 240 / 343, 400 368 / 381, 600 485 / 432;
-// u8-30m P 1024 t_low 80: 300 546 / 593, 400 651 / 639; f32-10m, 1,368 blocks,
-// no early stop: 400 462 / 1,016, t_low 16: 400 462 / 569, 700 710 / 645;
-// u8-10m k 100 t_low 16: 100 471 / 507, 300 584 / 524; P 64 t_low 4: 1 query
-// 81 / 103, 100 167 / 163; 1536-value fp32 rows, 456 blocks: 30 1,075 / 7,909,
-// 440 13,058 / 16,062. An early stop after few rounds makes the later spans of
-// a stream likely waste.
-bool whole_streams(int64_t nq, int64_t grid, int t_low, bool long_rows) {
-  if (long_rows) return nq >= grid;
-  const int64_t sixteenths = t_low == 0 || t_low >= 64 ? 10 : t_low >= 8 ? 5 : 2;
-  return nq * 16 >= grid * sixteenths;
+// cutting their streams only adds work per span (about 7 us each: the item, the
+// segment search, the first tile's latency, the commit) and, with an early stop,
+// rows read beyond it: the more, the smaller the part of a stream that t_low
+// rounds are. The line, in sixteenths of the blocks, lies where both sides
+// measured the same (k = 10, `blocks` as the kernel has them for each row size):
+// no early stop 18 to 30 (uint8 x 128 18-21, fp32 x 96 21, other rows 20-30; k =
+// 100 12); t_low rounds as long as the stream 14 to 24, a quarter of it uint8 5 to
+// 11 and fp32 6 to 15, a sixteenth 2 to 8 and 4 to 8. us, cut and whole: u8-10m P
+// = C = 256, no early stop: 400 queries 342 / 433, 600 461 / 499, 1,000 721 / 628;
+// t_low 16: 200 236 / 259, 300 297 / 269; f32-10m P 512, no early stop: 600 592 /
+// 688, 1,000 924 / 870; t_low 4: 150 204 / 220, 200 263 / 246; u8-30m P = C =
+// 1024, t_low 80: 150 435 / 492, 300 781 / 585; 768-value fp32 rows, no early
+// stop: 600 3,318 / 3,565, t_low 4: 100 597 / 638, 200 1,148 / 721.
+constexpr int kCutMost = 18;  // sixteenths, at most
+bool whole_streams(const nr_index *ix, int64_t nq, int k, int C, int64_t blocks) {
+  const int64_t stop = (int64_t)ix->params.t_low * ix->params.round_size;  // rows
+  const int64_t rows = (int64_t)C * (ix->t > 0 ? ix->t : 64);              // of a stream, some
+  const int64_t least = ix->dtype == 0 ? rows + 16 * stop : 2 * rows + 24 * stop;  // the line x rows
+  const int64_t most = k > 32 ? 12 : kCutMost;
+  return nq * 16 >= blocks * most || (stop > 0 && (double)nq * 16 * rows >= (double)blocks * least);
 }
 
 // Of whole streams: whether nearby queries go side by side (see plan_kernel).
@@ -674,13 +680,13 @@ cudaError_t nr_refine_room_of(const nr_index *ix, int k, nr_refine_room *room) {
     cudaError_t e;
     const int64_t blocks = resident(ix, refine_spans_kernel<S::DT, S::TR, S::CPR, S::KCC, S::ST, S::MINB>, S::TR,
                        nrq::refine_smem_bytes<S::DT, S::TR, S::CPR, S::KCC, S::ST, true>(ix->row_bytes, k), &e);
-    *room = {allowed(ix, blocks), blocks};  // whole_streams: less than a query a block
+    *room = {allowed(ix, blocks), blocks * kCutMost / 16};
     return e;
   });
 }
 
-bool nr_refine_cuts(const nr_index *ix, int64_t nq, const nr_refine_room &room) {
-  return !whole_streams(nq, room.blocks, ix->params.t_low, ix->dtype == 1 && ix->row_bytes > 1024);
+bool nr_refine_cuts(const nr_index *ix, int64_t nq, int k, int C, const nr_refine_room &room) {
+  return !whole_streams(ix, nq, k, C, room.blocks);
 }
 
 size_t nr_refine_scratch_bytes(int64_t nq, int k, bool cut) { return refine_scratch(nq, k, cut).total; }

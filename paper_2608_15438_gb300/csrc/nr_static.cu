@@ -100,7 +100,7 @@ extern "C" nr_status nr_search_static(nr_index *ix, const void *d_queries, int64
   nr_refine_room room;
   cudaError_t e = nr_refine_room_of(ix, k, &room);
   if (e != cudaSuccess) return cuda_status(e);
-  const bool cut = nr_refine_cuts(ix, nq, room) &&
+  const bool cut = nr_refine_cuts(ix, nq, k, C, room) &&
                    nr_refine_scratch_bytes(nq, k, true) <= NR_STATIC_SCRATCH_BYTES - o_refine;
   // every buffer below is fully written before it is read, except the
   // refinement's flags, which the selection clears
