@@ -608,17 +608,14 @@ __device__ __forceinline__ bool commit_block(const RefineParams &a, const Refine
   c.slot = c.off + TR;
   c.want = c.slot + TR;
   c.entry = reinterpret_cast<uint4 *>(c.want + 64);
-  int *ctl = m.sctl + 1;  // [0] the first span not to commit, [1] wanted spans; then counters
+  int *ctl = m.sctl + 1;  // [0] the first span not to commit; then counters
   const int rounds_span = (int)((span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
   const int rounds_last = (int)((n - (spans - 1u) * span_rows + (uint32_t)a.R - 1u) / (uint32_t)a.R);
   auto kth = [&]() { return r.hn == k ? m.hkey[r.cur * k + k - 1] : kEmpty; };
   while (next < spans) {
     const uint32_t x = next + tid;
     const uint32_t rdy = x < spans ? ld_acquire(&ready[x]) : 0u;
-    if (tid == 0) {
-      ctl[0] = TR;
-      ctl[1] = 0;
-    }
+    if (tid == 0) ctl[0] = TR;
     const bool logged = rdy > 1u && rdy != kSpanRedo;
     uint4 h = make_uint4(0xffffffffu, 0xffffffffu, 0u, 0u);
     if (logged) h = __ldcg(reinterpret_cast<const uint4 *>(hdr + x));
@@ -636,6 +633,9 @@ __device__ __forceinline__ bool commit_block(const RefineParams &a, const Refine
     }
     {  // stage, the earliest first
       const uint64_t top = kth();
+      // wanted spans, counted by every thread: a word of ctl would be cleared
+      // below while other warps may not have read it yet
+      int nw = 0;
       for (int i0 = 0, at = 0; i0 < nb && at < SLOTS; i0 += 32) {
         const unsigned b = __ballot_sync(kFull, i0 + lane < nb && c.min[min(i0 + lane, TR - 1)] < top);
         if (warp == 0 && ((b >> lane) & 1u)) {
@@ -646,10 +646,9 @@ __device__ __forceinline__ bool commit_block(const RefineParams &a, const Refine
           }
         }
         at += __popc(b);
-        if (tid == 0) ctl[1] = min(at, SLOTS);
+        nw = min(at, SLOTS);
       }
       __syncthreads();
-      const int nw = ctl[1];
       for (int e = tid; e < nw * kStagedEntries; e += TR) {
         const uint32_t at = c.off[c.want[e / kStagedEntries]] + (uint32_t)(e % kStagedEntries);
         if (at < cap) cp_async16((uint32_t)__cvta_generic_to_shared(c.entry + e), pool + at);
