@@ -400,8 +400,14 @@ __global__ void __launch_bounds__(TR, MINB) refine_spans_kernel(RefineArgs a) {
       }
       for (;;) {
         if (!held) {
-          if (!__syncthreads_or(tid == 0 && atomicCAS(&st->lock, 1, 2) == 1)) break;
-          __threadfence();
+          // the thread that takes the lock orders what its last holder wrote
+          // before the barrier, which hands that on to the block
+          bool took = false;
+          if (tid == 0 && atomicCAS(&st->lock, 1, 2) == 1) {
+            __threadfence();
+            took = true;
+          }
+          if (!__syncthreads_or(took)) break;
           held = true;
           r.cur = 0;
           r.hn = __ldcg(&st->hn);

@@ -54,7 +54,9 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
 // rounds and the stop of one block refining the whole stream. Whichever block
 // finishes the next span to commit takes the query's lock and commits every
 // consecutive finished span; a block that does not get the lock moves on (the
-// holder looks again after it unlocks), so no block ever waits for another.
+// holder looks again after it unlocks), so none depends on another's progress: a
+// holder with nothing else to do looks at most a fixed number of times for a
+// span in flight (polls) and then hands the top-k over.
 struct RefineParams {
   const uint8_t *vec;
   const uint32_t *ids;
