@@ -1,7 +1,7 @@
 // Index construction on the GPU (neuroute_build.h; paper Sec. 3.3, thresholds
 // Sec. 3.2.3): per-bit lower medians by a radix select over order-preserving
-// keys, codes, a stable sort of ids by code, bucket-local k-means with one
-// warp per bucket (one CTA for large buckets), the two CSR levels, and the
+// keys, codes, a stable sort of ids by code, bucket-local k-means (a warp, a CTA
+// or a CTA of more threads per bucket, by its size), the two CSR levels, and the
 // placement of the rows in stored order.
 //
 // The k-means arithmetic follows a fixed definition that does not depend on
