@@ -832,17 +832,23 @@ static nr_status search_impl(nr_index *ix, const void *d_q, const float *d_logit
   // workspace: [per-query stats][chunk buffers]
   const size_t stats_off = 0;
   const size_t chunk_off = align256(stats_off + (size_t)nq * NR_QSTATS * 8);
+  auto keep_whole = [&] {
+    cut_bytes = 0;
+    l = chunk_layout(ix, qc, P, C, whole_bytes);
+    slot_bytes = align256(l.total);
+  };
   if (chunk_off + slot_bytes * (size_t)slots > ix->ws_cap) {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
-    if (capture != cudaStreamCaptureStatusNone) {
-      // it cannot grow now: streams stay whole (captured after calls of a smaller k)
-      cut_bytes = 0;
-      l = chunk_layout(ix, qc, P, C, whole_bytes);
-      slot_bytes = align256(l.total);
-    }
+    // it cannot grow now: streams stay whole (captured after calls of a smaller k)
+    if (capture != cudaStreamCaptureStatusNone) keep_whole();
   }
-  if ((st = ensure_ws(ix, chunk_off + slot_bytes * (size_t)slots)) != NR_OK) return st;
+  st = ensure_ws(ix, chunk_off + slot_bytes * (size_t)slots);
+  if (st == NR_ERR_OOM && cut_bytes > 0) {  // no memory for spans: streams stay whole
+    keep_whole();
+    st = ensure_ws(ix, chunk_off + slot_bytes * (size_t)slots);
+  }
+  if (st != NR_OK) return st;
   if (pipe && (st = ensure_pipe(ix)) != NR_OK) return st;
   char *w = (char *)ix->ws;
   int64_t *stats = (int64_t *)(w + stats_off);

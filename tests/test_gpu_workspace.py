@@ -1,6 +1,7 @@
 """The search workspace: a batch whose streams stay whole takes no room for spans
 beyond what the largest cut batch needs, a smaller batch after a larger one needs
-no more, and a capture that would need more keeps its streams whole."""
+no more, and a capture that would need more keeps its streams whole, as does a
+call for whose spans there is no device memory."""
 import numpy as np
 import pytest
 
@@ -65,4 +66,34 @@ def test_captured_after_calls_of_a_smaller_k(index, tmp_path):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(out[0], ids[a:a + 40]) and torch.equal(out[1], dist[a:a + 40])
+    fresh.close()
+
+
+def test_without_memory_for_spans(index, tmp_path):
+    torch, ix, q = index
+    from paper_2608_15438_gb300 import neuroute as nr
+
+    k, P, C = 100, 8, 16
+    ix.set_params(t_low=0)
+    # both kinds of kernels are loaded: 2,000 queries stay whole, 400 are cut
+    ids, dist = (v[:400].clone() for v in ix.search(q[:2_000], k, P, C))
+    ix.search(q[:400], k, P, C)
+    fresh = nr.Index(str(tmp_path / "ws.nrix"), 0)
+    fresh.set_params(t_low=0)
+    fresh.search(q[:1], 1, P, C)
+    out = buffers(torch, 400, k)
+    torch.cuda.synchronize()
+    # the logs of 400 queries take 20 MB, the batch without them 1 MB or so
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (12 << 20), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        for o in out:
+            o.zero_()
+        fresh.search(q[:400], k, P, C, out=out)
+        torch.cuda.synchronize()
+        assert torch.equal(out[0], ids) and torch.equal(out[1], dist)
+    del fill
+    torch.cuda.empty_cache()
+    fresh.search(q[:400], k, P, C, out=out)
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], ids) and torch.equal(out[1], dist)
     fresh.close()
