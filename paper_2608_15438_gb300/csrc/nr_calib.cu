@@ -293,15 +293,23 @@ nr_status nr_index_locate(nr_index *ix, const int64_t *d_ids, int64_t n, int32_t
   // is none when every fourth row or more is asked for.
   uint32_t fbits = kSmallBits;
   while ((int64_t)fbits < 4096 * n && fbits < (1u << 27)) fbits <<= 1;
-  const bool filter = n < ix->N / 4;
+  bool filter = n < ix->N / 4;
   const uint32_t *cnull = nullptr;
   uint32_t *wnull = nullptr;
   size_t tb = 0;
   cudaError_t e = cub::DeviceRadixSort::SortPairs(nullptr, tb, cnull, wnull, cnull, wnull, n, 0, 32, s);
   if (e != cudaSuccess) return cuda_status(e);
-  const size_t vb = ((size_t)n * 4 + 255) & ~(size_t)255, fb = filter ? kSmallBits / 8 + fbits / 8 : 0;
+  const size_t vb = ((size_t)n * 4 + 255) & ~(size_t)255;
+  size_t fb = filter ? kSmallBits / 8 + fbits / 8 : 0;
   char *mem = nullptr;
-  if ((e = cudaMalloc((void **)&mem, 4 * vb + fb + (tb > 0 ? tb : 16))) != cudaSuccess) return cuda_status(e);
+  e = cudaMalloc((void **)&mem, 4 * vb + fb + (tb > 0 ? tb : 16));
+  if (e == cudaErrorMemoryAllocation && filter) {  // no memory for the filters: searches alone
+    cudaGetLastError();
+    filter = false;
+    fb = 0;
+    e = cudaMalloc((void **)&mem, 4 * vb + (tb > 0 ? tb : 16));
+  }
+  if (e != cudaSuccess) return cuda_status(e);
   uint32_t *keys = (uint32_t *)mem, *idx = (uint32_t *)(mem + vb), *skeys = (uint32_t *)(mem + 2 * vb),
            *sidx = (uint32_t *)(mem + 3 * vb), *small = filter ? (uint32_t *)(mem + 4 * vb) : nullptr,
            *large = filter ? small + kSmallBits / 32 : nullptr;

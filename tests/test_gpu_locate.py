@@ -1,5 +1,6 @@
 """nr_index_locate with few ids (found through the filters) and many (searched
-directly): repeats, ids that are not stored, negative and 2^32-range ids."""
+directly, or where the device has no memory for the filters): repeats, ids that
+are not stored, negative and 2^32-range ids."""
 import numpy as np
 import pytest
 
@@ -52,3 +53,23 @@ def test_locate_into_a_buffer_at_any_int32(tmp_path, offset):
     ix.close()
     assert torch.equal(out.view(-1, 4), exp)
     assert buf[:offset].eq(7).all() and buf[offset + 5_000 * 4:].eq(7).all()
+
+
+def test_locate_without_memory_for_the_filters(tmp_path):
+    torch = need_cuda()
+    from paper_2608_15438_gb300 import neuroute as nr
+
+    path, _, _ = build_small(tmp_path, "tiny", n=30_000, bits=10, name="loc")
+    ix = nr.Index(path, 0)
+    ids = torch.randint(-10, 30_010, (7_499,), device="cuda")
+    exp = ix.locate(ids)
+    out = torch.zeros_like(exp)
+    torch.cuda.synchronize()
+    # the filters of 7,499 ids take 4.1 MB, the rest 0.2
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (4 << 20), dtype=torch.uint8, device="cuda")
+    assert nr.lib().nr_index_locate(ix.h, ids.data_ptr(), 7_499, out.data_ptr(), None) == 0
+    assert torch.cuda.mem_get_info()[0] < 4_100_000
+    del fill
+    torch.cuda.empty_cache()
+    ix.close()
+    assert torch.equal(out, exp)
