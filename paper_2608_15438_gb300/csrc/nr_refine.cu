@@ -581,10 +581,16 @@ cudaError_t launch_spans(nr_index *ix, RefineArgs a, PlanArgs pa, int64_t grid, 
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   pa.rule.align = a.rf.R < TR ? TR / a.rf.R : 1;
-  // two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
+  // Two uint8 items a block, four of the slower fp32 ones (u8-10m k 100, 100
   // queries: 471 us at two, 506 at four; long fp32 rows, 30 queries: 1,144 and
-  // 1,075)
-  pa.rule.items_want = (unsigned int)((DT == 0 ? 2 : 4) * grid);
+  // 1,075). Three for two blocks where a large top-k makes the commits the longer
+  // part, which follow one another in a query: us a search at two items and at one
+  // and a half, u8-30m k 100, P 92, C 64, t_low 16: 70 queries 285 / 272; P = C =
+  // 256, no early stop: 16 351 / 359, 30 381 / 364, 250 587 / 575; P = C = 1024,
+  // t_low 80: 16 408 / 389, 150 568 / 540; u8-10m P = C = 256: 20 307 / 320, 200 446
+  // / 436; k 256, P 64, C 512: 20 481 / 444, 80 436 / 411. (k 50: 46 queries of P 92
+  // 206 / 195 at four for three, of P = C = 256 281 / 289, of 1024 329 / 336.)
+  pa.rule.items_want = (unsigned int)((DT == 0 ? (a.rf.k > 64 ? 3 : 4) : 8) * grid / 2);
   a.group = (int)grid;
   a.rule = pa.rule;
   a.own_plan = a.nq <= kOwnPlan;
